@@ -13,7 +13,8 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libep.so")
 SOURCES = [os.path.join(CSRC, "ep_api.cu"), os.path.join(CSRC, "ep_sdf.cu")]
-HEADERS = [os.path.join(CSRC, h) for h in ("ep_kernels.cuh", "ep_common.cuh", "ep_stencil.cuh", "ep_aux.cuh")]
+HEADERS = [os.path.join(CSRC, h) for h in ("ep_kernels.cuh", "ep_common.cuh", "ep_stencil.cuh", "ep_aux.cuh", "ep_tables.cuh",
+                                             "ep_sweep.cuh")]
 DEPS = SOURCES + HEADERS + [os.path.join(ROOT, "include", h) for h in ("ep.h", "ep_sdf.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

@@ -39,9 +39,10 @@ namespace {
 #endif
 constexpr int kZSeg = EP_ZSEG;     // default output planes per z-march segment
 constexpr int kZSegMin = 8;        // smallest segment length the batch autotuner tries
-constexpr int kSweepChunk = 64;    // sweeps per queued graph chunk
+constexpr int kSweepChunk = 64;    // sweeps per queued graph chunk (even: launches alternate in parity)
 constexpr int kSoloAllMembers = 8; // batch groups this small sweep every member in its own launches
 constexpr double kDivFactor = 1e16;
+constexpr int kNoAllocMaxPartials = 32768;   // ep_step_noalloc: stencil work items and reduction chunks
 
 struct StimDef {
     int lo[3], hi[3];
@@ -63,6 +64,8 @@ struct HostPlan {
     std::vector<Seg> segs;              // work items at the handle's z-planes per item
     std::vector<Seg> segs_z[4];         // work items at kZLens[i] planes per item (set-up picks one)
     std::vector<Seg> segs_e, segs_e_z[4];   // the same over the domain (torso handles only)
+    std::vector<Brick> bricks;          // tabulated operator: bricks over the tissue, and their lists' totals
+    long long n_vert = 0, n_part = 0, n_bound = 0;
 };
 
 constexpr int kZLens[4] = {8, 16, 24, 32};
@@ -122,6 +125,15 @@ struct ep_sim {
     void *x2 = nullptr;          // second correction buffer of the FP32 elliptic solve (correction form)
     long long ie_seen = 0;                // implicit sweeps counted by earlier calls
     long long step = 0;
+    // tabulated elliptic operator (ep_tables.cuh); lean: left out, where its memory is not to be had
+    bool lean = false;
+    size_t tab_total = 0;   // its device bytes
+    int tab = 0, nrows = 0, nbricks = 0, nsweep = 0;
+    int row_colour[9] = {};
+    void *rows = nullptr, *cheb_table = nullptr;
+    Brick *bricks = nullptr;
+    BrickLists lists{};
+    unsigned *sweep_arrive = nullptr;
     bool noalloc_call = false;   // inside ep_step_noalloc: scratch is the static array, no graph
     // device-time accounting (ep_profile_enable)
     bool prof_on = false;
@@ -233,14 +245,14 @@ int partition_far(std::vector<Seg> &segs, const uint8_t *heart, int nx, int ny, 
     return (int)(mid - segs.begin());
 }
 
-std::vector<Seg> build_segments(const uint8_t *m, int nx, int ny, int nz, int zseg)
+std::vector<Seg> build_segments(const uint8_t *m, int nx, int ny, int nz, int zseg, int tile = kTileY)
 {
     std::vector<Seg> segs;
-    const int nby = (ny + kTileY - 1) / kTileY;
+    const int nby = (ny + tile - 1) / tile;
     std::vector<char> has((size_t)nz * nx);   // (plane, column) holds tissue in some row of the band
     std::vector<char> col(nx);
     for (int by = 0; by < nby; ++by) {
-        const int ya = by * kTileY, yb = std::min(ya + kTileY, ny);
+        const int ya = by * tile, yb = std::min(ya + tile, ny);
         for (int k = 0; k < nz; ++k) {
             char *h = &has[(size_t)k * nx];
             std::fill(h, h + nx, 0);
@@ -279,6 +291,74 @@ std::vector<Seg> build_segments(const uint8_t *m, int nx, int ny, int nz, int zs
     return segs;
 }
 
+// Bricks over the tissue of a mask of 0 / 1 bytes, windows placed as the work items' are, and the lengths of their
+// lists: vertices with eight tissue voxels (full), with one to seven, and voxels whose eight vertices are full (inner).
+void build_bricks(const uint8_t *m, int nx, int ny, int nz, HostPlan &P)
+{
+    const size_t row = (size_t)nx + 1, vplane = row * ((size_t)ny + 1), prow = (size_t)nx + 2;
+    // tissue voxels of every vertex: 0 none, 1 some, 2 all
+    std::vector<uint8_t> cls(vplane * ((size_t)nz + 1)), zero(nx, 0), all(prow), any(prow);
+    for (int K = 0; K <= nz; ++K)
+        for (int J = 0; J <= ny; ++J) {
+            const uint8_t *r[4];
+            for (int c = 0; c < 4; ++c) {
+                const int j = J - 1 + (c & 1), k = K - 1 + (c >> 1);
+                r[c] = j < 0 || k < 0 || j >= ny || k >= nz ? zero.data() : m + (size_t)nx * (j + (size_t)ny * k);
+            }
+            all[0] = any[0] = all[nx + 1] = any[nx + 1] = 0;
+            for (int i = 0; i < nx; ++i) {
+                all[i + 1] = r[0][i] & r[1][i] & r[2][i] & r[3][i];
+                any[i + 1] = r[0][i] | r[1][i] | r[2][i] | r[3][i];
+            }
+            uint8_t *o = cls.data() + row * (J + ((size_t)ny + 1) * K);
+            for (int X = 0; X <= nx; ++X) o[X] = (uint8_t)((any[X] | any[X + 1]) + (all[X] & all[X + 1]));
+        }
+    P.bricks.clear();
+    P.n_vert = P.n_part = P.n_bound = 0;
+    long long nout = 0;
+    for (const Seg &g : build_segments(m, nx, ny, nz, kBrickZ, kBrickY)) {
+        Brick B{};
+        B.x0 = g.x0;
+        B.y0 = g.by * kBrickY;
+        B.z0 = g.k0;
+        B.planes = g.k1 - g.k0;
+        B.vbase = (int)P.n_vert;
+        B.pbase = (int)P.n_part;
+        B.obase = (int)nout;
+        B.fbase = (int)P.n_bound;
+        const int xe = std::min(kBrickX, nx - B.x0), ye = std::min(kBrickY, ny - B.y0);
+        for (int lz = 0; lz <= B.planes; ++lz)
+            for (int ly = 0; ly <= ye; ++ly) {
+                const uint8_t *c = cls.data() + row * (B.y0 + ly + ((size_t)ny + 1) * (B.z0 + lz)) + B.x0;
+                int some = 0, full = 0;
+                for (int lx = 0; lx <= xe; ++lx) {
+                    some += c[lx] != 0;
+                    full += c[lx] >> 1;
+                }
+                B.nvert += some;
+                B.nfull += full;
+            }
+        for (int oz = 0; oz < B.planes; ++oz)
+            for (int oy = 0; oy < ye; ++oy) {
+                const uint8_t *c = cls.data() + row * (B.y0 + oy + ((size_t)ny + 1) * (B.z0 + oz)) + B.x0;
+                const uint8_t *d = c + row, *e = c + vplane, *f = d + vplane;
+                const uint8_t *t = m + (size_t)nx * (B.y0 + oy + (size_t)ny * (B.z0 + oz)) + B.x0;
+                int out = 0, inner = 0;
+                for (int ox = 0; ox < xe; ++ox) {
+                    out += t[ox];
+                    inner += (c[ox] & c[ox + 1] & d[ox] & d[ox + 1] & e[ox] & e[ox + 1] & f[ox] & f[ox + 1]) >> 1;
+                }
+                B.nout += out;
+                B.ninner += inner;
+            }
+        P.n_vert += B.nvert;
+        P.n_part += B.nvert - B.nfull;
+        nout += B.nout;
+        P.n_bound += B.nout - B.ninner;
+        P.bricks.push_back(B);
+    }
+}
+
 // ---------------------------------------------------------------------------
 // set-up: layout built on the host from the mask, records on the device
 // ---------------------------------------------------------------------------
@@ -300,12 +380,60 @@ bool needs_spectrum(const ep_sim *s)
     return s->p.solver == EP_SOLVER_CHEBYSHEV || (s->p.solver == EP_SOLVER_JACOBI && s->p.jacobi_omega < 0.0);
 }
 
+// The elliptic sweeps of a bidomain handle without a torso run over the tabulated operator.  Below kTabMin tissue
+// voxels a sweep is a launch's latency on either path, and the handle stays as small as its fields.
+constexpr long long kTabMin = 4096;
+// Assembled rows for every tissue voxel (112 bytes a row in FP32) up to this many: the rows then stay in the L2
+// cache.  Above it the bricks: 671 thousand voxels (192^3 shell) take 15.5 us a sweep in rows and 18.3 in bricks, 831
+// thousand (160^3 heart) 23.1 and 19.8, 3.41 million (256^3 heart) 91 and 55.6.
+constexpr long long kRowsOnly = EP_ROWS_ONLY;
+constexpr int kMaxRowCtas = 4096;
+constexpr size_t kArriveBytes = sizeof(unsigned) * kArriveStride * (kArriveGroups + 1);
+
+struct TabPlan {
+    int tab = 0, nbricks = 0, nsweep = 0, parts = 1;
+    long long nrows = 0;
+};
+
+TabPlan tab_plan(const ep_sim *s)
+{
+    TabPlan t;
+    if (s->lean || !s->have_params || s->d.model != EP_BI || !s->torso.empty() || s->n_tissue < kTabMin) return t;
+    const bool gs = s->p.solver == EP_SOLVER_GAUSS_SEIDEL;
+    t.tab = 1;
+    t.parts = gs ? 8 : 1;
+    if (!gs && s->d.precision == EP_FP32 && s->n_tissue > kRowsOnly) {
+        t.nbricks = (int)s->plan.bricks.size();
+        t.nsweep = t.nbricks;
+        return t;
+    }
+    t.nrows = s->n_tissue;
+    const long long per = gs ? (t.nrows + 7) / 8 + (t.nrows + 15) / 16 : t.nrows;   // a colour's rows, or thereabouts
+    t.nsweep = (int)std::min<long long>(kMaxRowCtas, (per + kSweepThreads - 1) / kSweepThreads);
+    return t;
+}
+
+size_t tab_bytes(const ep_sim *s, const TabPlan &t, size_t rb)
+{
+    if (!t.tab) return 0;
+    const HostPlan &P = s->plan;
+    size_t b = 0;
+    if (t.nbricks)
+        b = abytes(sizeof(Brick) * (size_t)t.nbricks) + abytes(sizeof(float4) * (size_t)P.n_vert) +
+            abytes(sizeof(float2) * (size_t)P.n_vert) + abytes(2 * (size_t)P.n_vert) + abytes(2 * (size_t)P.n_part) +
+            abytes(sizeof(float2) * (size_t)s->n_tissue) + abytes((size_t)P.n_bound);
+    else
+        b = abytes(rb * kRowLen * (size_t)t.nrows);
+    return b + abytes(rb * kChebTable) + abytes(kArriveBytes);
+}
+
 // Residual partial sums per stencil work item: one, or one per colour pass of the
 // eight-colour sweep.
 long long partial_slots(const ep_sim *s)
 {
     const long long per = s->have_params && s->p.solver == EP_SOLVER_GAUSS_SEIDEL ? 8 : 1;
-    return std::max<long long>(per * s->max_items, s->nchunk);
+    const TabPlan t = tab_plan(s);
+    return std::max<long long>(std::max<long long>(per * s->max_items, s->nchunk), (long long)t.parts * t.nsweep);
 }
 
 // Set-up scratch of the Chebyshev interval estimate (0 when the interval is
@@ -337,6 +465,7 @@ void footprint(const ep_sim *s, size_t rb, size_t *resident, size_t *peak)
     r += abytes(sizeof(double) * (size_t)partial_slots(s)) + abytes(sizeof(Ctl));
     if (s->have_params && s->p.diffusion == EP_IMPLICIT) r += 2 * abytes(rb * n);   // second iterate, 1/(1 + a D)
     if (solve_eform(s, rb)) r += abytes(rb * n);
+    r += tab_bytes(s, tab_plan(s), rb);
     const bool torso = !s->torso.empty();
     if (torso) r += abytes(sizeof(float4) * n) + abytes(sizeof(Seg) * (size_t)s->max_items);   // domain records, items
     if (s->ecg_q[0] >= 0) r += abytes(sizeof(double) * 3 * (size_t)s->ecg_cap);
@@ -426,6 +555,8 @@ ep_status plan_layout(ep_sim *s)
     s->nchunk = (int)P.chunks.size();
     s->nseg = (int)P.segs.size();
     s->nseg_e = torso ? (int)P.segs_e.size() : s->nseg;
+    if (s->d.model == EP_BI && !torso && s->d.precision == EP_FP32 && s->n_tissue > kRowsOnly)
+        build_bricks(mh, nx, ny, nz, P);
     // capacity of the item buffers: the largest item count of the z-lengths set-up and the batch use
     s->max_items = std::max<long long>(most, std::max(s->nseg, s->nseg_e));
     footprint(s, s->d.precision == EP_FP64 ? sizeof(double) : sizeof(float), &s->fp_resident, &s->fp_peak);
@@ -578,6 +709,8 @@ ep_status setup_typed(ep_sim *s)
     const size_t rb = sizeof(real);
     s->rsz = rb;
     s->rec = (float4 *)dalloc(s, sizeof(float4) * n);
+    const TabPlan tp = tab_plan(s);
+    cudaStream_t st = s->stream;
     for (int i = 0; i < 2; ++i) {
         s->v[i] = dalloc(s, rb * n);
         s->w[i] = dalloc(s, rb * n);
@@ -603,6 +736,37 @@ ep_status setup_typed(ep_sim *s)
         s->x2 = dalloc(s, rb * n);
         if (!s->x2) return fail(s, EP_ENOMEM, "device allocation failed");
     }
+    s->tab = tp.tab;
+    s->nrows = (int)tp.nrows;
+    s->nbricks = tp.nbricks;
+    s->nsweep = tp.nsweep;
+    s->tab_total = tab_bytes(s, tp, rb);
+    s->rows = nullptr;
+    s->bricks = nullptr;
+    if (tp.tab) {
+        bool got = true;
+        auto take = [&](auto *&p, size_t count) {
+            using T = std::remove_reference_t<decltype(*p)>;
+            p = (T *)dalloc(s, sizeof(T) * count);
+            got = got && p;
+        };
+        if (tp.nbricks) {
+            const size_t nv = (size_t)P.n_vert, nt = (size_t)s->n_tissue;
+            take(s->bricks, (size_t)tp.nbricks);
+            take(s->lists.k4, nv);
+            take(s->lists.k2, nv);
+            take(s->lists.vloc, nv);
+            take(s->lists.vpair, (size_t)P.n_part);
+            take(s->lists.out, nt);
+            take(s->lists.oflag, (size_t)P.n_bound);
+        } else {
+            s->rows = dalloc(s, rb * kRowLen * (size_t)tp.nrows);
+            got = got && s->rows;
+        }
+        s->cheb_table = dalloc(s, rb * kChebTable);
+        s->sweep_arrive = (unsigned *)dalloc(s, kArriveBytes);
+        if (!got || !s->cheb_table || !s->sweep_arrive) return fail(s, EP_ENOMEM, "device allocation failed");
+    }
     s->rec_e = s->rec;
     s->segs_e = s->segs;
     if (torso) {
@@ -627,7 +791,6 @@ ep_status setup_typed(ep_sim *s)
     for (const void *p : all)
         if (!p) return fail(s, EP_ENOMEM, "device allocation failed");
     if (s->dev_bytes != want_peak) return fail(s, EP_ECUDA, "internal: set-up allocations differ from the footprint");
-    cudaStream_t st = s->stream;
     CK(cudaMemcpyAsync(s->segs, segs.data(), sizeof(Seg) * segs.size(), cudaMemcpyHostToDevice, st));
     CK(cudaMemcpyAsync(s->idx, order.data(), sizeof(int) * order.size(), cudaMemcpyHostToDevice, st));
     CK(cudaMemcpyAsync(s->chunks, chunks.data(), sizeof(Chunk) * chunks.size(), cudaMemcpyHostToDevice, st));
@@ -660,6 +823,40 @@ ep_status setup_typed(ep_sim *s)
         k_fill<real><<<grid_for(n, 256), 256, 0, st>>>((real *)s->ie_x, n, real(0));
         CK(cudaGetLastError());
     }
+    std::vector<int> rowq;   // outlives the copy below (the stream is synchronised at the end of set-up)
+    int *d_bad = nullptr;    // a list that differs from the host's count
+    if (tp.tab) {   // the tabulated elliptic operator; the staged fibres' space serves once the records are built
+        const double C = 1.0 / (8.0 * s->d.dx_mm * s->d.dx_mm);
+        CK(cudaMemsetAsync(s->sweep_arrive, 0, kArriveBytes, st));
+        if (tp.nbricks) {
+            d_bad = (int *)tmp_fib;
+            CK(cudaMemsetAsync(d_bad, 0, sizeof(int), st));
+            CK(cudaMemcpyAsync(s->bricks, P.bricks.data(), sizeof(Brick) * P.bricks.size(), cudaMemcpyHostToDevice, st));
+            k_build_bricks<<<tp.nbricks, 256, 0, st>>>(nx, ny, nz, sT, sL - sT, C, s->rec, s->bricks, s->lists, d_bad);
+        } else {
+            rowq.reserve((size_t)tp.nrows);
+            if (tp.parts == 8) {   // sorted by colour
+                for (int c = 0; c < 8; ++c) {
+                    s->row_colour[c] = (int)rowq.size();
+                    for (int k = c >> 2; k < nz; k += 2)
+                        for (int j = (c >> 1) & 1; j < ny; j += 2) {
+                            const int q0 = nx * (j + ny * k);
+                            for (int i = c & 1; i < nx; i += 2)
+                                if (m[q0 + i]) rowq.push_back(q0 + i);
+                        }
+                }
+                s->row_colour[8] = (int)rowq.size();
+            } else {
+                for (int q = 0; q < (int)n; ++q)
+                    if (m[q]) rowq.push_back(q);
+            }
+            int *d_rowq = (int *)tmp_fib;
+            CK(cudaMemcpyAsync(d_rowq, rowq.data(), sizeof(int) * rowq.size(), cudaMemcpyHostToDevice, st));
+            k_build_rows<real><<<grid_for(tp.nrows, 128), 128, 0, st>>>(nx, ny, nz, sT, sL - sT, 0.0, C, s->rec, d_rowq,
+                                                                        tp.nrows, (real *)s->rows);
+        }
+        CK(cudaGetLastError());
+    }
     // the spectrum of D^-1 A: for the Chebyshev solver, and for damped Jacobi with estimated damping
     if (needs_spectrum(s) && s->d.model == EP_BI) {
         if (s->p.cheb_lmin > 0.0) {
@@ -675,6 +872,10 @@ ep_status setup_typed(ep_sim *s)
         // for the estimate's error), the fastest contraction of the slow modes that stays stable
         if (s->p.jacobi_omega < 0.0) s->omega = std::min(1.0, 1.9 / s->cheb_lmax);
     }
+    if (tp.tab && s->p.solver == EP_SOLVER_CHEBYSHEV) {
+        const double rho = (s->cheb_lmax - s->cheb_lmin) / (s->cheb_lmax + s->cheb_lmin);
+        k_cheb_table<real><<<1, 1024, 0, st>>>(rho, std::acosh(1.0 / rho), (real *)s->cheb_table);
+    }
     // rest state
     for (int i = 0; i < 2; ++i) {
         k_fill<real><<<grid_for(n, 256), 256, 0, st>>>((real *)s->v[i], n, real(0));
@@ -686,7 +887,10 @@ ep_status setup_typed(ep_sim *s)
     k_fill<real><<<grid_for(n, 256), 256, 0, st>>>((real *)s->tact, n, real(-1));
     CK(cudaGetLastError());
     CK(cudaMemsetAsync(s->ctl, 0, sizeof(Ctl), st));
+    int bad = 0;
+    if (d_bad) CK(cudaMemcpyAsync(&bad, d_bad, sizeof(int), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
+    if (bad) return fail(s, EP_ECUDA, "internal: a brick's lists differ from the plan");
     // free the set-up temporaries
     for (void *t : {tmp_fib, tmp_mask, tmp_rec, tmp_lz, tmp_torso}) {
         if (!t) continue;
@@ -705,6 +909,7 @@ ep_status setup_typed(ep_sim *s)
     s->plan.comp_chunk0 = std::vector<int>();
     s->plan.segs = std::vector<Seg>();
     s->plan.segs_e = std::vector<Seg>();
+    s->plan.bricks = std::vector<Brick>();
     for (auto &v : s->plan.segs_z) v = std::vector<Seg>();
     for (auto &v : s->plan.segs_e_z) v = std::vector<Seg>();
     CK(cudaMallocHost((void **)&s->ctl_host, 2 * sizeof(Ctl)));
@@ -713,6 +918,29 @@ ep_status setup_typed(ep_sim *s)
     CK(cudaEventCreateWithFlags(&s->ev[1], cudaEventDisableTiming));
 
     return EP_OK;
+}
+
+// Gives a set-up handle's tables back; its sweeps take the general path.
+void drop_tables(ep_sim *s)
+{
+    if (!s->tab) return;
+    if (s->stream) cudaStreamSynchronize(s->stream);
+    for (void *t : {(void *)s->rows, s->cheb_table, (void *)s->sweep_arrive, (void *)s->bricks, (void *)s->lists.k4,
+                    (void *)s->lists.k2, (void *)s->lists.vloc, (void *)s->lists.vpair, (void *)s->lists.out,
+                    (void *)s->lists.oflag}) {
+        auto it = t ? std::find(s->allocs.begin(), s->allocs.end(), t) : s->allocs.end();
+        if (it == s->allocs.end()) continue;
+        if (s->d.dev_alloc && s->d.dev_free) s->d.dev_free(t, s->d.alloc_ctx);
+        else cudaFree(t);
+        s->allocs.erase(it);
+    }
+    s->dev_bytes -= s->tab_total;
+    s->tab = s->nrows = s->nbricks = s->nsweep = 0;
+    s->lean = true;
+    for (cudaGraphExec_t *g : {&s->sweep_graph, &s->ie_graph}) {
+        if (*g) cudaGraphExecDestroy(*g);
+        *g = nullptr;
+    }
 }
 
 // Descriptor of the elliptic sweeps: the work items and records of the domain
@@ -789,6 +1017,17 @@ Inst<real> make_inst(const ep_sim *s)
         I.cheb_rho = rho;
         I.cheb_theta = std::acosh(1.0 / rho);
     }
+    // ep_step_noalloc's scratch holds kNoAllocMaxPartials partial sums: a sweep of more CTAs takes the general path
+    I.tab = s->tab && !(s->noalloc_call && (I.solver == 2 ? 8 : 1) * s->nsweep > kNoAllocMaxPartials) ? 1 : 0;
+    I.nrows = s->nrows;
+    I.nbricks = s->nbricks;
+    I.nsweep = s->nsweep;
+    I.rows = (const real *)s->rows;
+    I.bricks = s->bricks;
+    I.lists = s->lists;
+    I.cheb_table = (const real *)s->cheb_table;
+    I.sweep_arrive = s->sweep_arrive;
+    for (int i = 0; i < 9; ++i) I.row_colour[i] = s->row_colour[i];
     I.torso = s->torso.empty() ? 0 : 1;
     I.pad4 = 0;
     I.sig_o = (real)(s->torso.empty() ? 0.0 : s->sig_o);
@@ -830,15 +1069,30 @@ ApplyIO<real> no_io()
 template <typename real, int MODE>
 struct OneSweep {
     Inst<real> I;
-    void operator()(cudaStream_t q) const
+    void operator()(cudaStream_t q, int) const
     {
         k_stencil<real, MODE><<<std::max(1, I.nseg), kThreads, kSmemBytes<real, MODE>, q>>>(I, no_io<real>());
+    }
+};
+// A sweep over the tabulated operator.
+template <typename real, int MODE>
+struct TabSweep {
+    Inst<real> I;
+    void operator()(cudaStream_t q, int parity) const
+    {
+        if constexpr (sizeof(real) == 4 && !kGS<MODE>) {
+            if (I.nbricks) {
+                k_sweep<real, MODE, true><<<I.nsweep, kSweepNT<true>, kSweepSmem<MODE, true>, q>>>(I, parity);
+                return;
+            }
+        }
+        k_sweep<real, MODE, false><<<I.nsweep, kSweepNT<false>, 0, q>>>(I, parity);
     }
 };
 template <typename real, int MODE_FAR, int MODE_NEAR>
 struct SplitSweep {
     Inst<real> far, near;   // far.nseg or near.nseg may be 0
-    void operator()(cudaStream_t q) const
+    void operator()(cudaStream_t q, int) const
     {
         if (far.nseg > 0) k_stencil<real, MODE_FAR><<<far.nseg, kThreads, kSmemBytes<real, MODE_FAR>, q>>>(far, no_io<real>());
         if (near.nseg > 0) k_stencil<real, MODE_NEAR><<<near.nseg, kThreads, kSmemBytes<real, MODE_NEAR>, q>>>(near, no_io<real>());
@@ -852,7 +1106,7 @@ ep_status build_sweep_graph(ep_sim *s, const Sweep &sweep, cudaGraphExec_t *out)
     if (*out) return EP_OK;
     cudaGraph_t g = nullptr;
     CK(cudaStreamBeginCapture(s->stream, cudaStreamCaptureModeThreadLocal));
-    for (int i = 0; i < kSweepChunk; ++i) sweep(s->stream);
+    for (int i = 0; i < kSweepChunk; ++i) sweep(s->stream, i & 1);
     cudaError_t e = cudaStreamEndCapture(s->stream, &g);
     if (e != cudaSuccess) return fail(s, EP_ECUDA, std::string("sweep graph capture: ") + cudaGetErrorString(e));
     e = cudaGraphInstantiate(out, g, 0);
@@ -885,7 +1139,7 @@ ep_status run_sweeps(ep_sim *s, const Sweep &sweep, cudaGraphExec_t *graph, long
             queued += kSweepChunk;
         } else {
             const long long stop = std::min(limit, queued + (long long)kSweepChunk);
-            for (; queued < stop; ++queued) sweep(st);
+            for (; queued < stop; ++queued) sweep(st, (int)(queued & 1));
             CK(cudaGetLastError());
         }
         CK(cudaMemcpyAsync(&s->ctl_host[c & 1], s->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, st));
@@ -952,6 +1206,15 @@ ep_status configure_kernels(ep_sim *s)
     if (e == cudaSuccess) e = allow_stencil<double>(Modes{});
     if (e == cudaSuccess)
         e = allow_stencil_batch(std::integer_sequence<int, M_PAR_MONO, M_PAR_BI, M_RHS, M_JAC, M_JAC_CHEB>{});
+    auto bricks = [&](auto *k) {
+        if (e == cudaSuccess) e = allow_smem(k, kSweepSmem<M_JAC_CHEB, true>);
+    };
+    bricks(k_sweep<float, M_JAC, true>);
+    bricks(k_sweep<float, M_JAC_CHEB, true>);
+    bricks(k_sweep_batch<float, M_JAC, true>);
+    bricks(k_sweep_batch<float, M_JAC_CHEB, true>);
+    bricks(k_sweep_active<float, M_JAC, true>);
+    bricks(k_sweep_active<float, M_JAC_CHEB, true>);
     if (e == cudaSuccess) e = allow_stencil_active(std::integer_sequence<int, M_JAC, M_JAC_CHEB>{});
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -993,7 +1256,13 @@ ep_status ensure_ready(ep_sim *s)
     }
     ep_status cs = configure_kernels(s);
     if (cs != EP_OK) return cs;
-    ep_status st = s->d.precision == EP_FP64 ? setup_typed<double>(s) : setup_typed<float>(s);
+    auto setup = [&] { return s->d.precision == EP_FP64 ? setup_typed<double>(s) : setup_typed<float>(s); };
+    ep_status st = setup();
+    if (st == EP_ENOMEM && s->tab) {   // the tables do not fit: without them
+        dfree_all(s);
+        s->lean = true;
+        st = setup();
+    }
     if (st != EP_OK) {
         dfree_all(s);
         return st;
@@ -1028,7 +1297,11 @@ ep_status solve_elliptic(ep_sim *s, const Inst<real> &I, int &iters, double &rel
     long long queued = 0;
     ep_status rs = EP_OK;
     const bool cheb = I.solver == 1;   // the sweep instance matches the handle's solver
-    if (I.solver == 2) {   // eight colour passes a sweep
+    if (I.tab) {
+        rs = I.solver == 2 ? run_sweeps(s, TabSweep<real, M_JAC_GS>{I}, &s->sweep_graph, &queued, 8)
+             : cheb        ? run_sweeps(s, TabSweep<real, M_JAC_CHEB>{I}, &s->sweep_graph, &queued)
+                           : run_sweeps(s, TabSweep<real, M_JAC>{I}, &s->sweep_graph, &queued);
+    } else if (I.solver == 2) {   // eight colour passes a sweep
         rs = run_sweeps(s, OneSweep<real, M_JAC_GS>{I}, &s->sweep_graph, &queued, 8);
     } else if (s->torso.empty()) {
         rs = cheb ? run_sweeps(s, OneSweep<real, M_JAC_CHEB>{I}, &s->sweep_graph, &queued)
@@ -1590,7 +1863,6 @@ ep_status ep_get_profile(ep_sim *s, ep_profile *prof)
 // on a device share it, so calls that overlap on the GPU race.
 // ---------------------------------------------------------------------------
 namespace {
-constexpr int kNoAllocMaxPartials = 32768;     // stencil work items and reduction chunks
 constexpr int kNoAllocMaxComponents = 4096;    // face-connected tissue components
 constexpr size_t kNoAllocCtlBytes = 256;       // control block slot
 constexpr size_t kNoAllocBytes =
@@ -1761,13 +2033,13 @@ struct ep_batch {
     int model = -1;
     // device tables: descriptors, packed stencil items, packed reduction chunks
     Inst<float> *d_inst = nullptr;
-    BItem *d_seg = nullptr, *d_chunk = nullptr;
+    BItem *d_seg = nullptr, *d_chunk = nullptr, *d_sweep = nullptr;   // d_sweep: sweep CTAs of tabulated members
     long long *d_steps_left = nullptr;
     // unfinished members of the group being solved and their item prefix counts
     ActRec *d_act = nullptr;
     int *d_counts = nullptr;
     int *d_packed = nullptr;       // per table row: 1 if its sweeps go through the packed kernel
-    size_t cap_inst = 0, cap_seg = 0, cap_chunk = 0, cap_act = 0, cap_packed = 0;
+    size_t cap_inst = 0, cap_seg = 0, cap_chunk = 0, cap_act = 0, cap_packed = 0, cap_sweep = 0;
     // members with at least solo_items stencil items, and every member of a group of at most
     // kSoloAllMembers, sweep in their own launches (descriptor by value, as in the
     // single-instance step), concurrently on their own capture streams
@@ -1789,8 +2061,10 @@ struct ep_batch {
         int inst0, inst1;         // table rows [inst0, inst1)
         long long seg0, nseg;     // range of its stencil items in d_seg
         std::vector<int> solo;    // rows swept in their own launches
-        long long packed_items;   // items of the other rows (packed sweep launches)
+        long long packed_items;   // items of the other rows without a tabulated operator (packed sweep launches)
         bool cheb;                // its members' solver: Chebyshev-accelerated (else damped Jacobi)
+        long long packed_tab[2];  // sweep CTAs of those with a tabulated operator, rows and bricks (packed launches each)
+        long long sw0, nsw;       // range of its tabulated members' sweep CTAs in d_sweep
     };
     std::vector<Group> groups;
     std::vector<Ctl> last;         // per table row, after the last step
@@ -1862,7 +2136,7 @@ ep_status rebuild_tables(ep_batch *b)
     std::stable_sort(b->order.begin(), b->order.end(), [&](int x, int y) { return !is_cheb(x) && is_cheb(y); });
     b->ninst = (int)b->order.size();
     std::vector<Inst<float>> insts;
-    std::vector<BItem> segs, chunks;
+    std::vector<BItem> segs, chunks, sweeps;
     for (int r = 0; r < b->ninst; ++r) {
         ep_sim *s = b->slot[b->order[r]];
         insts.push_back(make_inst<float>(s));
@@ -1882,6 +2156,7 @@ ep_status rebuild_tables(ep_batch *b)
                  (b->group_bytes == 0 || bytes + 20 * (size_t)b->slot[b->order[r1]]->n <= b->group_bytes));
         ep_batch::Group g;
         g.cheb = cheb;
+        g.sw0 = (long long)sweeps.size();
         g.inst0 = r;
         g.inst1 = r1;
         g.seg0 = (long long)segs.size();
@@ -1897,17 +2172,26 @@ ep_status rebuild_tables(ep_batch *b)
         });
         segs.insert(segs.end(), gs.begin(), gs.end());
         g.nseg = (long long)gs.size();
+        for (int q = r; q < r1; ++q) {
+            const ep_sim *s = b->slot[b->order[q]];
+            if (s->tab) for (int i = 0; i < s->nsweep; ++i) sweeps.push_back(BItem{q, i, s->nsweep, 0});
+        }
+        g.nsw = (long long)sweeps.size() - g.sw0;
+        g.packed_tab[0] = g.packed_tab[1] = 0;
         g.packed_items = 0;
         const bool few = r1 - r <= kSoloAllMembers;
         for (int q = r; q < r1; ++q) {
             ep_sim *s = b->slot[b->order[q]];
             if (few || s->nseg >= b->solo_items) g.solo.push_back(q);
+            else if (s->tab) g.packed_tab[s->nbricks > 0] += s->nsweep;
             else g.packed_items += s->nseg;
         }
         b->groups.push_back(g);
         r = r1;
     }
-    std::vector<int> packed(b->ninst, 1);
+    std::vector<int> packed(b->ninst, 1);   // 0 solo, 1 packed, 2 and 3 packed over rows and bricks
+    for (int r = 0; r < b->ninst; ++r)
+        if (b->slot[b->order[r]]->tab) packed[r] = b->slot[b->order[r]]->nbricks > 0 ? 3 : 2;
     for (const ep_batch::Group &g : b->groups)
         for (int q : g.solo) packed[q] = 0;
     b->nseg_items = (long long)segs.size();
@@ -1916,7 +2200,8 @@ ep_status rebuild_tables(ep_batch *b)
     if ((st = grow(b, &b->d_inst, &b->cap_inst, insts.size())) != EP_OK) return st;
     if ((st = grow(b, &b->d_seg, &b->cap_seg, segs.size())) != EP_OK) return st;
     if ((st = grow(b, &b->d_chunk, &b->cap_chunk, chunks.size())) != EP_OK) return st;
-    if ((st = grow(b, &b->d_act, &b->cap_act, insts.size() + 1)) != EP_OK) return st;
+    if ((st = grow(b, &b->d_act, &b->cap_act, 3 * (insts.size() + 1))) != EP_OK) return st;   // a list per kind of sweep
+    if ((st = grow(b, &b->d_sweep, &b->cap_sweep, sweeps.size())) != EP_OK) return st;
     if ((st = grow(b, &b->d_packed, &b->cap_packed, insts.size())) != EP_OK) return st;
     if (!insts.empty()) {
         CKB(cudaMemcpyAsync(b->d_packed, packed.data(), sizeof(int) * packed.size(), cudaMemcpyHostToDevice,
@@ -1924,6 +2209,7 @@ ep_status rebuild_tables(ep_batch *b)
         CKB(cudaMemcpyAsync(b->d_inst, insts.data(), sizeof(Inst<float>) * insts.size(), cudaMemcpyHostToDevice,
                             b->stream));
         CKB(cudaMemcpyAsync(b->d_seg, segs.data(), sizeof(BItem) * segs.size(), cudaMemcpyHostToDevice, b->stream));
+        CKB(cudaMemcpyAsync(b->d_sweep, sweeps.data(), sizeof(BItem) * sweeps.size(), cudaMemcpyHostToDevice, b->stream));
         CKB(cudaMemcpyAsync(b->d_chunk, chunks.data(), sizeof(BItem) * chunks.size(), cudaMemcpyHostToDevice,
                             b->stream));
     }
@@ -1946,7 +2232,7 @@ ep_status build_batch_graph(ep_batch *b)
 {
     if (b->graph) return EP_OK;
     size_t need = 0;
-    for (const ep_batch::Group &gr : b->groups) need = std::max(need, gr.solo.size());
+    for (const ep_batch::Group &gr : b->groups) need = std::max(need, gr.solo.size() + 2);   // one branch each, and two for packed sweeps over tables
     if (need && !b->ev_fork) CKB(cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming));
     while (b->aux.size() < need) {
         cudaStream_t a = nullptr;
@@ -1994,7 +2280,14 @@ ep_status build_batch_graph(ep_batch *b)
             const int gn = gr.inst1 - gr.inst0;
             const Inst<float> *gi_inst = b->d_inst + gr.inst0;
             const int *gi_packed = b->d_packed + gr.inst0;
-            k_active_list<float><<<1, kActThreads, 0, st>>>(gi_inst, gi_packed, gn, b->d_act, b->d_counts, hg[gi]);
+            ActRec *act_tab[2] = {b->d_act + (b->ninst + 1), b->d_act + 2 * (b->ninst + 1)};
+            auto active_lists = [&](cudaStream_t q) {   // of the packed members; the loop's condition
+                k_active_list<float><<<1, kActThreads, 0, q>>>(gi_inst, gi_packed, gn, 1, b->d_act, b->d_counts, hg[gi]);
+                for (int f = 0; f < 2; ++f)
+                    if (gr.packed_tab[f] > 0)
+                        k_active_list<float><<<1, kActThreads, 0, q>>>(gi_inst, gi_packed, gn, 2 + f, act_tab[f], b->d_counts, hg[gi]);
+            };
+            active_lists(st);
             // inner loop: sweeps of the unfinished members until every solve of the group is finished
             cudaStreamCaptureStatus cs;
             cudaGraph_t cg = nullptr;
@@ -2015,35 +2308,55 @@ ep_status build_batch_graph(ep_batch *b)
             CKB(cudaStreamBeginCaptureToGraph(b->side, ibody, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
             // solo members: their own sweep chains on forked streams (parallel graph branches)
             const int nsolo = (int)gr.solo.size();
-            if (nsolo) CKB(cudaEventRecord(b->ev_fork, b->side));
+            int nbranch = nsolo;   // packed sweeps over tables run beside the others, each kind on its own branch
+            if (nsolo || gr.packed_tab[0] > 0 || gr.packed_tab[1] > 0) CKB(cudaEventRecord(b->ev_fork, b->side));
             // sweeps between loop checks: about 1 ms of sweeps (a loop pass costs tens of us), or as set
             int spc = b->sweeps_per_check;
             if (b->spc_auto) {
                 long long widest = gr.packed_items;
+                widest = std::max(widest, gr.packed_tab[0] / 4 + gr.packed_tab[1] / 2);
                 for (int q : gr.solo) widest = std::max<long long>(widest, b->slot[b->order[q]]->nseg);
                 const double waves = std::max(1.0, (double)widest / (double)(b->nsm * kMinBlocks));
                 spc = (int)std::min(64.0, std::max(8.0, std::round(1000.0 / (15.0 * waves))));
             }
+            spc += spc & 1;   // launches alternate in parity
             for (int j = 0; j < nsolo; ++j) {
                 cudaStream_t a = b->aux[j];
                 CKB(cudaStreamWaitEvent(a, b->ev_fork, 0));
                 const Inst<float> I = make_inst<float>(b->slot[b->order[gr.solo[j]]]);
                 for (int i = 0; i < spc; ++i) {
-                    if (gr.cheb) k_stencil<float, M_JAC_CHEB><<<I.nseg, kThreads, kSmemBytes<float, M_JAC_CHEB>, a>>>(I, no_io<float>());
+                    if (I.tab && gr.cheb) TabSweep<float, M_JAC_CHEB>{I}(a, i & 1);
+                    else if (I.tab) TabSweep<float, M_JAC>{I}(a, i & 1);
+                    else if (gr.cheb) k_stencil<float, M_JAC_CHEB><<<I.nseg, kThreads, kSmemBytes<float, M_JAC_CHEB>, a>>>(I, no_io<float>());
                     else k_stencil<float, M_JAC><<<I.nseg, kThreads, kSmemBytes<float, M_JAC>, a>>>(I, no_io<float>());
                 }
                 CKB(cudaEventRecord(b->ev_join[j], a));
             }
             // the other members: packed sweeps over the unfinished ones
+            auto packed_sweep = [&](auto bricks, cudaStream_t a, int i) {
+                constexpr bool B = decltype(bricks)::value;
+                const int gp = (int)gr.packed_tab[B];
+                if (gr.cheb) k_sweep_active<float, M_JAC_CHEB, B><<<gp, kSweepNT<B>, kSweepSmem<M_JAC_CHEB, B>, a>>>(gi_inst, act_tab[B], gn, i & 1);
+                else k_sweep_active<float, M_JAC, B><<<gp, kSweepNT<B>, kSweepSmem<M_JAC, B>, a>>>(gi_inst, act_tab[B], gn, i & 1);
+            };
+            for (int f = 0; f < 2; ++f) {
+                if (gr.packed_tab[f] == 0) continue;
+                cudaStream_t a = b->aux[nbranch];
+                CKB(cudaStreamWaitEvent(a, b->ev_fork, 0));
+                for (int i = 0; i < spc; ++i) {
+                    if (f) packed_sweep(std::true_type{}, a, i);
+                    else packed_sweep(std::false_type{}, a, i);
+                }
+                CKB(cudaEventRecord(b->ev_join[nbranch++], a));
+            }
             if (gr.packed_items > 0)
                 for (int i = 0; i < spc; ++i) {
                     const int gp = grid_of(gr.packed_items, 1 << 30);
                     if (gr.cheb) k_stencil_active<float, M_JAC_CHEB><<<gp, kThreads, kSmemBytes<float, M_JAC_CHEB>, b->side>>>(gi_inst, b->d_act, gn);
                     else k_stencil_active<float, M_JAC><<<gp, kThreads, kSmemBytes<float, M_JAC>, b->side>>>(gi_inst, b->d_act, gn);
                 }
-            for (int j = 0; j < nsolo; ++j) CKB(cudaStreamWaitEvent(b->side, b->ev_join[j], 0));
-            k_active_list<float><<<1, kActThreads, 0, b->side>>>(gi_inst, gi_packed, gn, b->d_act, b->d_counts,
-                                                                 hg[gi]);
+            for (int j = 0; j < nbranch; ++j) CKB(cudaStreamWaitEvent(b->side, b->ev_join[j], 0));
+            active_lists(b->side);
             CKB(cudaStreamEndCapture(b->side, nullptr));
         }
         k_comp_mean_batch<float><<<gc, kRedThreads, 0, st>>>(b->d_inst, b->d_chunk, nc, (int)RED_X_FINAL);
@@ -2140,6 +2453,21 @@ ep_status ep_batch_add(ep_batch *b, ep_sim *s, int *slot)
     if (free_slot < 0) return bfail(b, EP_EBUSY, "batch is full");
     ep_status st = ensure_ready(s);
     if (st != EP_OK) return bfail(b, st, std::string("set-up of the handle failed: ") + s->err);
+    // a budget that the handles meet without their tables admits them without
+    if (b->budget && used + s->dev_bytes > b->budget) {
+        size_t bare = used + s->dev_bytes - (s->tab ? s->tab_total : 0);
+        for (ep_sim *t : b->slot)
+            if (t && t->tab) bare -= t->tab_total;
+        if (bare <= b->budget) {
+            drop_tables(s);
+            for (ep_sim *t : b->slot)
+                if (t && t->tab && used + s->dev_bytes > b->budget) {
+                    used -= t->tab_total;
+                    drop_tables(t);
+                    b->dirty = true;
+                }
+        }
+    }
     if (b->budget && used + s->dev_bytes > b->budget)
         return bfail(b, EP_EREJECTED, "admission refused: device memory budget exceeded");
     if (s->stream) {
@@ -2261,6 +2589,7 @@ ep_status ep_batch_autotune(ep_batch *b, int trial_sweeps)
             for (int r = 0; r < b->ninst; ++r) {
                 Ctl c = ctl0[r];
                 c.done = 0; c.sweep = 0; c.arrive = 0; c.jarrive = 0; c.thresh2 = -1.0; c.bnorm2 = 1e300;
+                c.unit[0] = c.unit[1] = 0;
                 c.cycle0 = 0; c.r0n2 = 0.0;
                 CKB(cudaMemcpyAsync(b->slot[b->order[r]]->ctl, &c, sizeof(Ctl), cudaMemcpyHostToDevice, s0));
             }
@@ -2268,9 +2597,23 @@ ep_status ep_batch_autotune(ep_batch *b, int trial_sweeps)
             double ms_total = 0.0;
             for (const ep_batch::Group &gr : b->groups) {
                 const int gs = grid_of(gr.nseg, 1 << 30);
+                bool gl = false;   // a member without a tabulated operator
+                for (int r = gr.inst0; r < gr.inst1; ++r) gl = gl || !b->slot[b->order[r]]->tab;
+                int parity = 1;
                 auto sweep = [&]() {
-                    if (gr.cheb) k_stencil_batch<float, M_JAC_CHEB><<<gs, kThreads, kSmemBytes<float, M_JAC_CHEB>, s0>>>(b->d_inst, b->d_seg + gr.seg0);
-                    else k_stencil_batch<float, M_JAC><<<gs, kThreads, kSmemBytes<float, M_JAC>, s0>>>(b->d_inst, b->d_seg + gr.seg0);
+                    parity ^= 1;
+                    const int gw = (int)gr.nsw;   // every member's items on the general path, the tabulated ones skipped there
+                    auto tables = [&](auto bricks) {
+                        constexpr bool B = decltype(bricks)::value;
+                        if (gr.cheb) k_sweep_batch<float, M_JAC_CHEB, B><<<gw, kSweepNT<B>, kSweepSmem<M_JAC_CHEB, B>, s0>>>(b->d_inst, b->d_sweep + gr.sw0, parity);
+                        else k_sweep_batch<float, M_JAC, B><<<gw, kSweepNT<B>, kSweepSmem<M_JAC, B>, s0>>>(b->d_inst, b->d_sweep + gr.sw0, parity);
+                    };
+                    if (gw) {
+                        tables(std::true_type{});
+                        tables(std::false_type{});
+                    }
+                    if (gl && gr.cheb) k_stencil_batch<float, M_JAC_CHEB><<<gs, kThreads, kSmemBytes<float, M_JAC_CHEB>, s0>>>(b->d_inst, b->d_seg + gr.seg0);
+                    else if (gl) k_stencil_batch<float, M_JAC><<<gs, kThreads, kSmemBytes<float, M_JAC>, s0>>>(b->d_inst, b->d_seg + gr.seg0);
                 };
                 sweep();
                 CKB(cudaEventRecord(e0, s0));
@@ -2366,6 +2709,7 @@ void ep_batch_destroy(ep_batch *b)
     if (b->d_inst) cudaFree(b->d_inst);
     if (b->d_seg) cudaFree(b->d_seg);
     if (b->d_chunk) cudaFree(b->d_chunk);
+    if (b->d_sweep) cudaFree(b->d_sweep);
     if (b->d_act) cudaFree(b->d_act);
     if (b->d_packed) cudaFree(b->d_packed);
     for (cudaStream_t a : b->aux) cudaStreamDestroy(a);
@@ -2486,6 +2830,10 @@ void serve_loop(ep_server *v)
                 srv_erase(v->queue, r);
                 srv_finish(v, r, r->plan_status);
                 continue;
+            }
+            if (budget && r->peak > budget && !r->sim->ready && !r->sim->lean) {   // without its tables it may fit
+                r->sim->lean = true;
+                if (plan_layout(r->sim) == EP_OK) r->peak = r->sim->fp_peak;
             }
             if (budget && r->peak > budget) {
                 srv_erase(v->queue, r);

@@ -250,6 +250,7 @@ __device__ __forceinline__ void comp_subtract_item(const Inst<real> &I, int item
         ctl->jarrive = 0;
         ctl->iters = 0;
         ctl->cycle0 = 0;
+        ctl->unit[0] = ctl->unit[1] = 0;
         ctl->r0n2 = 0.0;
         ctl->converged = (t == 0.0);
         ctl->diverged = 0;
@@ -314,6 +315,7 @@ __global__ void __launch_bounds__(kRedThreads) k_ie_start(Inst<real> I)
         ctl->jarrive = 0;
         ctl->iters = 0;
         ctl->cycle0 = 0;
+        ctl->unit[0] = ctl->unit[1] = 0;
         ctl->r0n2 = 0.0;
         ctl->converged = (t == 0.0);
         ctl->diverged = 0;
@@ -594,7 +596,7 @@ __global__ void k_fill(real *p, long long n, real v)
         p[i] = v;
 }
 
-// Members of rows [0, n) swept by the packed kernel (packed[i] != 0) whose
+// Members of rows [0, n) swept by the packed kernel (packed[i] == kind) whose
 // solve is unfinished, in row order: act[k] = {items before member k, its
 // row, its control block}; entries n_active .. n hold {total items, -1,
 // null}, so the rest of the list never matches an item; counts = {total
@@ -605,7 +607,7 @@ constexpr int kActThreads = 1024;
 
 template <typename real>
 __global__ void __launch_bounds__(kActThreads)
-k_active_list(const Inst<real> *insts, const int *packed, int n, ActRec *act, int *counts,
+k_active_list(const Inst<real> *insts, const int *packed, int n, int kind, ActRec *act, int *counts,
               cudaGraphConditionalHandle h)
 {
     __shared__ int swa[32], swc[32];
@@ -620,9 +622,9 @@ k_active_list(const Inst<real> *insts, const int *packed, int n, ActRec *act, in
         Ctl *ctl = i < n ? insts[i].ctl : nullptr;
         const bool live = i < n && !*(volatile int *)&ctl->done;
         running |= live ? 1 : 0;
-        if (live && packed[i]) {
+        if (live && packed[i] == kind) {
             a = 1;
-            c = insts[i].nseg;
+            c = insts[i].tab ? insts[i].nsweep : insts[i].nseg;
         }
         int sa = a, sc = c;   // inclusive scans within the warp
         for (int o = 1; o < 32; o <<= 1) {

@@ -19,6 +19,21 @@ namespace gbep {
 constexpr int kWarps = EP_WARPS;            // warps per CTA: one per voxel-row pair
 constexpr int kThreads = kWarps * 32;
 constexpr int kTileY = kWarps - 1;          // output rows per CTA (warps 1..kWarps-1)
+#ifndef EP_BRICK_Y
+#define EP_BRICK_Y 6
+#endif
+#ifndef EP_BRICK_Z
+#define EP_BRICK_Z 8
+#endif
+#ifndef EP_SWEEP_BLOCKS
+#define EP_SWEEP_BLOCKS 8
+#endif
+#ifndef EP_BRICK_BLOCKS
+#define EP_BRICK_BLOCKS 4
+#endif
+#ifndef EP_ROWS_ONLY
+#define EP_ROWS_ONLY 720000
+#endif
 constexpr int kMinBlocks = EP_MIN_BLOCKS;   // occupancy hint for the stencil kernels
 constexpr int kTileX = 30;                  // output voxels per row (lanes 1..30)
 constexpr int kMaxStim = 8;
@@ -73,9 +88,12 @@ struct StimSet {
 };
 
 // Device control block of one instance: step counter and the elliptic solve.
-struct Ctl {
-    unsigned int arrive;  // work items that finished the current launch (reset by the last one)
+struct alignas(16) Ctl {
+    // read together by every sweep CTA over the tabulated operator
     int done;             // solve finished: converged, capped, diverged or empty rhs
+    int cycle0;           // Chebyshev / Jacobi in correction form: the sweep that starts the current cycle
+    int unit[2];          // launch index of the solve: a launch of parity p reads unit[p] and leaves unit[p ^ 1]
+    unsigned int arrive;  // work items that finished the current launch (reset by the last one)
     int sweep;            // sweeps done in the current solve, as of its last residual check
     int iters;            // sweeps of the finished solve
     int converged;
@@ -92,15 +110,31 @@ struct Ctl {
     // jarrive / nitems = j; sweeps that do not check the residual only add to it
     unsigned long long jarrive;
     long long ie_total;   // sweeps of the implicit parabolic solves, summed over steps
-    // Chebyshev solve in correction form: the sweep that starts the current cycle, and
-    // ||r||^2 at that cycle's start
-    int cycle0, pad_c;
-    double r0n2;
+    double r0n2;          // correction form: ||r||^2 at the current cycle's start
 };
 
 struct Chunk {
     int start, end, comp;  // [start, end) into the component-sorted tissue index list
 };
+
+// One brick of the tabulated operator: voxels x in [x0, x0 + 30), y in [y0, y0 + kBrickY), z in [z0, z0 + planes);
+// its vertices are entries [vbase, vbase + nvert) of the vertex lists, the full ones first; its tissue voxels are
+// entries [obase, obase + nout) of the voxel lists, the inner ones first.
+struct Brick {
+    int x0, y0, z0, planes;
+    int vbase, nfull, nvert, pbase;
+    int obase, ninner, nout, fbase;
+};
+struct BrickLists {
+    float4 *k4;               // K00 K11 K22 K01 of a vertex
+    float2 *k2;               // K02 K12
+    unsigned short *vloc;     // its place in the lattice, 5 + 4 + 4 bits
+    unsigned short *vpair;    // valid pairs of a vertex that is not full (entry pbase + rank)
+    float2 *out;              // a voxel's 1/Dhat and (as bits) its place in the brick
+    unsigned char *oflag;     // tissue flags of the neighbours -x +x -y +y -z +z of a boundary voxel (fbase + rank)
+};
+constexpr int kChebTable = 8192;    // tabulated Chebyshev weights
+constexpr int kArriveGroups = 32, kArriveStride = 32;   // counters, and words between them
 
 // Everything a kernel needs about one simulation instance.  Passed by value
 // to the single-instance kernels and read from a device table by the
@@ -157,6 +191,15 @@ struct Inst {
     // by a factor 1e3 (kRestart2)
     real *x2;
     int eform, pad5;
+    // tabulated elliptic operator (tab != 0): a sweep is nsweep CTAs over its bricks or its assembled rows
+    // (the eight-colour sweep: rows [row_colour[c], row_colour[c + 1]) in pass c)
+    int tab, nrows, nbricks, nsweep;
+    const real *rows;
+    const Brick *bricks;
+    BrickLists lists;
+    const real *cheb_table;
+    unsigned *sweep_arrive;   // arrivals of a checking sweep: kArriveGroups counters and the groups', 128 bytes apart
+    int row_colour[9], pad6;
 };
 
 // A correction-form cycle restarts when ||r||^2 has fallen below this fraction of

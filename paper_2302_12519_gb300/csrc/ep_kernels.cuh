@@ -4,3 +4,5 @@
 #include "ep_common.cuh"
 #include "ep_stencil.cuh"
 #include "ep_aux.cuh"
+#include "ep_tables.cuh"
+#include "ep_sweep.cuh"

@@ -527,6 +527,31 @@ __device__ __forceinline__ void ring_plane(const Inst<real> &I, const Op<real> &
     plane_step<real, MODE>(I, o, g, k, k > kbeg, k > kbeg + 1, P, Cn, L, sF, sT, ts, check, acc);
 }
 
+// Decision of a checking sweep, by one thread: s is ||r||^2 of the sweep's input.
+template <typename real>
+__device__ __forceinline__ void sweep_decide(const Inst<real> &I, int sweep, bool eform, double s)
+{
+    Ctl *ctl = I.ctl;
+    const int j = sweep + 1;
+    ctl->sweep = j;
+    ctl->rnorm2 = s;
+    if (!(s == s) || isinf(s)) {
+        ctl->nonfinite = 1; ctl->done = 1; ctl->iters = j;
+    } else if (s <= ctl->thresh2) {
+        ctl->converged = 1; ctl->done = 1; ctl->iters = j;
+    } else if (s > I.div_factor * ctl->bnorm2) {
+        ctl->diverged = 1; ctl->noconv = 1; ctl->done = 1; ctl->iters = j;
+    } else if (eform) {   // correction form: sweep 0 starts the first cycle; a cycle that
+        if (sweep == 0) {  // has cut ||r|| by 1e3 restarts at the next sweep
+            ctl->r0n2 = s;
+        } else if (s <= kRestart2 * ctl->r0n2) {
+            ctl->cycle0 = j;
+            ctl->r0n2 = s;
+        }
+    }
+    __threadfence();
+}
+
 // End of a sweep's work item: count its arrival; on a checking sweep the item
 // that arrives last sums the FP64 partial norms in a fixed order and decides
 // the stop (converged, diverged, non-finite) in the control block.
@@ -559,26 +584,7 @@ __device__ __forceinline__ void sweep_finish(const Inst<real> &I, int sweep, int
         double s = 0;
         for (int i = threadIdx.x; i < parts * nitems; i += kThreads) s += ((volatile double *)I.partials)[i];
         s = block_sum<kThreads>(s, sred);
-        if (threadIdx.x == 0) {
-            const int j = sweep + 1;
-            ctl->sweep = j;
-            ctl->rnorm2 = s;
-            if (!(s == s) || isinf(s)) {
-                ctl->nonfinite = 1; ctl->done = 1; ctl->iters = j;
-            } else if (s <= ctl->thresh2) {
-                ctl->converged = 1; ctl->done = 1; ctl->iters = j;
-            } else if (s > I.div_factor * ctl->bnorm2) {
-                ctl->diverged = 1; ctl->noconv = 1; ctl->done = 1; ctl->iters = j;
-            } else if (eform) {   // correction form: sweep 0 starts the first cycle; a cycle that
-                if (sweep == 0) {  // has cut ||r|| by 1e3 restarts at the next sweep
-                    ctl->r0n2 = s;
-                } else if (s <= kRestart2 * ctl->r0n2) {
-                    ctl->cycle0 = j;
-                    ctl->r0n2 = s;
-                }
-            }
-            __threadfence();
-        }
+        if (threadIdx.x == 0) sweep_decide(I, sweep, eform, s);
         __syncthreads();
     }
 }
@@ -801,6 +807,7 @@ k_stencil_batch(const Inst<real> *insts, const BItem *items)
     StencilSmem<real, MODE> &sm = dyn_smem<StencilSmem<real, MODE>>();
     __shared__ Inst<real> sI;
     const BItem it = items[blockIdx.x];
+    if (kJac<MODE> && insts[it.inst].tab) return;   // this member's sweeps run over its tabulated operator
     if (kJac<MODE> && cta_done(insts[it.inst].ctl, &sm.sflag)) return;
     const Inst<real> &I = stage_inst(insts + it.inst, sI);
     stencil_item<real, MODE>(I, it.item, it.item, it.nitems, nullptr, sm);

@@ -1,0 +1,433 @@
+// ep_sweep.cuh -- sweeps of the elliptic solve over the tabulated operator (ep_tables.cuh).
+//
+// Rows: a thread a row, 112 bytes of coefficients and 26 neighbours all in flight together, so a sweep is two rounds
+// of memory latency whatever the grid's shape.  Bound by latency while the rows stay in L2 (48^3 shell, 10.5 thousand
+// voxels: 3.2 us a sweep, the z-march 8.1; 128^3 shell, 199 thousand: 6.7 against 11.6), by their bytes above that.
+// A colour pass of Gauss-Seidel reads its own eighth of the rows only: 6.9 us a pass on 1.10 million voxels, where
+// the march forms every flux for one voxel in eight, 32 us.
+// Bricks: 36 bytes of K and place a voxel (30 x 6 x 8 bricks share their lattices' faces), 16 of fields.  Bound by
+// memory latency: the lists alone stream in 32 us of the 256^3 heart's 55.6 (3.41 million voxels; the march 69.9, bound
+// by its instructions, 53 million against 33).  Measured against it and dropped: a z-march over K with packed columns
+// and masked loads (54 us with the surface voxels as rows; its loads wait on one another), the same with a cp.async
+// ring (65 us), bricks of 6 x 6 (58.7) and 8 x 12 (91), two bricks in flight a CTA (58), all loads of a brick at
+// once (61).
+#pragma once
+
+#include "ep_stencil.cuh"
+#include "ep_tables.cuh"
+
+namespace gbep {
+
+// Loads under a predicate, else the given value: no branch, so the loads of a row or a plane are all in flight
+// together.  Volatile: the iterates change between launches, not within one, but b and x_{k-1} are overwritten by
+// the thread that reads them.
+__device__ __forceinline__ float load_if(bool on, const float *p, float other)
+{
+    float x = other;
+    asm volatile("{ .reg .pred p; setp.ne.u32 p, %1, 0; @p ld.global.f32 %0, [%2]; }" : "+f"(x) : "r"((unsigned)on), "l"(p));
+    return x;
+}
+__device__ __forceinline__ double load_if(bool on, const double *p, double other)
+{
+    double x = other;
+    asm volatile("{ .reg .pred p; setp.ne.u32 p, %1, 0; @p ld.global.f64 %0, [%2]; }" : "+d"(x) : "r"((unsigned)on), "l"(p));
+    return x;
+}
+
+constexpr int kSweepThreads = 128;
+constexpr int kBrickThreads = 32 * kTileRows;
+
+// What a sweep works on, from the control block and the descriptor.
+template <typename real>
+struct SweepOp {
+    real coef;         // omega / C, or tau / C
+    real cheb_w;       // Chebyshev weight (1: the basic step)
+    int cform;         // kRestart | kFold | kPrev0
+    int cheb;          // semi-iteration active in this sweep
+    int sweep, unit, colour;
+    bool check;
+};
+
+// False when the solve is finished or at its cap.  Every thread reads the control block itself, one 16-byte load
+// that the SM's CTAs share through L1: the flag changes within a launch only at the cap, where every warp of the
+// launch leaves here on either reading.  The launch index comes from the slot of this launch's parity, which the
+// launch before wrote: counting arrivals on one address instead cost 10 ns a CTA, 17 us a sweep at 1600 CTAs.
+template <typename real, int MODE>
+__device__ __forceinline__ bool sweep_begin(const Inst<real> &I, int parity, SweepOp<real> &o)
+{
+    Ctl *ctl = I.ctl;
+    const int4 c = *reinterpret_cast<const int4 *>(ctl);   // done, cycle0, unit[2]
+    const int cycle0 = c.y;
+    if (c.x) return false;
+    o.unit = parity ? c.w : c.z;
+    o.sweep = kGS<MODE> ? o.unit >> 3 : o.unit;
+    o.colour = o.unit & 7;
+    if (o.sweep >= I.max_iter) {
+        if (threadIdx.x == 0) {
+            ctl->noconv = 1;
+            ctl->iters = o.sweep;
+            __threadfence();
+            ctl->done = 1;
+        }
+        return false;
+    }
+    o.check = (o.sweep % I.check_every) == 0;
+    o.coef = I.coef_jac;
+    o.cform = o.cheb = 0;
+    o.cheb_w = real(1);
+    if (kGS<MODE>) return true;
+    int kc = o.sweep;
+    if (I.eform) {   // the iterate is x0 + e: sweep 0 reads x0 (e = 0), later sweeps read e
+        kc = o.sweep - cycle0;
+        o.cform = (kc == 0 ? kRestart : 0) | (kc == 0 && o.sweep > 0 ? kFold : 0) | (kc == 1 ? kPrev0 : 0);
+    }
+    if (kCheb<MODE>) {
+        o.coef = I.cheb_tau_c;
+        if (kc > 0) {
+            o.cheb = 1;
+            if (kc < kChebTable - 1 || 2.0 * I.cheb_theta * kc > 45.0) o.cheb_w = I.cheb_table[min(kc, kChebTable - 1)];
+            else o.cheb_w = (real)cheb_weight(kc, I.cheb_rho, I.cheb_theta);   // a tiny interval, not at its limit yet
+        }
+    }
+    return true;
+}
+
+// Iterate read and written by a launch of this parity (Chebyshev: the latter holds x_{k-1} until then).  A solve's
+// first launch has parity 0, so the parity is the sweep's own and the buffers are known without the control block,
+// but for the first sweep of a correction-form solve, which reads x0.
+template <typename real, int MODE>
+__device__ __forceinline__ const real *sweep_src(const Inst<real> &I, int parity)
+{
+    if (kGS<MODE>) return I.x0;
+    return parity ? I.x1 : I.eform ? I.x2 : I.x0;
+}
+template <typename real, int MODE>
+__device__ __forceinline__ real *sweep_dst(const Inst<real> &I, int parity)
+{
+    if (kGS<MODE>) return I.x0;
+    return !parity ? I.x1 : I.eform ? I.x2 : I.x0;
+}
+
+// New value of voxel q from its value u, the operator's Lu, b_q, 1/Dhat and x_{k-1}; returns the residual.
+template <typename real, int MODE>
+__device__ __forceinline__ real sweep_out(const Inst<real> &I, const SweepOp<real> &o, real *out, int q, real u,
+                                          real Lu, real b, real d, real prev)
+{
+    const real r = b - Lu;
+    if (o.cform & kRestart) {   // first sweep of a cycle: fold e into x0, r becomes the right-hand side
+        if (o.cform & kFold) I.x0[q] += u;
+        I.b[q] = r;
+        out[q] = o.coef * d * r;
+    } else {
+        const real basic = u + o.coef * d * r;
+        if (kCheb<MODE> && o.cheb) {
+            if (o.cform & kPrev0) prev = real(0);
+            out[q] = o.cheb_w * (basic - prev) + prev;
+        } else {
+            out[q] = basic;
+        }
+    }
+    return r;
+}
+
+// The 28 values of an assembled row.
+template <typename real>
+__device__ __forceinline__ void row_load(const Inst<real> &I, int row, real (&c)[kRowLen])
+{
+    using V = typename Vec4<real>::type;
+    const V *R = reinterpret_cast<const V *>(I.rows) + row;
+#pragma unroll
+    for (int g = 0; g < kRowLen / 4; ++g) {
+        const V a = R[(size_t)g * I.nrows];
+        c[4 * g] = a.x; c[4 * g + 1] = a.y; c[4 * g + 2] = a.z; c[4 * g + 3] = a.w;
+    }
+}
+
+// L u = sum A(q, q') (u_q' - u_q) of a row at s = &u_q.  A zero coefficient reads nothing (its neighbour may lie off
+// the grid or the domain).
+template <typename real>
+__device__ __forceinline__ real row_apply(const Inst<real> &I, const real (&c)[kRowLen], const real *s, real u)
+{
+    const int plane = I.nx * I.ny;
+    real nb[26];
+#pragma unroll
+    for (int t = 0; t < 26; ++t) {
+        nb[t] = load_if(c[t] != real(0), s + (nb_dx(t) + I.nx * nb_dy(t) + plane * nb_dz(t)), u);
+    }
+    real Lu0 = real(0), Lu1 = real(0);
+#pragma unroll
+    for (int t = 0; t < 26; t += 2) {
+        Lu0 += c[t] * (nb[t] - u);
+        Lu1 += c[t + 1] * (nb[t + 1] - u);
+    }
+    return Lu0 + Lu1;
+}
+
+template <typename real, int MODE>
+__device__ __forceinline__ real sweep_row(const Inst<real> &I, const SweepOp<real> &o, const real *src, real *out,
+                                          int row)
+{
+    real c[kRowLen];
+    row_load(I, row, c);
+    const int q = row_index(c[27]);
+    const real u = src[q], b = I.b[q];
+    const real prev = kCheb<MODE> && o.cheb ? out[q] : real(0);
+    return sweep_out<real, MODE>(I, o, out, q, u, row_apply(I, c, src + q, u), b, c[26], prev);
+}
+
+struct BrickSmem {
+    float u[kTile];
+    float c[4][kLat];
+};
+
+// One brick, in three rounds: the tile of u into shared memory (cp.async); the flux F = K g of every vertex of the
+// list; and the transposed gradient at every tissue voxel.  A voxel takes from each of its eight vertices
+// +-F0 +-F1 +-F2 with the signs of the vertex's place, so a vertex leaves c0 = F0 + F1 + F2, c1 = F0 + F1 - F2,
+// c2 = F0 - F1 + F2 and c3 = -F0 + F1 + F2 and an inner voxel reads eight values instead of 24.  A boundary voxel
+// drops the components towards neighbours that are not tissue: it reads F0 = (c1 + c2) / 2 and so on.
+// The lists make every lane work on tissue; a thread loads its next entries while it works on these.
+template <int MODE>
+__device__ __forceinline__ void sweep_brick(const Inst<float> &I, const SweepOp<float> &o, const float *src,
+                                            float *out, const Brick &B, BrickSmem &sm, double &acc)
+{
+    static_assert(kBrickThreads == 32 * kTileRows, "a warp loads one row of each tile plane");
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int nx = I.nx, plane = I.nx * I.ny;
+    {
+        const int x = B.x0 - 1 + lane, y = B.y0 - 1 + wid;
+        if (x >= 0 && x < nx && y >= 0 && y < I.ny) {
+            const int z0 = B.z0 > 0 ? -1 : 0, z1 = B.z0 + B.planes < I.nz ? B.planes : B.planes - 1;
+            const float *g = src + (x + nx * y + plane * (B.z0 + z0));
+            float *d = sm.u + 32 * (wid + kTileRows * (z0 + 1)) + lane;
+            for (int z = z0; z <= z1; ++z, g += plane, d += 32 * kTileRows) cp_async_n<4>(d, g);
+        }
+        cp_async_commit();
+    }
+    // K and places of the thread's next two vertices, a pair ahead
+    float4 ka0, ka1;
+    float2 kb0, kb1;
+    unsigned loc0 = 0, loc1 = 0;
+    auto vertex = [&](int t, float4 &ka, float2 &kb, unsigned &loc) {
+        if (t < B.nvert) {
+            ka = __ldcs(I.lists.k4 + (B.vbase + t));
+            kb = __ldcs(I.lists.k2 + (B.vbase + t));
+            loc = __ldcs(I.lists.vloc + (B.vbase + t));
+        }
+    };
+    vertex(threadIdx.x, ka0, kb0, loc0);
+    vertex(threadIdx.x + kBrickThreads, ka1, kb1, loc1);
+    // the thread's voxels: list entries two ahead, b and x_{k-1} one ahead
+    const int q0 = B.x0 + nx * B.y0 + plane * B.z0;
+    float2 e0 = make_float2(0.f, 0.f), e1 = e0;
+    float b0 = 0.f, p0 = 0.f;
+    auto voxel = [&](int t, float2 &e) {
+        if (t < B.nout) e = __ldcs(I.lists.out + (B.obase + t));
+    };
+    auto place = [&](const float2 &e) {
+        const int at = __float_as_int(e.y);
+        return q0 + (at & 31) + nx * ((at >> 5) & 15) + plane * (at >> 9);
+    };
+    auto own = [&](int t, const float2 &e) {
+        if (t < B.nout) {
+            b0 = I.b[place(e)];
+            if (kCheb<MODE> && o.cheb) p0 = out[place(e)];
+        }
+    };
+    voxel(threadIdx.x, e0);
+    cp_async_wait<0>();
+    __syncthreads();
+    auto flux = [&](int t, const float4 &ka, const float2 &kb, unsigned loc) {
+        const int lx = loc & 31, ly = (loc >> 5) & 15, lz = loc >> 9;
+        const float *u = sm.u + lx + 32 * (ly + kTileRows * lz);
+        const float u0 = u[0], u1 = u[1], u2 = u[32], u3 = u[33];
+        const float *v = u + 32 * kTileRows;
+        const float u4 = v[0], u5 = v[1], u6 = v[32], u7 = v[33];
+        float gx, gy, gz;
+        if (t < B.nfull) {
+            const float s0 = u0 + u1, s1 = u2 + u3, s2 = u4 + u5, s3 = u6 + u7;
+            gx = ((u1 - u0) + (u3 - u2)) + ((u5 - u4) + (u7 - u6));
+            gy = (s1 - s0) + (s3 - s2);
+            gz = (s2 - s0) + (s3 - s1);
+        } else {
+            const unsigned w = I.lists.vpair[B.pbase + t - B.nfull];
+            auto pair = [&](int bit, float lo, float hi) { return (w >> bit) & 1u ? hi - lo : 0.f; };
+            gx = (pair(0, u0, u1) + pair(1, u2, u3)) + (pair(2, u4, u5) + pair(3, u6, u7));
+            gy = (pair(4, u0, u2) + pair(5, u1, u3)) + (pair(6, u4, u6) + pair(7, u5, u7));
+            gz = (pair(8, u0, u4) + pair(9, u1, u5)) + (pair(10, u2, u6) + pair(11, u3, u7));
+        }
+        const float F0 = ka.x * gx + ka.w * gy + kb.x * gz;
+        const float F1 = ka.w * gx + ka.y * gy + kb.y * gz;
+        const float F2 = kb.x * gx + kb.y * gy + ka.z * gz;
+        float *c = sm.c[0] + lx + kLatX * (ly + kLatY * lz);
+        c[0] = (F0 + F1) + F2;
+        c[kLat] = (F0 + F1) - F2;
+        c[2 * kLat] = (F0 - F1) + F2;
+        c[3 * kLat] = (F1 - F0) + F2;
+    };
+    for (int t = threadIdx.x; t < B.nvert; t += 2 * kBrickThreads) {
+        const float4 a = ka0, e = ka1;
+        const float2 b = kb0, f = kb1;
+        const unsigned la = loc0, le = loc1;
+        vertex(t + 2 * kBrickThreads, ka0, kb0, loc0);
+        vertex(t + 3 * kBrickThreads, ka1, kb1, loc1);
+        flux(t, a, b, la);
+        if (t + kBrickThreads < B.nvert) flux(t + kBrickThreads, e, f, le);
+    }
+    own(threadIdx.x, e0);
+    voxel(threadIdx.x + kBrickThreads, e1);
+    __syncthreads();
+    for (int t = threadIdx.x; t < B.nout; t += kBrickThreads) {
+        const int at = __float_as_int(e0.y), ox = at & 31, oy = (at >> 5) & 15, oz = at >> 9, q = place(e0);
+        const float bt = b0, dt = e0.x, pt = p0;
+        e0 = e1;
+        own(t + kBrickThreads, e0);
+        voxel(t + 2 * kBrickThreads, e1);
+        const int l = ox + kLatX * (oy + kLatY * oz);
+        constexpr int Y = kLatX, Z = kLatX * kLatY;
+        float Lu;
+        if (t < B.ninner) {
+            const float *c0 = sm.c[0] + l, *c1 = sm.c[1] + l, *c2 = sm.c[2] + l, *c3 = sm.c[3] + l;
+            Lu = ((c0[0] - c0[1 + Y + Z]) + (c1[Z] - c1[1 + Y])) + ((c2[Y] - c2[1 + Z]) + (c3[1] - c3[Y + Z]));
+        } else {
+            const unsigned f = I.lists.oflag[B.fbase + t - B.ninner];
+            float x0 = 0.f, x1 = 0.f, y0 = 0.f, y1 = 0.f, z0 = 0.f, z1 = 0.f;   // twice the sums over each face
+#pragma unroll
+            for (int v = 0; v < 8; ++v) {
+                const int m = l + (v & 1) + Y * ((v >> 1) & 1) + Z * (v >> 2);
+                const float c1 = sm.c[1][m], c2 = sm.c[2][m], c3 = sm.c[3][m];
+                (v & 1 ? x1 : x0) += c1 + c2;
+                (v & 2 ? y1 : y0) += c1 + c3;
+                (v & 4 ? z1 : z0) += c2 + c3;
+            }
+            auto face = [&](int bit, float s) { return (f >> bit) & 1u ? s : 0.f; };
+            Lu = 0.5f * (((face(0, x0) - face(1, x1)) + (face(2, y0) - face(3, y1))) + (face(4, z0) - face(5, z1)));
+        }
+        const float u = sm.u[ox + 1 + 32 * (oy + 1 + kTileRows * (oz + 1))];
+        const float r = sweep_out<float, MODE>(I, o, out, q, u, Lu, bt, dt, pt);
+        if (o.check) acc += (double)(r * r);
+    }
+}
+
+// The work of CTA `cta` of the I.nsweep CTAs of a sweep, a brick or a share of the rows.  BRICKS: the handle's form,
+// and NT threads.
+template <typename real, int MODE, bool BRICKS>
+__device__ __forceinline__ void sweep_cta(const Inst<real> &I, int parity, int cta, BrickSmem *sm, double *sred,
+                                          int *sflag)
+{
+    constexpr int NT = BRICKS ? kBrickThreads : kSweepThreads;
+    SweepOp<real> o;
+    Brick B{};
+    if constexpr (BRICKS) B = I.bricks[cta];
+    if (!sweep_begin<real, MODE>(I, parity, o)) return;
+    if (cta == 0 && threadIdx.x == 0) I.ctl->unit[parity ^ 1] = o.unit + 1;
+    const real *src = !kGS<MODE> && I.eform && o.sweep == 0 ? I.x0 : sweep_src<real, MODE>(I, parity);
+    real *out = sweep_dst<real, MODE>(I, parity);
+    double acc = 0.0;
+    if constexpr (BRICKS) {
+        sweep_brick<MODE>(I, o, src, out, B, *sm, acc);
+    } else {
+        const int r0 = kGS<MODE> ? I.row_colour[o.colour] : 0, r1 = kGS<MODE> ? I.row_colour[o.colour + 1] : I.nrows;
+        for (int i = r0 + cta * NT + threadIdx.x; i < r1; i += I.nsweep * NT) {
+            const real r = sweep_row<real, MODE>(I, o, src, out, i);
+            if (o.check) {
+                const float f = (float)r;
+                acc += (double)(f * f);
+            }
+        }
+    }
+    if (!o.check) return;
+    // FP64 partial norms, summed in a fixed order by the CTA that arrives last.  CTAs count in groups, each counter
+    // on its own line, and the last of a group counts the group.
+    const int part = kGS<MODE> ? o.colour : 0, parts = kGS<MODE> ? 8 : 1;
+    const double tot = block_sum<NT>(acc, sred);
+    if (threadIdx.x == 0) {
+        I.partials[part * I.nsweep + cta] = tot;
+        __threadfence();
+        const int g = cta % kArriveGroups, groups = min(I.nsweep, kArriveGroups);
+        const unsigned size = (unsigned)((I.nsweep - g + kArriveGroups - 1) / kArriveGroups);
+        unsigned *mine = I.sweep_arrive + (g + 1) * kArriveStride;
+        bool last = atomicAdd(mine, 1u) == size - 1u;
+        if (last) {
+            *mine = 0u;
+            __threadfence();
+            last = atomicAdd(I.sweep_arrive, 1u) == (unsigned)groups - 1u;
+            if (last) *I.sweep_arrive = 0u;
+        }
+        *sflag = last && part == parts - 1;
+    }
+    __syncthreads();
+    if (*sflag) {
+        __threadfence();
+        double s = 0;
+        for (int i = threadIdx.x; i < parts * I.nsweep; i += NT) s += ((volatile double *)I.partials)[i];
+        s = block_sum<NT>(s, sred);
+        if (threadIdx.x == 0) sweep_decide(I, o.sweep, !kGS<MODE> && I.eform, s);
+    }
+}
+
+// Bytes of dynamic shared memory and threads of a sweep CTA.
+template <int MODE, bool BRICKS>
+constexpr size_t kSweepSmem = BRICKS ? sizeof(BrickSmem) : 0;
+template <bool BRICKS>
+constexpr int kSweepNT = BRICKS ? kBrickThreads : kSweepThreads;
+template <typename real, bool BRICKS>
+constexpr int kSweepMinBlocks = sizeof(real) == 8 ? 2 : BRICKS ? EP_BRICK_BLOCKS : EP_SWEEP_BLOCKS;
+
+// Single instance.
+template <typename real, int MODE, bool BRICKS>
+__global__ void __launch_bounds__(kSweepNT<BRICKS>, kSweepMinBlocks<real, BRICKS>) k_sweep(Inst<real> I, int parity)
+{
+    extern __shared__ __align__(16) unsigned char ep_sweep_smem[];
+    __shared__ double sred[kSweepNT<BRICKS> / 32];
+    __shared__ int sflag;
+    sweep_cta<real, MODE, BRICKS>(I, parity, blockIdx.x, reinterpret_cast<BrickSmem *>(ep_sweep_smem), sred, &sflag);
+}
+
+// Batched: the sweep CTAs of all members of a list with this form (the batch's trial sweeps).
+template <typename real, int MODE, bool BRICKS>
+__global__ void __launch_bounds__(kSweepNT<BRICKS>, kSweepMinBlocks<real, BRICKS>)
+k_sweep_batch(const Inst<real> *insts, const BItem *items, int parity)
+{
+    extern __shared__ __align__(16) unsigned char ep_sweep_smem[];
+    __shared__ double sred[kSweepNT<BRICKS> / 32];
+    __shared__ int sflag;
+    __shared__ Inst<real> sI;
+    const BItem it = items[blockIdx.x];
+    const Inst<real> &I = stage_inst(insts + it.inst, sI);
+    if ((I.nbricks > 0) != BRICKS) return;
+    sweep_cta<real, MODE, BRICKS>(I, parity, it.item, reinterpret_cast<BrickSmem *>(ep_sweep_smem), sred, &sflag);
+}
+
+// Batched: the unfinished members of a list (see k_stencil_active).  The descriptor is copied before the finished
+// flag is read, so a warp that leaves early has done its share.
+template <typename real, int MODE, bool BRICKS>
+__global__ void __launch_bounds__(kSweepNT<BRICKS>, kSweepMinBlocks<real, BRICKS>)
+k_sweep_active(const Inst<real> *insts, const ActRec *act, int n, int parity)
+{
+    extern __shared__ __align__(16) unsigned char ep_sweep_smem[];
+    __shared__ double sred[kSweepNT<BRICKS> / 32];
+    __shared__ int sflag, sk;
+    __shared__ Inst<real> sI;
+    const int i = blockIdx.x;
+    if (threadIdx.x == 0) sk = -1;
+    __syncthreads();
+    for (int k = threadIdx.x; k < n; k += blockDim.x) {
+        const ActRec a = act[k];
+        if (a.inst >= 0 && a.cum <= i && i < act[k + 1].cum) sk = k;
+    }
+    __syncthreads();
+    if (sk < 0) return;
+    const ActRec r = act[sk];
+    const Inst<real> &I = stage_inst(insts + r.inst, sI);
+    sweep_cta<real, MODE, BRICKS>(I, parity, i - r.cum, reinterpret_cast<BrickSmem *>(ep_sweep_smem), sred, &sflag);
+}
+
+// cheb_weight(k) for k < kChebTable - 1; the last entry is the weights' limit 2 e^-theta / rho.
+template <typename real>
+__global__ void k_cheb_table(double rho, double theta, real *t)
+{
+    for (int k = threadIdx.x; k < kChebTable; k += blockDim.x)
+        t[k] = (real)(k < kChebTable - 1 ? cheb_weight(k, rho, theta) : (2.0 / rho) * exp(-theta));
+}
+
+}  // namespace gbep

@@ -1,0 +1,93 @@
+"""Sweeps over the tabulated operator (assembled rows and bricks) against the FP64 oracle: a few capped sweeps from a
+random state, so that every voxel's value depends on its own row or brick entries, at sizes around the edges of a
+row CTA (128 rows), a brick (30 x 6 x 8 voxels) and its lattice, ragged grids, grids with holes and thin ones."""
+import numpy as np
+import pytest
+
+import oracle
+import paper_2302_12519_gb300 as ep
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+SWEEPS = 4
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_2302_12519_gb300 import build
+    build.build()
+    ep.load()
+
+
+def _mask(kind, seed, nx, ny, nz):
+    rng = np.random.default_rng(seed)
+    if kind == "full":
+        return np.ones((nz, ny, nx), np.uint8)
+    if kind == "holes":
+        return (rng.random((nz, ny, nx)) > 0.03).astype(np.uint8)
+    return W.random_mask(rng, nx, ny, nz, 0.8)
+
+
+def _check(kind, seed, nx, ny, nz, solver, precision):
+    c = W.random_case(seed, nx, ny, nz, mask=_mask(kind, seed, nx, ny, nz), precision=precision).fibres_as_float32()
+    p = c.params
+    p.solver, p.max_iter, p.rel_tol, p.check_every = solver, SWEEPS, 0.0, 2
+    p.cheb_lmin, p.cheb_lmax = (0.01, 5.5) if solver == 1 else (0.0, 0.0)
+    p.omega = 1.3 if solver == 2 else 0.0
+    v, w, ve = W.random_state(seed, c)
+    s, ref = ep.sim_from_case(c), oracle.Sim(c)
+    s.set_state(v, w, ve, 0)
+    ref.set_state(v, w, ve, 0)
+    st = s.step(1, allow_noconv=True)
+    ref.step()
+    assert st.iters == SWEEPS
+    want = ref.state()
+    # a sweep moves a voxel by omega / D times sums of at most 26 products of coefficients (their sum at most 6 D)
+    # and values: 32 roundings of 2^-24 (FP64: 2^-53, but 1/D is stored in FP32) of 6 max|x| a sweep, after the
+    # rounding of v, the right-hand side and the start, four more of the same size
+    x = max(1.0, float(np.abs(want["ve"]).max()))
+    eps = 2.0 ** -24
+    tol = (32 * 6 * SWEEPS + 4 * 32) * eps * x if precision == W.FP32 else 6 * SWEEPS * eps * x
+    assert np.abs(s.read(ep.EP_VE) - want["ve"]).max() <= tol
+    s.close()
+    ref.close()
+
+
+# up to 720 000 tissue voxels: rows.  4 096 is the smallest tabulated handle, 4 095 the largest general one.
+@pytest.mark.parametrize("precision", [W.FP32, W.FP64])
+@pytest.mark.parametrize("solver", [0, 1, 2])
+@pytest.mark.parametrize("kind,nx,ny,nz", [("full", 16, 16, 16), ("full", 4095, 1, 1), ("holes", 33, 31, 29),
+                                           ("blobs", 47, 40, 23), ("full", 2, 64, 65)])
+def test_rows(kind, nx, ny, nz, solver, precision):
+    _check(kind, 3, nx, ny, nz, solver, precision)
+
+
+@pytest.mark.parametrize("solver", [0, 1])
+@pytest.mark.parametrize("kind,nx,ny,nz", [("full", 91, 91, 89), ("holes", 120, 84, 78), ("holes", 31, 161, 151),
+                                           ("blobs", 122, 107, 91)])
+def test_bricks(kind, nx, ny, nz, solver):
+    _check(kind, 5, nx, ny, nz, solver, W.FP32)
+
+
+def test_tables_give_way_to_a_budget():
+    """A batch budget that two handles meet without their tables, but not with them, admits both; they give the
+    results of a handle that never had tables to the rounding of the operator's two forms."""
+    c = W.random_case(8, 40, 30, 20, mask=np.ones((20, 30, 40), np.uint8))
+    hs = [ep.sim_from_case(c, use_torch=False) for _ in range(3)]
+    v, w, ve = W.random_state(8, c)
+    for h in hs:
+        h.set_state(v, w, ve, 0)
+    full = hs[0].info().device_bytes
+    rows = 112 * c.n_tissue
+    b = ep.Batch(2, hbm_budget_bytes=2 * full - rows)
+    for h in hs[:2]:
+        b.add(h)
+    assert sum(h.info().device_bytes for h in hs[:2]) <= 2 * full - rows
+    b.step(2)
+    hs[2].step(2)
+    for h in hs[:2]:
+        assert np.abs(h.read(ep.EP_VE) - hs[2].read(ep.EP_VE)).max() <= 1e-5
+    b.close()
+    for h in hs:
+        h.close()
