@@ -121,6 +121,7 @@ struct ep_sim {
     cudaEvent_t ev[2] = {nullptr, nullptr};
     cudaGraphExec_t sweep_graph = nullptr;
     cudaGraphExec_t ie_graph = nullptr;   // implicit-diffusion sweeps
+    cudaGraphExec_t step_graph = nullptr; // explicit monodomain steps over the tabulated operator
     void *ie_x = nullptr, *ie_inv = nullptr;
     void *x2 = nullptr;          // second correction buffer of the FP32 elliptic solve (correction form)
     long long ie_seen = 0;                // implicit sweeps counted by earlier calls
@@ -380,7 +381,8 @@ bool needs_spectrum(const ep_sim *s)
     return s->p.solver == EP_SOLVER_CHEBYSHEV || (s->p.solver == EP_SOLVER_JACOBI && s->p.jacobi_omega < 0.0);
 }
 
-// The elliptic sweeps of a bidomain handle without a torso run over the tabulated operator.  Below kTabMin tissue
+// The elliptic sweeps of a bidomain handle without a torso, and the diffusion of a monodomain one, run over the
+// tabulated operator.  Below kTabMin tissue
 // voxels a sweep is a launch's latency on either path, and the handle stays as small as its fields.
 constexpr long long kTabMin = 4096;
 // Assembled rows for every tissue voxel (112 bytes a row in FP32) up to this many: the rows then stay in the L2
@@ -398,8 +400,10 @@ struct TabPlan {
 TabPlan tab_plan(const ep_sim *s)
 {
     TabPlan t;
-    if (s->lean || !s->have_params || s->d.model != EP_BI || !s->torso.empty() || s->n_tissue < kTabMin) return t;
-    const bool gs = s->p.solver == EP_SOLVER_GAUSS_SEIDEL;
+    if (s->lean || !s->have_params || !s->torso.empty() || s->n_tissue < kTabMin) return t;
+    const bool mono = s->d.model == EP_MONO;
+    if (mono && s->d.precision == EP_FP32 && s->n_tissue > kRowsOnly) return t;
+    const bool gs = !mono && s->p.solver == EP_SOLVER_GAUSS_SEIDEL;
     t.tab = 1;
     t.parts = gs ? 8 : 1;
     if (!gs && s->d.precision == EP_FP32 && s->n_tissue > kRowsOnly) {
@@ -825,14 +829,16 @@ ep_status setup_typed(ep_sim *s)
     }
     std::vector<int> rowq;   // outlives the copy below (the stream is synchronised at the end of set-up)
     int *d_bad = nullptr;    // a list that differs from the host's count
-    if (tp.tab) {   // the tabulated elliptic operator; the staged fibres' space serves once the records are built
+    if (tp.tab) {   // the tabulated operator; the staged fibres' space serves once the records are built
+        const bool mono = s->d.model == EP_MONO;
+        const double tT = mono ? s->p.sig_iT : sT, tL = mono ? s->p.sig_iL : sL;
         const double C = 1.0 / (8.0 * s->d.dx_mm * s->d.dx_mm);
         CK(cudaMemsetAsync(s->sweep_arrive, 0, kArriveBytes, st));
         if (tp.nbricks) {
             d_bad = (int *)tmp_fib;
             CK(cudaMemsetAsync(d_bad, 0, sizeof(int), st));
             CK(cudaMemcpyAsync(s->bricks, P.bricks.data(), sizeof(Brick) * P.bricks.size(), cudaMemcpyHostToDevice, st));
-            k_build_bricks<<<tp.nbricks, 256, 0, st>>>(nx, ny, nz, sT, sL - sT, C, s->rec, s->bricks, s->lists, d_bad);
+            k_build_bricks<<<tp.nbricks, 256, 0, st>>>(nx, ny, nz, tT, tL - tT, C, s->rec, s->bricks, s->lists, d_bad);
         } else {
             rowq.reserve((size_t)tp.nrows);
             if (tp.parts == 8) {   // sorted by colour
@@ -852,8 +858,9 @@ ep_status setup_typed(ep_sim *s)
             }
             int *d_rowq = (int *)tmp_fib;
             CK(cudaMemcpyAsync(d_rowq, rowq.data(), sizeof(int) * rowq.size(), cudaMemcpyHostToDevice, st));
-            k_build_rows<real><<<grid_for(tp.nrows, 128), 128, 0, st>>>(nx, ny, nz, sT, sL - sT, 0.0, C, s->rec, d_rowq,
-                                                                        tp.nrows, (real *)s->rows);
+            k_build_rows<real><<<grid_for(tp.nrows, 128), 128, 0, st>>>(nx, ny, nz, tT, tL - tT, 0.0, C, s->rec, d_rowq,
+                                                                        tp.nrows, mono ? (const real *)s->ie_inv : nullptr,
+                                                                        (real *)s->rows);
         }
         CK(cudaGetLastError());
     }
@@ -937,7 +944,7 @@ void drop_tables(ep_sim *s)
     s->dev_bytes -= s->tab_total;
     s->tab = s->nrows = s->nbricks = s->nsweep = 0;
     s->lean = true;
-    for (cudaGraphExec_t *g : {&s->sweep_graph, &s->ie_graph}) {
+    for (cudaGraphExec_t *g : {&s->sweep_graph, &s->ie_graph, &s->step_graph}) {
         if (*g) cudaGraphExecDestroy(*g);
         *g = nullptr;
     }
@@ -1080,7 +1087,7 @@ struct TabSweep {
     Inst<real> I;
     void operator()(cudaStream_t q, int parity) const
     {
-        if constexpr (sizeof(real) == 4 && !kGS<MODE>) {
+        if constexpr (sizeof(real) == 4 && !kGS<MODE> && MODE != M_IE) {
             if (I.nbricks) {
                 k_sweep<real, MODE, true><<<I.nsweep, kSweepNT<true>, kSweepSmem<MODE, true>, q>>>(I, parity);
                 return;
@@ -1350,6 +1357,52 @@ ep_status solve_elliptic(ep_sim *s, const Inst<real> &I, int &iters, double &rel
     return EP_OK;
 }
 
+// Explicit monodomain steps over the tabulated operator: two launches a step, replayed in graphs of kStepChunk steps.
+constexpr int kStepChunk = 32;   // even: a graph starts on an even step
+
+template <typename real>
+ep_status mono_steps(ep_sim *s, const Inst<real> &I, int n_steps)
+{
+    cudaStream_t st = s->stream;
+    const int gr = grid_for(s->n_tissue, kSweepThreads);
+    auto one = [&](int parity) {
+        k_react<real><<<gr, kSweepThreads, 0, st>>>(I, parity);
+        k_diffuse_rows<real><<<gr, kSweepThreads, 0, st>>>(I, parity);
+    };
+    const long long tick[2] = {s->step, s->step};
+    CK(cudaMemcpyAsync((char *)s->ctl + offsetof(Ctl, tick), tick, sizeof(tick), cudaMemcpyHostToDevice, st));
+    for (int it = 0; it < n_steps;) {
+        if (!s->noalloc_call && !(s->step & 1) && n_steps - it >= kStepChunk) {
+            if (!s->step_graph) {
+                cudaGraph_t g = nullptr;
+                CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
+                for (int i = 0; i < kStepChunk; ++i) one(i & 1);
+                cudaError_t e = cudaStreamEndCapture(st, &g);
+                if (e == cudaSuccess) {
+                    e = cudaGraphInstantiate(&s->step_graph, g, 0);
+                    cudaGraphDestroy(g);
+                }
+                if (e != cudaSuccess) {
+                    cudaGetLastError();
+                    s->step_graph = nullptr;
+                    return fail(s, EP_ECUDA, std::string("step graph: ") + cudaGetErrorString(e));
+                }
+            }
+            CK(cudaGraphLaunch(s->step_graph, st));
+            it += kStepChunk;
+            s->step += kStepChunk;
+        } else {
+            one((int)(s->step & 1));
+            CK(cudaGetLastError());
+            ++it;
+            ++s->step;
+        }
+    }
+    const long long step = s->step;   // the handle's counter follows
+    CK(cudaMemcpyAsync((char *)s->ctl + offsetof(Ctl, step), &step, sizeof(step), cudaMemcpyHostToDevice, st));
+    return EP_OK;
+}
+
 template <typename real>
 ep_status step_typed(ep_sim *s, int n_steps, ep_step_stats *stats)
 {
@@ -1368,7 +1421,22 @@ ep_status step_typed(ep_sim *s, int n_steps, ep_step_stats *stats)
         const int zero[3] = {0, 0, 0};
         CK(cudaMemcpyAsync((char *)s->ctl + offsetof(Ctl, nonfinite), zero, sizeof(zero), cudaMemcpyHostToDevice, st));
     }
-    for (int it = 0; it < n_steps; ++it) {
+    const bool mono_rows = I.tab && s->d.model == EP_MONO && !ie;
+    if (mono_rows) {
+        if (s->prof_on) CK(cudaEventRecord(s->pev[0], st));
+        const ep_status e = mono_steps<real>(s, I, n_steps);
+        if (e != EP_OK) return e;
+        if (s->prof_on) {
+            CK(cudaEventRecord(s->pev[1], st));
+            CK(cudaEventSynchronize(s->pev[1]));
+            float ms = 0.f;
+            CK(cudaEventElapsedTime(&ms, s->pev[0], s->pev[1]));
+            s->prof.other_ms += ms;
+            s->prof.other_launches += 2LL * n_steps;
+            s->prof.steps += n_steps;
+        }
+    }
+    for (int it = 0; it < n_steps && !mono_rows; ++it) {
         const double sweep_ms0 = s->prof.sweep_ms;
         if (s->prof_on) CK(cudaEventRecord(s->pev[0], st));
         if (ie) {
@@ -1381,7 +1449,8 @@ ep_status step_typed(ep_sim *s, int n_steps, ep_step_stats *stats)
             CK(cudaGetLastError());
             if (s->prof_on) CK(cudaEventRecord(s->pev[4], st));
             long long queued = 0;
-            ep_status e = run_sweeps(s, OneSweep<real, M_IE>{I}, &s->ie_graph, &queued);
+            ep_status e = I.tab && s->d.model == EP_MONO ? run_sweeps(s, TabSweep<real, M_IE>{I}, &s->ie_graph, &queued)
+                                                         : run_sweeps(s, OneSweep<real, M_IE>{I}, &s->ie_graph, &queued);
             if (e != EP_OK) return e;
             if (s->prof_on) {
                 CK(cudaEventRecord(s->pev[5], st));
@@ -2008,6 +2077,7 @@ void ep_destroy(ep_sim *s)
     if (s->ready && s->stream) cudaStreamSynchronize(s->stream);
     if (s->sweep_graph) cudaGraphExecDestroy(s->sweep_graph);
     if (s->ie_graph) cudaGraphExecDestroy(s->ie_graph);
+    if (s->step_graph) cudaGraphExecDestroy(s->step_graph);
     for (auto &e : s->ev)
         if (e) cudaEventDestroy(e);
     for (auto &e : s->pev)
@@ -2269,7 +2339,15 @@ ep_status build_batch_graph(ep_batch *b)
         for (int gi = 0; gi < ngroups; ++gi) CKB(cudaGraphConditionalHandleCreate(&hg[gi], body, 1, 0));
 
     CKB(cudaStreamBeginCaptureToGraph(st, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-    if (b->model == EP_MONO) k_stencil_batch<float, M_PAR_MONO><<<gs, kThreads, kSmemBytes<float, M_PAR_MONO>, st>>>(b->d_inst, b->d_seg);
+    if (b->model == EP_MONO) {
+        bool any = false, general = false;
+        for (int r = 0; r < b->ninst; ++r) (b->slot[b->order[r]]->tab ? any : general) = true;
+        if (general) k_stencil_batch<float, M_PAR_MONO><<<gs, kThreads, kSmemBytes<float, M_PAR_MONO>, st>>>(b->d_inst, b->d_seg);
+        if (any) {
+            k_mono_batch<float, false><<<nc, kSweepThreads, 0, st>>>(b->d_inst, b->d_chunk);
+            k_mono_batch<float, true><<<nc, kSweepThreads, 0, st>>>(b->d_inst, b->d_chunk);
+        }
+    }
     else k_stencil_batch<float, M_PAR_BI><<<gs, kThreads, kSmemBytes<float, M_PAR_BI>, st>>>(b->d_inst, b->d_seg);
     if (b->model == EP_BI) {
         k_stencil_batch<float, M_RHS><<<gs, kThreads, kSmemBytes<float, M_RHS>, st>>>(b->d_inst, b->d_seg);

@@ -111,6 +111,7 @@ struct alignas(16) Ctl {
     unsigned long long jarrive;
     long long ie_total;   // sweeps of the implicit parabolic solves, summed over steps
     double r0n2;          // correction form: ||r||^2 at the current cycle's start
+    long long tick[2];    // step of the explicit monodomain launches of either parity
 };
 
 struct Chunk {

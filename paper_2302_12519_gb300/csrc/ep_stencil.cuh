@@ -807,7 +807,7 @@ k_stencil_batch(const Inst<real> *insts, const BItem *items)
     StencilSmem<real, MODE> &sm = dyn_smem<StencilSmem<real, MODE>>();
     __shared__ Inst<real> sI;
     const BItem it = items[blockIdx.x];
-    if (kJac<MODE> && insts[it.inst].tab) return;   // this member's sweeps run over its tabulated operator
+    if ((kJac<MODE> || MODE == M_PAR_MONO) && insts[it.inst].tab) return;   // this member has a tabulated operator
     if (kJac<MODE> && cta_done(insts[it.inst].ctl, &sm.sflag)) return;
     const Inst<real> &I = stage_inst(insts + it.inst, sI);
     stencil_item<real, MODE>(I, it.item, it.item, it.nitems, nullptr, sm);

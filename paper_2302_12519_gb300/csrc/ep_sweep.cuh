@@ -72,6 +72,7 @@ __device__ __forceinline__ bool sweep_begin(const Inst<real> &I, int parity, Swe
         return false;
     }
     o.check = (o.sweep % I.check_every) == 0;
+    if (MODE == M_IE) return true;
     o.coef = I.coef_jac;
     o.cform = o.cheb = 0;
     o.cheb_w = real(1);
@@ -99,12 +100,14 @@ template <typename real, int MODE>
 __device__ __forceinline__ const real *sweep_src(const Inst<real> &I, int parity)
 {
     if (kGS<MODE>) return I.x0;
+    if (MODE == M_IE) return parity ? I.ie_x : I.v[(I.ctl->step & 1) ^ 1];
     return parity ? I.x1 : I.eform ? I.x2 : I.x0;
 }
 template <typename real, int MODE>
 __device__ __forceinline__ real *sweep_dst(const Inst<real> &I, int parity)
 {
     if (kGS<MODE>) return I.x0;
+    if (MODE == M_IE) return !parity ? I.ie_x : I.v[(I.ctl->step & 1) ^ 1];
     return !parity ? I.x1 : I.eform ? I.x2 : I.x0;
 }
 
@@ -171,8 +174,14 @@ __device__ __forceinline__ real sweep_row(const Inst<real> &I, const SweepOp<rea
     row_load(I, row, c);
     const int q = row_index(c[27]);
     const real u = src[q], b = I.b[q];
-    const real prev = kCheb<MODE> && o.cheb ? out[q] : real(0);
-    return sweep_out<real, MODE>(I, o, out, q, u, row_apply(I, c, src + q, u), b, c[26], prev);
+    if constexpr (MODE == M_IE) {   // r = f - (I + a L) x; x+ = x + r / (1 + a D), which the row holds (Eq. iejac1)
+        const real r = b - u - I.alpha_ie * row_apply(I, c, src + q, u);
+        out[q] = u + c[26] * r;
+        return r;
+    } else {
+        const real prev = kCheb<MODE> && o.cheb ? out[q] : real(0);
+        return sweep_out<real, MODE>(I, o, out, q, u, row_apply(I, c, src + q, u), b, c[26], prev);
+    }
 }
 
 struct BrickSmem {
@@ -320,7 +329,7 @@ __device__ __forceinline__ void sweep_cta(const Inst<real> &I, int parity, int c
     if constexpr (BRICKS) B = I.bricks[cta];
     if (!sweep_begin<real, MODE>(I, parity, o)) return;
     if (cta == 0 && threadIdx.x == 0) I.ctl->unit[parity ^ 1] = o.unit + 1;
-    const real *src = !kGS<MODE> && I.eform && o.sweep == 0 ? I.x0 : sweep_src<real, MODE>(I, parity);
+    const real *src = kJac<MODE> && !kGS<MODE> && I.eform && o.sweep == 0 ? I.x0 : sweep_src<real, MODE>(I, parity);
     real *out = sweep_dst<real, MODE>(I, parity);
     double acc = 0.0;
     if constexpr (BRICKS) {
@@ -361,7 +370,7 @@ __device__ __forceinline__ void sweep_cta(const Inst<real> &I, int parity, int c
         double s = 0;
         for (int i = threadIdx.x; i < parts * I.nsweep; i += NT) s += ((volatile double *)I.partials)[i];
         s = block_sum<NT>(s, sred);
-        if (threadIdx.x == 0) sweep_decide(I, o.sweep, !kGS<MODE> && I.eform, s);
+        if (threadIdx.x == 0) sweep_decide(I, o.sweep, kJac<MODE> && !kGS<MODE> && I.eform, s);
     }
 }
 
@@ -420,6 +429,82 @@ k_sweep_active(const Inst<real> *insts, const ActRec *act, int n, int parity)
     const ActRec r = act[sk];
     const Inst<real> &I = stage_inst(insts + r.inst, sI);
     sweep_cta<real, MODE, BRICKS>(I, parity, i - r.cum, reinterpret_cast<BrickSmem *>(ep_sweep_smem), sred, &sflag);
+}
+
+// Explicit monodomain step over the rows, two launches: the reaction at every tissue voxel (v* into b, the new w),
+// then the diffusion of v* (the new v, activation times, the non-finite flag).  The fused walk recomputes the
+// reaction of its halo and rebuilds the tensors; in FP64, where this GPU does two operations a clock and SM, that is
+// most of its time.  Launches of step parity p read the step from tick[p]; the second writes tick[p ^ 1].
+template <typename real>
+__device__ __forceinline__ void react_voxels(const Inst<real> &I, long long step, int first, int end, int stride)
+{
+    const int parity = (int)(step & 1);
+    const double tn = (double)step * I.dt_d;
+    const real *v = I.v[parity], *w = I.w[parity];
+    real *wn = I.w[parity ^ 1];
+    bool stim = false;
+    for (int s = 0; s < I.stim.n; ++s) stim = stim || (tn >= I.stim.box[s].t0 && tn < I.stim.box[s].t1);
+    for (int i = first; i < end; i += stride) {
+        const int q = I.idx[i];
+        int x = 0, y = 0, z = 0;   // used by active stimuli only
+        if (stim) {
+            x = q % I.nx;
+            y = (q / I.nx) % I.ny;
+            z = q / (I.nx * I.ny);
+        }
+        real vs, ws;
+        ms_step(I, tn, v[q], w[q], x, y, z, vs, ws);
+        I.b[q] = vs;
+        wn[q] = ws;
+    }
+}
+
+template <typename real>
+__device__ __forceinline__ void diffuse_rows(const Inst<real> &I, long long step, int first, int end, int stride)
+{
+    const int parity = (int)(step & 1);
+    const double tn = (double)step * I.dt_d;
+    const real *v = I.v[parity];
+    real *vn = I.v[parity ^ 1];
+    for (int i = first; i < end; i += stride) {
+        real c[kRowLen];
+        row_load(I, i, c);
+        const int q = row_index(c[27]);
+        const real u = I.b[q], vold = v[q];
+        const real vnew = u - I.coef_par * row_apply(I, c, I.b + q, u);
+        vn[q] = vnew;
+        if (vold < real(0.5) && vnew >= real(0.5) && I.tact[q] < real(0))
+            I.tact[q] = (real)(tn + I.dt_d * (0.5 - (double)vold) / ((double)vnew - (double)vold));
+        if (!isfinite((double)vnew)) atomicOr(&I.ctl->nonfinite, 1);
+    }
+}
+
+template <typename real>
+__global__ void __launch_bounds__(kSweepThreads) k_react(Inst<real> I, int parity)
+{
+    react_voxels(I, I.ctl->tick[parity], blockIdx.x * kSweepThreads + threadIdx.x, I.nrows, gridDim.x * kSweepThreads);
+}
+
+template <typename real>
+__global__ void __launch_bounds__(kSweepThreads, sizeof(real) == 8 ? 2 : EP_SWEEP_BLOCKS) k_diffuse_rows(Inst<real> I, int parity)
+{
+    const long long step = I.ctl->tick[parity];
+    diffuse_rows(I, step, blockIdx.x * kSweepThreads + threadIdx.x, I.nrows, gridDim.x * kSweepThreads);
+    if (blockIdx.x == 0 && threadIdx.x == 0) I.ctl->tick[parity ^ 1] = step + 1;
+}
+
+// Batched: a share of a member's rows per entry of the packed reduction-chunk list (members with rows only); the
+// step counter moves at the end of the batched step.
+template <typename real, bool DIFFUSE>
+__global__ void __launch_bounds__(kSweepThreads, EP_SWEEP_BLOCKS) k_mono_batch(const Inst<real> *insts, const BItem *items)
+{
+    __shared__ Inst<real> sI;
+    const BItem it = items[blockIdx.x];
+    const Inst<real> &I = stage_inst(insts + it.inst, sI);
+    if (!I.tab) return;
+    const int r0 = (int)((long long)I.nrows * it.item / it.nitems), r1 = (int)((long long)I.nrows * (it.item + 1) / it.nitems);
+    if (DIFFUSE) diffuse_rows(I, I.ctl->step, r0 + threadIdx.x, r1, kSweepThreads);
+    else react_voxels(I, I.ctl->step, r0 + threadIdx.x, r1, kSweepThreads);
 }
 
 // cheb_weight(k) for k < kChebTable - 1; the last entry is the weights' limit 2 e^-theta / rho.

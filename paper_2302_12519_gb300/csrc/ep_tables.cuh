@@ -47,7 +47,7 @@ __device__ __forceinline__ int row_index(double t) { return __double2loint(t); }
 // term (records with torso voxels); one thread a row.
 template <typename real>
 __global__ void k_build_rows(int nx, int ny, int nz, double sT, double dS, double so, double C, const float4 *rec,
-                             const int *rowq, long long nrows, real *rows)
+                             const int *rowq, long long nrows, const real *ie_inv, real *rows)
 {
     for (long long r = blockIdx.x * (long long)blockDim.x + threadIdx.x; r < nrows;
          r += (long long)gridDim.x * blockDim.x) {
@@ -102,7 +102,7 @@ __global__ void k_build_rows(int nx, int ny, int nz, double sT, double dS, doubl
         }
         auto put = [&](int e, real x) { rows[((long long)(e / 4) * nrows + r) * 4 + e % 4] = x; };
         for (int t = 0; t < 26; ++t) put(t, (real)(C * a[nb_cell(t)]));
-        put(26, (real)rec[q].w);
+        put(26, ie_inv ? ie_inv[q] : (real)rec[q].w);   // implicit diffusion: 1 / (1 + a D)
         put(27, row_tag(q, real(0)));
     }
 }

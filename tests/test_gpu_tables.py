@@ -63,6 +63,36 @@ def test_rows(kind, nx, ny, nz, solver, precision):
     _check(kind, 3, nx, ny, nz, solver, precision)
 
 
+# 37 steps from step 3 (one step to an even one, a graph of 32, four more), a stimulus that starts and ends inside
+@pytest.mark.parametrize("diffusion", [0, 1])
+@pytest.mark.parametrize("precision", [W.FP32, W.FP64])
+@pytest.mark.parametrize("kind,nx,ny,nz", [("full", 17, 16, 16), ("holes", 33, 23, 19), ("full", 4200, 1, 1)])
+def test_monodomain_rows(kind, nx, ny, nz, precision, diffusion):
+    c = W.random_case(7, nx, ny, nz, model=W.MONO, mask=_mask(kind, 7, nx, ny, nz),
+                      precision=precision).fibres_as_float32()
+    c.params.diffusion = diffusion
+    c.params.rel_tol = 1e-12 if precision == W.FP64 else 1e-6
+    c.stimuli = [W.Stimulus((1, 0, 0), (nx - 1, 5, 5), 0.4, 0.6, 0.5)]
+    v, w, _ = W.random_state(7, c)
+    s, ref = ep.sim_from_case(c), oracle.Sim(c)
+    s.set_state(v, w, None, 3)
+    ref.set_state(v, w, None, 3)
+    assert s.step(37).step == 40
+    for _ in range(37):
+        ref.step()
+    want = ref.state()
+    # 40 roundings of 2^-24 a step (FP64: of 2^-53, and the implicit solves' 1e-12), carried at most exp(37 dt 0.25 / tau_in)
+    grow = np.exp(37 * c.params.dt * 0.25 / c.params.tau_in)
+    tol = 37 * grow * (40 * 2.0 ** -24 + (1e-6 if diffusion else 0.0)) if precision == W.FP32 else \
+        37 * grow * (40 * 2.0 ** -53 + (1e-11 if diffusion else 0.0))
+    assert np.abs(s.read(ep.EP_V) - want["v"]).max() <= tol
+    assert np.abs(s.read(ep.EP_W) - want["w"]).max() <= tol
+    a, b = s.read(ep.EP_TACT), want["tact"]
+    assert np.array_equal(a >= 0, b >= 0) and np.abs(a - b).max() <= 100 * tol
+    s.close()
+    ref.close()
+
+
 @pytest.mark.parametrize("solver", [0, 1])
 @pytest.mark.parametrize("kind,nx,ny,nz", [("full", 91, 91, 89), ("holes", 120, 84, 78), ("holes", 31, 161, 151),
                                            ("blobs", 122, 107, 91)])
