@@ -276,11 +276,12 @@ __global__ void __launch_bounds__(kRedThreads) k_ie_react(Inst<real> I)
     const real *v = I.v[cur], *w = I.w[cur];
     real *vn = I.v[cur ^ 1], *wn = I.w[cur ^ 1];
     const long long nt = (long long)I.chunks[I.nchunk - 1].end;
+    const unsigned stim = active_stimuli(I, tn);
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nt; i += (long long)gridDim.x * blockDim.x) {
         const int q = I.idx[i];
         const int x = q % I.nx, y = (q / I.nx) % I.ny, z = q / (I.nx * I.ny);
         real vs, ws;
-        ms_step(I, tn, v[q], w[q], x, y, z, vs, ws);
+        ms_step(I, stim, v[q], w[q], x, y, z, vs, ws);
         I.b[q] = vs;
         vn[q] = vs;
         wn[q] = ws;

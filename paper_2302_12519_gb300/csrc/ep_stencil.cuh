@@ -88,6 +88,7 @@ struct Op {
     // (Chebyshev)
     int cform;
     int colour;        // eight-colour sweep: the colour this launch updates
+    unsigned stim;     // the stimuli active in this step
 };
 
 constexpr int kRestart = 1, kFold = 2, kPrev0 = 4;
@@ -183,8 +184,8 @@ __device__ __forceinline__ void plane_step(const Inst<real> &I, const Op<real> &
     C.e0 = C.e1 = C.e2 = real(0);
     if (MODE == M_PAR_MONO || MODE == M_PAR_BI || MODE == M_IE_RHS) {
         real vs, wn, vs2, wn2;
-        ms_step(I, o.tn, L.uLo, L.wLo, g.x, g.ylo, k, vs, wn);
-        ms_step(I, o.tn, L.uHi, L.wHi, g.x, g.ylo + 1, k, vs2, wn2);
+        ms_step(I, o.stim, L.uLo, L.wLo, g.x, g.ylo, k, vs, wn);
+        ms_step(I, o.stim, L.uHi, L.wHi, g.x, g.ylo + 1, k, vs2, wn2);
         if (MODE == M_IE_RHS) {   // the stencil acts on ve alone
             ulo = tlo ? L.veLo : real(0);
             uhi = thi ? L.veHi : real(0);
@@ -698,6 +699,8 @@ __device__ __forceinline__ void stencil_item(const Inst<real> &I, int seg_index,
         o.sT = I.sTi; o.dS = I.dSi; o.coef = I.coef_par;
         o.tn = (double)step * I.dt_d;
     }
+
+    o.stim = MODE == M_PAR_MONO || MODE == M_PAR_BI || MODE == M_IE_RHS ? active_stimuli(I, o.tn) : 0u;
 
     Lane g;
     g.lane = threadIdx.x & 31;

@@ -2,7 +2,7 @@
 //
 // Rows: a thread a row, 112 bytes of coefficients and 26 neighbours all in flight together, so a sweep is two rounds
 // of memory latency whatever the grid's shape.  Bound by latency while the rows stay in L2 (48^3 shell, 10.5 thousand
-// voxels: 3.2 us a sweep, the z-march 8.1; 128^3 shell, 199 thousand: 6.7 against 11.6), by their bytes above that.
+// voxels: 2.6 us a sweep, the z-march 8.1; 128^3 shell, 199 thousand: 5.7 against 11.6), by their bytes above that.
 // A colour pass of Gauss-Seidel reads its own eighth of the rows only: 6.9 us a pass on 1.10 million voxels, where
 // the march forms every flux for one voxel in eight, 32 us.
 // Bricks: 36 bytes of K and place a voxel (30 x 6 x 8 bricks share their lattices' faces), 16 of fields.  Bound by
@@ -34,6 +34,10 @@ __device__ __forceinline__ double load_if(bool on, const double *p, double other
     return x;
 }
 
+// c != 0 on the bits: an FP64 comparison would cost as much as the row's arithmetic on one neighbour.
+__device__ __forceinline__ bool nonzero(float c) { return c != 0.f; }
+__device__ __forceinline__ bool nonzero(double c) { return ((__double2hiint(c) & 0x7fffffff) | __double2loint(c)) != 0; }
+
 constexpr int kSweepThreads = 128;
 constexpr int kBrickThreads = 32 * kTileRows;
 
@@ -53,15 +57,16 @@ struct SweepOp {
 // launch leaves here on either reading.  The launch index comes from the slot of this launch's parity, which the
 // launch before wrote: counting arrivals on one address instead cost 10 ns a CTA, 17 us a sweep at 1600 CTAs.
 template <typename real, int MODE>
-__device__ __forceinline__ bool sweep_begin(const Inst<real> &I, int parity, SweepOp<real> &o)
+__device__ __forceinline__ bool sweep_begin(const Inst<real> &I, int phase, SweepOp<real> &o)
 {
+    const int parity = phase & 1;
     Ctl *ctl = I.ctl;
     const int4 c = *reinterpret_cast<const int4 *>(ctl);   // done, cycle0, unit[2]
     const int cycle0 = c.y;
     if (c.x) return false;
     o.unit = parity ? c.w : c.z;
     o.sweep = kGS<MODE> ? o.unit >> 3 : o.unit;
-    o.colour = o.unit & 7;
+    o.colour = phase;
     if (o.sweep >= I.max_iter) {
         if (threadIdx.x == 0) {
             ctl->noconv = 1;
@@ -93,13 +98,21 @@ __device__ __forceinline__ bool sweep_begin(const Inst<real> &I, int parity, Swe
     return true;
 }
 
+// A sweep may be launched while the one before it still runs (programmatic dependent launch): what changes between
+// sweeps is read after this, the tables before.  Nothing to wait for in an ordinary launch.
+__device__ __forceinline__ void after_previous_launch()
+{
+    cudaTriggerProgrammaticLaunchCompletion();
+    cudaGridDependencySynchronize();
+}
+
 // Iterate read and written by a launch of this parity (Chebyshev: the latter holds x_{k-1} until then).  A solve's
 // first launch has parity 0, so the parity is the sweep's own and the buffers are known without the control block,
 // but for the first sweep of a correction-form solve, which reads x0.
 template <typename real, int MODE>
-__device__ __forceinline__ const real *sweep_src(const Inst<real> &I, int parity)
+__device__ __forceinline__ const real *sweep_src(const Inst<real> &I, int parity, const SweepOp<real> &o)
 {
-    if (kGS<MODE>) return I.x0;
+    if (kGS<MODE> || (kJac<MODE> && I.eform && o.sweep == 0)) return I.x0;
     if (MODE == M_IE) return parity ? I.ie_x : I.v[(I.ctl->step & 1) ^ 1];
     return parity ? I.x1 : I.eform ? I.x2 : I.x0;
 }
@@ -155,7 +168,7 @@ __device__ __forceinline__ real row_apply(const Inst<real> &I, const real (&c)[k
     real nb[26];
 #pragma unroll
     for (int t = 0; t < 26; ++t) {
-        nb[t] = load_if(c[t] != real(0), s + (nb_dx(t) + I.nx * nb_dy(t) + plane * nb_dz(t)), u);
+        nb[t] = load_if(nonzero(c[t]), s + (nb_dx(t) + I.nx * nb_dy(t) + plane * nb_dz(t)), u);
     }
     real Lu0 = real(0), Lu1 = real(0);
 #pragma unroll
@@ -168,10 +181,8 @@ __device__ __forceinline__ real row_apply(const Inst<real> &I, const real (&c)[k
 
 template <typename real, int MODE>
 __device__ __forceinline__ real sweep_row(const Inst<real> &I, const SweepOp<real> &o, const real *src, real *out,
-                                          int row)
+                                          const real (&c)[kRowLen])
 {
-    real c[kRowLen];
-    row_load(I, row, c);
     const int q = row_index(c[27]);
     const real u = src[q], b = I.b[q];
     if constexpr (MODE == M_IE) {   // r = f - (I + a L) x; x+ = x + r / (1 + a D), which the row holds (Eq. iejac1)
@@ -320,30 +331,38 @@ __device__ __forceinline__ void sweep_brick(const Inst<float> &I, const SweepOp<
 // The work of CTA `cta` of the I.nsweep CTAs of a sweep, a brick or a share of the rows.  BRICKS: the handle's form,
 // and NT threads.
 template <typename real, int MODE, bool BRICKS>
-__device__ __forceinline__ void sweep_cta(const Inst<real> &I, int parity, int cta, BrickSmem *sm, double *sred,
+__device__ __forceinline__ void sweep_cta(const Inst<real> &I, int phase, int cta, BrickSmem *sm, double *sred,
                                           int *sflag)
 {
     constexpr int NT = BRICKS ? kBrickThreads : kSweepThreads;
+    const int parity = phase & 1;
     SweepOp<real> o;
-    Brick B{};
-    if constexpr (BRICKS) B = I.bricks[cta];
-    if (!sweep_begin<real, MODE>(I, parity, o)) return;
-    if (cta == 0 && threadIdx.x == 0) I.ctl->unit[parity ^ 1] = o.unit + 1;
-    const real *src = kJac<MODE> && !kGS<MODE> && I.eform && o.sweep == 0 ? I.x0 : sweep_src<real, MODE>(I, parity);
-    real *out = sweep_dst<real, MODE>(I, parity);
     double acc = 0.0;
     if constexpr (BRICKS) {
-        sweep_brick<MODE>(I, o, src, out, B, *sm, acc);
+        const Brick B = I.bricks[cta];
+        after_previous_launch();
+        if (!sweep_begin<real, MODE>(I, phase, o)) return;
+        sweep_brick<MODE>(I, o, sweep_src<real, MODE>(I, parity, o), sweep_dst<real, MODE>(I, parity), B, *sm, acc);
     } else {
-        const int r0 = kGS<MODE> ? I.row_colour[o.colour] : 0, r1 = kGS<MODE> ? I.row_colour[o.colour + 1] : I.nrows;
-        for (int i = r0 + cta * NT + threadIdx.x; i < r1; i += I.nsweep * NT) {
-            const real r = sweep_row<real, MODE>(I, o, src, out, i);
+        const int r0 = kGS<MODE> ? I.row_colour[phase] : 0, r1 = kGS<MODE> ? I.row_colour[phase + 1] : I.nrows;
+        int i = r0 + cta * NT + threadIdx.x;
+        real c[kRowLen];
+        if (i < r1) row_load(I, i, c);   // constants: read while the sweep before this one ends
+        after_previous_launch();
+        if (!sweep_begin<real, MODE>(I, phase, o)) return;
+        const real *src = sweep_src<real, MODE>(I, parity, o);
+        real *out = sweep_dst<real, MODE>(I, parity);
+        while (i < r1) {
+            const real r = sweep_row<real, MODE>(I, o, src, out, c);
             if (o.check) {
                 const float f = (float)r;
                 acc += (double)(f * f);
             }
+            i += I.nsweep * NT;
+            if (i < r1) row_load(I, i, c);
         }
     }
+    if (cta == 0 && threadIdx.x == 0) I.ctl->unit[parity ^ 1] = o.unit + 1;
     if (!o.check) return;
     // FP64 partial norms, summed in a fixed order by the CTA that arrives last.  CTAs count in groups, each counter
     // on its own line, and the last of a group counts the group.
@@ -375,7 +394,7 @@ __device__ __forceinline__ void sweep_cta(const Inst<real> &I, int parity, int c
 }
 
 // Bytes of dynamic shared memory and threads of a sweep CTA.
-template <int MODE, bool BRICKS>
+template <bool BRICKS>
 constexpr size_t kSweepSmem = BRICKS ? sizeof(BrickSmem) : 0;
 template <bool BRICKS>
 constexpr int kSweepNT = BRICKS ? kBrickThreads : kSweepThreads;
@@ -384,18 +403,18 @@ constexpr int kSweepMinBlocks = sizeof(real) == 8 ? 2 : BRICKS ? EP_BRICK_BLOCKS
 
 // Single instance.
 template <typename real, int MODE, bool BRICKS>
-__global__ void __launch_bounds__(kSweepNT<BRICKS>, kSweepMinBlocks<real, BRICKS>) k_sweep(Inst<real> I, int parity)
+__global__ void __launch_bounds__(kSweepNT<BRICKS>, kSweepMinBlocks<real, BRICKS>) k_sweep(Inst<real> I, int phase)
 {
     extern __shared__ __align__(16) unsigned char ep_sweep_smem[];
     __shared__ double sred[kSweepNT<BRICKS> / 32];
     __shared__ int sflag;
-    sweep_cta<real, MODE, BRICKS>(I, parity, blockIdx.x, reinterpret_cast<BrickSmem *>(ep_sweep_smem), sred, &sflag);
+    sweep_cta<real, MODE, BRICKS>(I, phase, blockIdx.x, reinterpret_cast<BrickSmem *>(ep_sweep_smem), sred, &sflag);
 }
 
 // Batched: the sweep CTAs of all members of a list with this form (the batch's trial sweeps).
 template <typename real, int MODE, bool BRICKS>
 __global__ void __launch_bounds__(kSweepNT<BRICKS>, kSweepMinBlocks<real, BRICKS>)
-k_sweep_batch(const Inst<real> *insts, const BItem *items, int parity)
+k_sweep_batch(const Inst<real> *insts, const BItem *items, int phase)
 {
     extern __shared__ __align__(16) unsigned char ep_sweep_smem[];
     __shared__ double sred[kSweepNT<BRICKS> / 32];
@@ -404,14 +423,14 @@ k_sweep_batch(const Inst<real> *insts, const BItem *items, int parity)
     const BItem it = items[blockIdx.x];
     const Inst<real> &I = stage_inst(insts + it.inst, sI);
     if ((I.nbricks > 0) != BRICKS) return;
-    sweep_cta<real, MODE, BRICKS>(I, parity, it.item, reinterpret_cast<BrickSmem *>(ep_sweep_smem), sred, &sflag);
+    sweep_cta<real, MODE, BRICKS>(I, phase, it.item, reinterpret_cast<BrickSmem *>(ep_sweep_smem), sred, &sflag);
 }
 
 // Batched: the unfinished members of a list (see k_stencil_active).  The descriptor is copied before the finished
 // flag is read, so a warp that leaves early has done its share.
 template <typename real, int MODE, bool BRICKS>
 __global__ void __launch_bounds__(kSweepNT<BRICKS>, kSweepMinBlocks<real, BRICKS>)
-k_sweep_active(const Inst<real> *insts, const ActRec *act, int n, int parity)
+k_sweep_active(const Inst<real> *insts, const ActRec *act, int n, int phase)
 {
     extern __shared__ __align__(16) unsigned char ep_sweep_smem[];
     __shared__ double sred[kSweepNT<BRICKS> / 32];
@@ -428,13 +447,14 @@ k_sweep_active(const Inst<real> *insts, const ActRec *act, int n, int parity)
     if (sk < 0) return;
     const ActRec r = act[sk];
     const Inst<real> &I = stage_inst(insts + r.inst, sI);
-    sweep_cta<real, MODE, BRICKS>(I, parity, i - r.cum, reinterpret_cast<BrickSmem *>(ep_sweep_smem), sred, &sflag);
+    sweep_cta<real, MODE, BRICKS>(I, phase, i - r.cum, reinterpret_cast<BrickSmem *>(ep_sweep_smem), sred, &sflag);
 }
 
 // Explicit monodomain step over the rows, two launches: the reaction at every tissue voxel (v* into b, the new w),
 // then the diffusion of v* (the new v, activation times, the non-finite flag).  The fused walk recomputes the
 // reaction of its halo and rebuilds the tensors; in FP64, where this GPU does two operations a clock and SM, that is
-// most of its time.  Launches of step parity p read the step from tick[p]; the second writes tick[p ^ 1].
+// most of its time: 121 us a step of the 32^3 slab against 10 here.  In FP32 small grids are bound by latency: 61 x 45
+// x 53, 19.5 us a step in the walk, 7.3 here (two launches).  Launches of step parity p read the step from tick[p]; the second writes tick[p ^ 1].
 template <typename real>
 __device__ __forceinline__ void react_voxels(const Inst<real> &I, long long step, int first, int end, int stride)
 {
@@ -442,8 +462,7 @@ __device__ __forceinline__ void react_voxels(const Inst<real> &I, long long step
     const double tn = (double)step * I.dt_d;
     const real *v = I.v[parity], *w = I.w[parity];
     real *wn = I.w[parity ^ 1];
-    bool stim = false;
-    for (int s = 0; s < I.stim.n; ++s) stim = stim || (tn >= I.stim.box[s].t0 && tn < I.stim.box[s].t1);
+    const unsigned stim = active_stimuli(I, tn);
     for (int i = first; i < end; i += stride) {
         const int q = I.idx[i];
         int x = 0, y = 0, z = 0;   // used by active stimuli only
@@ -453,7 +472,7 @@ __device__ __forceinline__ void react_voxels(const Inst<real> &I, long long step
             z = q / (I.nx * I.ny);
         }
         real vs, ws;
-        ms_step(I, tn, v[q], w[q], x, y, z, vs, ws);
+        ms_step(I, stim, v[q], w[q], x, y, z, vs, ws);
         I.b[q] = vs;
         wn[q] = ws;
     }
@@ -482,12 +501,14 @@ __device__ __forceinline__ void diffuse_rows(const Inst<real> &I, long long step
 template <typename real>
 __global__ void __launch_bounds__(kSweepThreads) k_react(Inst<real> I, int parity)
 {
+    after_previous_launch();
     react_voxels(I, I.ctl->tick[parity], blockIdx.x * kSweepThreads + threadIdx.x, I.nrows, gridDim.x * kSweepThreads);
 }
 
 template <typename real>
 __global__ void __launch_bounds__(kSweepThreads, sizeof(real) == 8 ? 2 : EP_SWEEP_BLOCKS) k_diffuse_rows(Inst<real> I, int parity)
 {
+    after_previous_launch();
     const long long step = I.ctl->tick[parity];
     diffuse_rows(I, step, blockIdx.x * kSweepThreads + threadIdx.x, I.nrows, gridDim.x * kSweepThreads);
     if (blockIdx.x == 0 && threadIdx.x == 0) I.ctl->tick[parity ^ 1] = step + 1;
