@@ -360,6 +360,21 @@ void build_bricks(const uint8_t *m, int nx, int ny, int nz, HostPlan &P)
     }
 }
 
+// Marks the clear items of a list over mask m.
+void mark_clear(std::vector<Seg> &segs, const uint8_t *m, int nx, int ny, int nz)
+{
+    for (Seg &g : segs) {
+        const int xa = std::max(0, g.x0 - 1), xb = std::min(nx, g.x0 + kTileX + 1);
+        const int ya = std::max(0, g.by * kTileY - 1), yb = std::min(ny, g.by * kTileY + kTileY + 1);
+        const int za = std::max(0, g.k0 - 1), zb = std::min(nz, g.k1 + 1);
+        bool clear = true;
+        for (int k = za; k < zb && clear; ++k)
+            for (int j = ya; j < yb && clear; ++j)
+                clear = !std::memchr(m + (size_t)nx * (j + (size_t)ny * k) + xa, 0, (size_t)(xb - xa));
+        if (clear) g.by |= kClearItem;
+    }
+}
+
 // ---------------------------------------------------------------------------
 // set-up: layout built on the host from the mask, records on the device
 // ---------------------------------------------------------------------------
@@ -407,6 +422,7 @@ TabPlan tab_plan(const ep_sim *s)
     t.tab = 1;
     t.parts = gs ? 8 : 1;
     if (!gs && s->d.precision == EP_FP32 && s->n_tissue > kRowsOnly) {
+        if (s->plan.n_vert > 2147483647LL) return TabPlan();   // the lists are indexed in 32 bits
         t.nbricks = (int)s->plan.bricks.size();
         t.nsweep = t.nbricks;
         return t;
@@ -696,6 +712,12 @@ ep_status setup_typed(ep_sim *s)
         s->nseg_e = tor ? (int)s->plan.segs_e.size() : s->nseg;
         s->nseg_far = tor ? partition_far(s->plan.segs_e, s->mask.data(), s->d.nx, s->d.ny, s->d.nz) : 0;
         s->zseg = kZLens[pick];
+        mark_clear(s->plan.segs, m, nx, ny, nz);
+        if (tor) {
+            std::vector<uint8_t> dom(s->mask);
+            for (long long q = 0; q < n; ++q) dom[q] |= s->torso[q];
+            mark_clear(s->plan.segs_e, dom.data(), nx, ny, nz);
+        }
     }
     const HostPlan &P = s->plan;
     const std::vector<int> &order = P.order;
@@ -2191,6 +2213,7 @@ ep_status relayout_segments(ep_sim *s, int zseg)
     if (zseg == s->zseg) return EP_OK;
     std::vector<Seg> segs = build_segments(s->mask.data(), s->d.nx, s->d.ny, s->d.nz, zseg);
     if ((long long)segs.size() > s->max_items) return fail(s, EP_EINVAL, "segment capacity exceeded");
+    mark_clear(segs, s->mask.data(), s->d.nx, s->d.ny, s->d.nz);
     CK(cudaMemcpyAsync(s->segs, segs.data(), sizeof(Seg) * segs.size(), cudaMemcpyHostToDevice, s->stream));
     CK(cudaStreamSynchronize(s->stream));
     s->nseg = (int)segs.size();

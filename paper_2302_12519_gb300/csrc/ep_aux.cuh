@@ -348,7 +348,7 @@ __global__ void __launch_bounds__(kRedThreads) k_ie_finish(Inst<real> I)
         const real v0 = vold[q];
         if (v0 < real(0.5) && v1 >= real(0.5) && I.tact[q] < real(0))
             I.tact[q] = (real)(tn + I.dt_d * (0.5 - (double)v0) / ((double)v1 - (double)v0));
-        if (!isfinite((double)v1)) atomicOr(&ctl->nonfinite, 1);
+        if (!isfinite(v1)) atomicOr(&ctl->nonfinite, 1);
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) ctl->ie_total += iters;
 }

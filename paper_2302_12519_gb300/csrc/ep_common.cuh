@@ -72,9 +72,11 @@ enum Model { MODEL_MONO = 0, MODEL_BI = 1 };
 
 // One stencil work item: voxel columns x in [x0, x0 + 30), rows
 // y in [kTileY by, kTileY by + kTileY), output planes [k0, k1).
+// kClearItem in by: every voxel of the item and of the voxels around it that lies in the grid is in the mask.
 struct Seg {
     int x0, by, k0, k1;
 };
+constexpr int kClearItem = 1 << 30;
 
 struct StimBox {
     int lo[3], hi[3];

@@ -494,7 +494,7 @@ __device__ __forceinline__ void diffuse_rows(const Inst<real> &I, long long step
         vn[q] = vnew;
         if (vold < real(0.5) && vnew >= real(0.5) && I.tact[q] < real(0))
             I.tact[q] = (real)(tn + I.dt_d * (0.5 - (double)vold) / ((double)vnew - (double)vold));
-        if (!isfinite((double)vnew)) atomicOr(&I.ctl->nonfinite, 1);
+        if (!isfinite(vnew)) atomicOr(&I.ctl->nonfinite, 1);
     }
 }
 

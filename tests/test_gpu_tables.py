@@ -1,6 +1,7 @@
-"""Sweeps over the tabulated operator (assembled rows and bricks) against the FP64 oracle: a few capped sweeps from a
-random state, so that every voxel's value depends on its own row or brick entries, at sizes around the edges of a
-row CTA (128 rows), a brick (30 x 6 x 8 voxels) and its lattice, ragged grids, grids with holes and thin ones."""
+"""The tabulated operator (assembled rows and bricks) and the walk over clear items against the FP64 oracle: a few
+capped sweeps or steps from a random state, so that every voxel's value depends on its own entries, at sizes around
+the edges of a row CTA (128 rows), a brick (30 x 6 x 8 voxels), a work item (30 x 7 x 32), ragged grids, grids with
+holes and thin ones."""
 import numpy as np
 import pytest
 
@@ -98,6 +99,32 @@ def test_monodomain_rows(kind, nx, ny, nz, precision, diffusion):
                                            ("blobs", 122, 107, 91)])
 def test_bricks(kind, nx, ny, nz, solver):
     _check(kind, 5, nx, ny, nz, solver, W.FP32)
+
+
+# above 720 000 voxels the FP32 monodomain walks; a block is made of clear items (31 x 151 x 155 and 91 x 91 x 89 end
+# inside a window, a row band and a plane block), one with a hole of clear and general ones
+@pytest.mark.parametrize("diffusion", [0, 1])
+@pytest.mark.parametrize("kind,nx,ny,nz", [("full", 91, 91, 89), ("full", 31, 151, 155), ("hole", 120, 85, 78)])
+def test_clear_items(kind, nx, ny, nz, diffusion):
+    mask = np.ones((nz, ny, nx), np.uint8)
+    if kind == "hole":
+        mask[40:44, 30:33, 50:60] = 0
+    c = W.random_case(9, nx, ny, nz, model=W.MONO, mask=mask).fibres_as_float32()
+    c.params.diffusion = diffusion
+    v, w, _ = W.random_state(9, c)
+    s, ref = ep.sim_from_case(c), oracle.Sim(c)
+    s.set_state(v, w, None, 0)
+    ref.set_state(v, w, None, 0)
+    s.step(3)
+    for _ in range(3):
+        ref.step()
+    want = ref.state()
+    grow = np.exp(3 * c.params.dt * 0.25 / c.params.tau_in)
+    tol = 3 * grow * (40 * 2.0 ** -24 + (1e-6 if diffusion else 0.0))   # as above
+    assert np.abs(s.read(ep.EP_V) - want["v"]).max() <= tol
+    assert np.abs(s.read(ep.EP_W) - want["w"]).max() <= tol
+    s.close()
+    ref.close()
 
 
 def test_tables_give_way_to_a_budget():
