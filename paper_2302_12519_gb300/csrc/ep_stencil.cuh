@@ -543,8 +543,10 @@ __device__ __forceinline__ void ring_plane(const Inst<real> &I, const Op<real> &
 // The walk over a clear item (kClearItem).  The mask there is the grid itself, so a lane's pair counts are constants
 // of its column and rows, and off the grid u and the records are 0: no flag or count is formed in the loop, and the
 // sums s and differences d of a column's two voxels carry the gradient (g_x: s - s_left over both planes, g_y:
-// d + d_left, g_z: the change of s + s_left) and, transposed, the scatter.  164 instructions a plane and warp of the
-// implicit sweep instead of 230; the 256^3 monodomain slab takes 217 us a step, 298 without.
+// d + d_left, g_z: the change of s + s_left) and, transposed, the scatter.  Bound by instruction issue and the shared
+// memory pipe (shuffles, records); 164 instructions a plane and warp of the implicit sweep instead of 230 before the
+// rows were shared.  256^3 monodomain slab: 298 us a step without, 217 with rings of each thread's own, 189 with the
+// shared one.
 template <typename real>
 struct ClearState {
     real X, Y, A;       // gradient sums of this plane
@@ -555,111 +557,192 @@ struct ClearState {
 template <typename real>
 struct ClearLane {
     real ax, ay, az, iso;   // 1 / pair counts of one plane (az: of two) and sigma_T x voxels of one plane
-    bool lo, hi;            // rows in the grid
+    bool lo;                // the lower row's voxel lies in the grid
 };
 
-template <typename real, int MODE, int S>
-__device__ __forceinline__ void clear_plane(const Inst<real> &I, const Op<real> &o, const Lane &g, const ClearLane<real> &c,
-                                            int k, int kbeg, int kend, int qhi, Ring<real, MODE> &R,
-                                            const ClearState<real> &P, ClearState<real> &C, real (*sF)[3][kWarps][32],
-                                            bool check, float &acc)
-{
-    constexpr int D = Ring<real, MODE>::D;
-    if (k + D - 1 <= kend) ring_issue<real, MODE>(o, R, (S + D - 1) % D, k + D - 1, c.lo, c.hi, g.qlo, qhi, g.plane);
-    cp_async_commit();
-    cp_async_wait<D - 1>();
-    Ld<real, MODE> L;
-    ring_read<real, MODE>(R, S % D, L, o.cheb != 0);
-    const bool kin = (unsigned)k < (unsigned)o.nz;
-    real lo = L.uLo, hi = L.uHi;
-    if (MODE == M_PAR_MONO) {
-        real wn, wn2;
-        ms_step(I, o.stim, L.uLo, L.wLo, g.x, g.ylo, k, lo, wn);
-        ms_step(I, o.stim, L.uHi, L.wHi, g.x, g.ylo + 1, k, hi, wn2);
-        C.e0 = lo; C.e1 = wn; C.e2 = L.uLo;
-        if (!c.lo || !kin) lo = real(0);
-        if (!c.hi || !kin) hi = real(0);
-    } else if (MODE == M_IE) {
-        C.e0 = L.bLo; C.e1 = L.iLo; C.e2 = real(0);
-    } else {
-        C.e0 = L.bLo; C.e1 = (real)L.rLo.w; C.e2 = L.iLo;
-    }
-    C.u = lo;
-    const real a0 = (real)L.rLo.x, a1 = (real)L.rLo.y, a2 = (real)L.rLo.z;
-    const real b0 = (real)L.rHi.x, b1 = (real)L.rHi.y, b2 = (real)L.rHi.z;
-    const real Z[6] = {a0 * a0 + b0 * b0, a1 * a1 + b1 * b1, a2 * a2 + b2 * b2,
-                       a0 * a1 + b0 * b1, a0 * a2 + b0 * b2, a1 * a2 + b1 * b2};
-#pragma unroll
-    for (int j = 0; j < 6; ++j) C.M[j] = Z[j] + __shfl_up_sync(kFull, Z[j], 1);
-    const real s = lo + hi, d = hi - lo;
-    const real sl = __shfl_up_sync(kFull, s, 1), dl = __shfl_up_sync(kFull, d, 1);
-    C.X = s - sl;
-    C.Y = d + dl;
-    C.A = s + sl;
-    real F0 = real(0), F1 = real(0), F2 = real(0);
-    if (k > kbeg) {
-        const bool both = kin && k > 0;   // planes of the vertex plane in the grid: two, or one at its ends
-        const real f = both ? real(0.5) : real(1), iso = both ? c.iso + c.iso : c.iso;
-        const real rx = c.ax * f, ry = c.ay * f, rz = both ? c.az : real(0);
-        const real hx = (P.X + C.X) * rx, hy = (P.Y + C.Y) * ry, hz = (C.A - P.A) * rz;
-        const real M0 = P.M[0] + C.M[0], M1 = P.M[1] + C.M[1], M2 = P.M[2] + C.M[2];
-        const real M3 = P.M[3] + C.M[3], M4 = P.M[4] + C.M[4], M5 = P.M[5] + C.M[5];
-        F0 = rx * (iso * hx + o.dS * (M0 * hx + M3 * hy + M4 * hz));
-        F1 = ry * (iso * hy + o.dS * (M3 * hx + M1 * hy + M5 * hz));
-        F2 = rz * (iso * hz + o.dS * (M4 * hx + M5 * hy + M2 * hz));
-    }
-    const int par = k & 1;
-    sF[par][0][g.wid][g.lane] = F0;
-    sF[par][1][g.wid][g.lane] = F1;
-    sF[par][2][g.wid][g.lane] = F2;
-    __syncthreads();
-    const int below = g.wid >= 1 ? g.wid - 1 : 0;   // the first warp writes nothing
-    const real p = sF[par][0][below][g.lane] + F0, q = sF[par][1][below][g.lane] - F1, r = sF[par][2][below][g.lane] + F2;
-    const real w = (p + q) + __shfl_down_sync(kFull, q - p, 1), z = r + __shfl_down_sync(kFull, r, 1);
-    C.S = w + z;
-    if (k > kbeg + 1 && g.out_lane)
-        emit<real, MODE>(I, o, g.qlo + (k - 1) * g.plane, P.u, o.C * (P.S + (w - z)), P.e0, P.e1, P.e2, check, acc);
-}
+// Staged planes of a clear item, shared by the CTA: warp w copies voxel row w of the item (its lower row), warp 0 also
+// the ninth; a barrier a plane, the one that publishes the fluxes, publishes the next plane too.  Half the copies and
+// the reactions of the ring a thread keeps for itself.
+template <typename real, int MODE>
+struct ClearRing {
+    static constexpr int D = sizeof(real) == 4 ? 4 : 2;
+    float4 rec[D][kWarps + 1][32];
+    real u[D][kWarps + 1][32];
+    real x[D][2][kWarps + 1][32];     // the copying thread's own: b and x_{k-1}, f and 1 / (1 + a D), or w
+    real vs[2][kWarps + 1][32];       // v* of the monodomain step
+};
 
 template <typename real, int MODE>
-__device__ __forceinline__ void clear_walk(const Inst<real> &I, const Op<real> &o, const Lane &g, bool lo_in, bool hi_in,
-                                           int qhi, int kbeg, int kend, Ring<real, MODE> &R, real (*sF)[3][kWarps][32],
-                                           bool check, float &acc)
-{
+struct ClearWalk {
+    static_assert(sizeof(ClearRing<real, MODE>) <= sizeof(Ring<real, MODE>), "it takes the ring's place");
+    static constexpr int D = ClearRing<real, MODE>::D;
+    const Inst<real> &I;
+    const Op<real> &o;
+    const Lane &g;
     ClearLane<real> c;
+    ClearRing<real, MODE> &R;
+    real (*sF)[3][kWarps][32];
+    int kbeg, kend, qx;    // qx: the ninth row's voxel (warp 0)
+    bool ninth;            // it lies in the grid
+    bool check;
+    float acc;
+
+    __device__ __forceinline__ void copy_row(int slot, int row, int q, bool own)
     {
-        const bool left = g.x >= 1 && g.x - 1 < I.nx, own = g.x >= 0 && g.x < I.nx;
-        const bool yl = g.ylo >= 0 && g.ylo < I.ny, yh = g.ylo + 1 < I.ny;   // the upper row is never below the grid
-        const int cols = (left ? 1 : 0) + (own ? 1 : 0), rows = (yl ? 1 : 0) + (yh ? 1 : 0);
-        c.ax = rcp_count<real>(real(cols == 2 ? rows : 0));
-        c.ay = rcp_count<real>(real(rows == 2 ? cols : 0));
-        c.az = rcp_count<real>(real(cols * rows));
-        c.iso = o.sT * real(cols * rows);
-        c.lo = lo_in;
-        c.hi = hi_in;
+        cp_async_n<16>(&R.rec[slot][row][g.lane], o.rec + q);
+        cp_async_n<sizeof(real)>(&R.u[slot][row][g.lane], o.src + q);
+        if (MODE == M_PAR_MONO) {
+            cp_async_n<sizeof(real)>(&R.x[slot][0][row][g.lane], o.w + q);
+        } else if (own) {
+            cp_async_n<sizeof(real)>(&R.x[slot][0][row][g.lane], o.b + q);
+            if (MODE == M_IE) cp_async_n<sizeof(real)>(&R.x[slot][1][row][g.lane], o.inv + q);
+            if (kCheb<MODE> && o.cheb) cp_async_n<sizeof(real)>(&R.x[slot][1][row][g.lane], o.out + q);
+        }
     }
-    ClearState<real> S0, S1;
-    S0.X = S0.Y = S0.A = S0.S = S0.u = S0.e0 = S0.e1 = S0.e2 = real(0);
-#pragma unroll
-    for (int j = 0; j < 6; ++j) S0.M[j] = real(0);
-    S1 = S0;
-    constexpr int D = Ring<real, MODE>::D;
-#pragma unroll
-    for (int j = 0; j < D - 1; ++j) {
-        if (kbeg + j <= kend) ring_issue<real, MODE>(o, R, j, kbeg + j, lo_in, hi_in, g.qlo, qhi, g.plane);
+    __device__ __forceinline__ void zero_row(int slot, int row)
+    {
+        R.rec[slot][row][g.lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+        R.u[slot][row][g.lane] = real(0);
+    }
+    // Plane k into its slot; rows and columns off the grid hold zeros from the start.
+    __device__ __forceinline__ void issue(int k, int slot)
+    {
+        if (k <= kend) {
+            if ((unsigned)k < (unsigned)o.nz) {
+                if (c.lo) copy_row(slot, g.wid, g.qlo + k * g.plane, true);
+                if (g.wid == 0 && ninth) copy_row(slot, kWarps, qx + k * g.plane, false);
+            } else {
+                zero_row(slot, g.wid);
+                if (g.wid == 0) zero_row(slot, kWarps);
+            }
+        }
         cp_async_commit();
     }
-    for (int k = kbeg;;) {
-        clear_plane<real, MODE, 0>(I, o, g, c, k, kbeg, kend, qhi, R, S1, S0, sF, check, acc);
-        if (++k > kend) break;
-        clear_plane<real, MODE, 1>(I, o, g, c, k, kbeg, kend, qhi, R, S0, S1, sF, check, acc);
-        if (++k > kend) break;
-        clear_plane<real, MODE, 2>(I, o, g, c, k, kbeg, kend, qhi, R, S1, S0, sF, check, acc);
-        if (++k > kend) break;
-        clear_plane<real, MODE, 3>(I, o, g, c, k, kbeg, kend, qhi, R, S0, S1, sF, check, acc);
-        if (++k > kend) break;
+    // The reaction of the rows this warp copied, of plane k (monodomain step).
+    __device__ __forceinline__ void react(int k, int slot, ClearState<real> &C)
+    {
+        const bool kin = (unsigned)k < (unsigned)o.nz;
+        const real v = R.u[slot][g.wid][g.lane];
+        ms_step(I, o.stim, v, R.x[slot][0][g.wid][g.lane], g.x, g.ylo, k, C.e0, C.e1);
+        C.e2 = v;
+        R.vs[k & 1][g.wid][g.lane] = c.lo && kin ? C.e0 : real(0);
+        if (g.wid == 0) {
+            real vs, wn;
+            ms_step(I, o.stim, R.u[slot][kWarps][g.lane], R.x[slot][0][kWarps][g.lane], g.x, g.ylo + kWarps, k, vs, wn);
+            R.vs[k & 1][kWarps][g.lane] = ninth && kin ? vs : real(0);
+        }
     }
-    cp_async_wait<0>();
+
+    // Plane k in slot S: P the state of plane k - 1, C receives that of plane k (its e0 .. e2 are in place), N takes the
+    // e0 .. e2 of plane k + 1 (N is P's storage, read before).
+    template <int S>
+    __device__ __forceinline__ void plane(int k, ClearState<real> &P, ClearState<real> &C)
+    {
+        const int row = g.wid, lane = g.lane, par = k & 1;
+        real lo, hi;
+        if (MODE == M_PAR_MONO) {
+            lo = R.vs[par][row][lane];
+            hi = R.vs[par][row + 1][lane];
+        } else {
+            lo = R.u[S][row][lane];
+            hi = R.u[S][row + 1][lane];
+        }
+        const float4 ra = R.rec[S][row][lane], rb = R.rec[S][row + 1][lane];
+        if (MODE == M_IE) {
+            C.e0 = R.x[S][0][row][lane]; C.e1 = R.x[S][1][row][lane];
+        } else if (MODE != M_PAR_MONO) {
+            C.e0 = R.x[S][0][row][lane]; C.e1 = (real)ra.w;
+            if (kCheb<MODE>) C.e2 = o.cheb ? R.x[S][1][row][lane] : real(0);
+        }
+        C.u = lo;
+        const real a0 = (real)ra.x, a1 = (real)ra.y, a2 = (real)ra.z;
+        const real b0 = (real)rb.x, b1 = (real)rb.y, b2 = (real)rb.z;
+        const real Z[6] = {a0 * a0 + b0 * b0, a1 * a1 + b1 * b1, a2 * a2 + b2 * b2,
+                           a0 * a1 + b0 * b1, a0 * a2 + b0 * b2, a1 * a2 + b1 * b2};
+#pragma unroll
+        for (int j = 0; j < 6; ++j) C.M[j] = Z[j] + __shfl_up_sync(kFull, Z[j], 1);
+        const real s = lo + hi, d = hi - lo;
+        const real sl = __shfl_up_sync(kFull, s, 1), dl = __shfl_up_sync(kFull, d, 1);
+        C.X = s - sl;
+        C.Y = d + dl;
+        C.A = s + sl;
+        real F0 = real(0), F1 = real(0), F2 = real(0);
+        if (k > kbeg) {
+            const bool both = k < o.nz && k > 0;   // planes of the vertex plane in the grid: two, or one at its ends
+            const real f = both ? real(0.5) : real(1), iso = both ? c.iso + c.iso : c.iso;
+            const real rx = c.ax * f, ry = c.ay * f, rz = both ? c.az : real(0);
+            const real hx = (P.X + C.X) * rx, hy = (P.Y + C.Y) * ry, hz = (C.A - P.A) * rz;
+            const real M0 = P.M[0] + C.M[0], M1 = P.M[1] + C.M[1], M2 = P.M[2] + C.M[2];
+            const real M3 = P.M[3] + C.M[3], M4 = P.M[4] + C.M[4], M5 = P.M[5] + C.M[5];
+            F0 = rx * (iso * hx + o.dS * (M0 * hx + M3 * hy + M4 * hz));
+            F1 = ry * (iso * hy + o.dS * (M3 * hx + M1 * hy + M5 * hz));
+            F2 = rz * (iso * hz + o.dS * (M4 * hx + M5 * hy + M2 * hz));
+        }
+        sF[par][0][row][lane] = F0;
+        sF[par][1][row][lane] = F1;
+        sF[par][2][row][lane] = F2;
+        const real pe0 = P.e0, pe1 = P.e1, pe2 = P.e2, pu = P.u, pS = P.S;
+        issue(k + D - 1, (S + D - 1) % D);   // into the slot of plane k - 1, which every warp has read
+        cp_async_wait<D - 2>();              // plane k + 1 of this thread's rows
+        if (MODE == M_PAR_MONO) react(k + 1, (S + 1) % D, P);
+        __syncthreads();
+        const int below = row >= 1 ? row - 1 : 0;   // the first warp writes nothing
+        const real p = sF[par][0][below][lane] + F0, q = sF[par][1][below][lane] - F1, r = sF[par][2][below][lane] + F2;
+        const real w = (p + q) + __shfl_down_sync(kFull, q - p, 1), z = r + __shfl_down_sync(kFull, r, 1);
+        C.S = w + z;
+        if (k > kbeg + 1 && g.out_lane)
+            emit<real, MODE>(I, o, g.qlo + (k - 1) * g.plane, pu, o.C * (pS + (w - z)), pe0, pe1, pe2, check, acc);
+    }
+
+    __device__ __forceinline__ void walk()
+    {
+        ClearState<real> S0, S1;
+        S0.X = S0.Y = S0.A = S0.S = S0.u = S0.e0 = S0.e1 = S0.e2 = real(0);
+#pragma unroll
+        for (int j = 0; j < 6; ++j) S0.M[j] = real(0);
+        S1 = S0;
+#pragma unroll
+        for (int j = 0; j < D; ++j) {   // what no copy ever fills
+            if (!c.lo) zero_row(j, g.wid);
+            if (g.wid == 0 && !ninth) zero_row(j, kWarps);
+        }
+#pragma unroll
+        for (int j = 0; j < D - 1; ++j) issue(kbeg + j, j);
+        cp_async_wait<D - 2>();
+        if (MODE == M_PAR_MONO) react(kbeg, 0, S0);
+        __syncthreads();
+        for (int k = kbeg;;) {
+            plane<0>(k, S1, S0);
+            if (++k > kend) break;
+            plane<1 % D>(k, S0, S1);
+            if (++k > kend) break;
+            plane<2 % D>(k, S1, S0);
+            if (++k > kend) break;
+            plane<3 % D>(k, S0, S1);
+            if (++k > kend) break;
+        }
+        cp_async_wait<0>();
+    }
+};
+
+template <typename real, int MODE>
+__device__ __forceinline__ void clear_walk(const Inst<real> &I, const Op<real> &o, const Lane &g, bool lo_in, int kbeg,
+                                           int kend, ClearRing<real, MODE> &R, real (*sF)[3][kWarps][32], bool check,
+                                           float &acc)
+{
+    const bool left = g.x >= 1 && g.x - 1 < I.nx, own = g.x >= 0 && g.x < I.nx;
+    const bool yl = g.ylo >= 0 && g.ylo < I.ny, yh = g.ylo + 1 < I.ny;   // the upper row is never below the grid
+    const int cols = (left ? 1 : 0) + (own ? 1 : 0), rows = (yl ? 1 : 0) + (yh ? 1 : 0);
+    ClearLane<real> c;
+    c.ax = rcp_count<real>(real(cols == 2 ? rows : 0));
+    c.ay = rcp_count<real>(real(rows == 2 ? cols : 0));
+    c.az = rcp_count<real>(real(cols * rows));
+    c.iso = o.sT * real(cols * rows);
+    c.lo = lo_in;
+    const int y8 = g.ylo + kWarps;   // used by warp 0
+    ClearWalk<real, MODE> W{I, o, g, c, R, sF, kbeg, kend, g.x + I.nx * y8, own && y8 >= 0 && y8 < I.ny, check, acc};
+    W.walk();
+    acc = W.acc;
 }
 
 // Decision of a checking sweep, by one thread: s is ||r||^2 of the sweep's input.
@@ -865,7 +948,7 @@ __device__ __forceinline__ void stencil_item(const Inst<real> &I, int seg_index,
         Ring<real, MODE> &R = sm.ring;
         const bool walked = kClearWalk<MODE> && clear;
         if constexpr (kClearWalk<MODE>)
-            if (clear) clear_walk<real, MODE>(I, o, g, lo_in, hi_in, qhi, kbeg, kend, R, sF, check, acc);
+            if (clear) clear_walk<real, MODE>(I, o, g, lo_in, kbeg, kend, reinterpret_cast<ClearRing<real, MODE> &>(R), sF, check, acc);
 #pragma unroll
         for (int j = 0; j < D - 1; ++j) {
             if (!walked && kbeg + j <= kend) ring_issue<real, MODE>(o, R, j, kbeg + j, lo_in, hi_in, g.qlo, qhi, g.plane);
