@@ -3,7 +3,7 @@
 // Rows: a thread a row, 112 bytes of coefficients and 26 neighbours all in flight together, so a sweep is two rounds
 // of memory latency whatever the grid's shape.  Bound by latency while the rows stay in L2 (48^3 shell, 10.5 thousand
 // voxels: 2.6 us a sweep, the z-march 8.1; 128^3 shell, 199 thousand: 5.7 against 11.6), by their bytes above that.
-// A colour pass of Gauss-Seidel reads its own eighth of the rows only: 6.9 us a pass on 1.10 million voxels, where
+// A colour pass of Gauss-Seidel reads its own eighth of the rows only: 6.4 us a pass on 1.10 million voxels, where
 // the march forms every flux for one voxel in eight, 32 us.
 // Bricks: 36 bytes of K and place a voxel (30 x 6 x 8 bricks share their lattices' faces), 16 of fields.  Bound by
 // memory latency: the lists alone stream in 32 us of the 256^3 heart's 55.6 (3.41 million voxels; the march 69.9, bound
@@ -398,12 +398,14 @@ template <bool BRICKS>
 constexpr size_t kSweepSmem = BRICKS ? sizeof(BrickSmem) : 0;
 template <bool BRICKS>
 constexpr int kSweepNT = BRICKS ? kBrickThreads : kSweepThreads;
-template <typename real, bool BRICKS>
-constexpr int kSweepMinBlocks = sizeof(real) == 8 ? 2 : BRICKS ? EP_BRICK_BLOCKS : EP_SWEEP_BLOCKS;
+// Resident CTAs asked for: 6 of rows (80 registers; 8 spill), 5 in a colour pass, whose gathers take more (176^3 heart:
+// 6.4 us a pass at 5, 6.9 at 6).
+template <typename real, bool BRICKS, int MODE = M_JAC>
+constexpr int kSweepMinBlocks = sizeof(real) == 8 ? 2 : BRICKS ? EP_BRICK_BLOCKS : kGS<MODE> ? 5 : EP_SWEEP_BLOCKS;
 
 // Single instance.
 template <typename real, int MODE, bool BRICKS>
-__global__ void __launch_bounds__(kSweepNT<BRICKS>, kSweepMinBlocks<real, BRICKS>) k_sweep(Inst<real> I, int phase)
+__global__ void __launch_bounds__(kSweepNT<BRICKS>, kSweepMinBlocks<real, BRICKS, MODE>) k_sweep(Inst<real> I, int phase)
 {
     extern __shared__ __align__(16) unsigned char ep_sweep_smem[];
     __shared__ double sred[kSweepNT<BRICKS> / 32];
