@@ -39,7 +39,7 @@ namespace {
 #endif
 constexpr int kZSeg = EP_ZSEG;     // default output planes per z-march segment
 constexpr int kZSegMin = 8;        // smallest segment length the batch autotuner tries
-constexpr int kSweepChunk = 64;    // sweeps per queued graph chunk (a multiple of 8: launches know their phase)
+constexpr int kSweepChunk[2] = {16, 64};   // launches of the queued graphs (multiples of 8: launches know their phase)
 constexpr int kSoloAllMembers = 8; // batch groups this small sweep every member in its own launches
 constexpr double kDivFactor = 1e16;
 constexpr int kNoAllocMaxPartials = 32768;   // ep_step_noalloc: stencil work items and reduction chunks
@@ -119,8 +119,18 @@ struct ep_sim {
     Ctl *ctl = nullptr;
     Ctl *ctl_host = nullptr;   // pinned, 2 slots
     cudaEvent_t ev[2] = {nullptr, nullptr};
-    cudaGraphExec_t sweep_graph = nullptr;
-    cudaGraphExec_t ie_graph = nullptr;   // implicit-diffusion sweeps
+    struct SweepGraphs {
+        cudaGraphExec_t g[2] = {nullptr, nullptr};   // kSweepChunk[i] launches
+        long long last = 0;                          // launches that the solve before needed (0: none yet)
+        void drop()
+        {
+            for (cudaGraphExec_t &e : g) {
+                if (e) cudaGraphExecDestroy(e);
+                e = nullptr;
+            }
+        }
+    };
+    SweepGraphs sweep_graph, ie_graph;    // of the elliptic solve and of the implicit diffusion
     cudaGraphExec_t step_graph = nullptr; // explicit monodomain steps over the tabulated operator
     void *ie_x = nullptr, *ie_inv = nullptr;
     void *x2 = nullptr;          // second correction buffer of the FP32 elliptic solve (correction form)
@@ -966,10 +976,10 @@ void drop_tables(ep_sim *s)
     s->dev_bytes -= s->tab_total;
     s->tab = s->nrows = s->nbricks = s->nsweep = 0;
     s->lean = true;
-    for (cudaGraphExec_t *g : {&s->sweep_graph, &s->ie_graph, &s->step_graph}) {
-        if (*g) cudaGraphExecDestroy(*g);
-        *g = nullptr;
-    }
+    s->sweep_graph.drop();
+    s->ie_graph.drop();
+    if (s->step_graph) cudaGraphExecDestroy(s->step_graph);
+    s->step_graph = nullptr;
 }
 
 // Descriptor of the elliptic sweeps: the work items and records of the domain
@@ -1154,14 +1164,14 @@ struct SplitSweep {
     }
 };
 
-// A CUDA graph of kSweepChunk sweeps of one solve.
+// A CUDA graph of n launches of one solve's sweeps.
 template <typename Sweep>
-ep_status build_sweep_graph(ep_sim *s, const Sweep &sweep, cudaGraphExec_t *out)
+ep_status build_sweep_graph(ep_sim *s, const Sweep &sweep, int n, cudaGraphExec_t *out)
 {
     if (*out) return EP_OK;
     cudaGraph_t g = nullptr;
     CK(cudaStreamBeginCapture(s->stream, cudaStreamCaptureModeThreadLocal));
-    for (int i = 0; i < kSweepChunk; ++i) sweep(s->stream, i & 7);
+    for (int i = 0; i < n; ++i) sweep(s->stream, i & 7);
     cudaError_t e = cudaStreamEndCapture(s->stream, &g);
     if (e != cudaSuccess) return fail(s, EP_ECUDA, std::string("sweep graph capture: ") + cudaGetErrorString(e));
     e = cudaGraphInstantiate(out, g, 0);
@@ -1173,39 +1183,50 @@ ep_status build_sweep_graph(ep_sim *s, const Sweep &sweep, cudaGraphExec_t *out)
     return EP_OK;
 }
 
-// Queues the sweeps of one solve in graph chunks with one chunk of look-ahead:
-// the host reads the control block one chunk behind, so the GPU never waits
-// for it.  At most max_iter sweeps (per_sweep launches each) do work; the
-// launch after them marks a capped solve done.  Returns the launches queued in
-// *queued_out.
+// Queues the sweeps of one solve in graphs of 64 launches and reads the control block one graph behind, so that the GPU
+// never waits for the host.  Around the number that the solve before needed the graphs have 16 launches, and from that
+// number on each graph's own flag is waited for: queued launches after the end return at once, but in 1.5 us each (a
+// solve of 11 sweeps under two graphs of 64 spent 175 us of its 950 us step on them).  At most max_iter sweeps
+// (per_sweep launches each) do work; the launch
+// after them marks a capped solve done.  Returns the launches queued in *queued_out.
 template <typename Sweep>
-ep_status run_sweeps(ep_sim *s, const Sweep &sweep, cudaGraphExec_t *graph, long long *queued_out, int per_sweep = 1)
+ep_status run_sweeps(ep_sim *s, const Sweep &sweep, ep_sim::SweepGraphs *graphs, long long *queued_out, int per_sweep = 1)
 {
     cudaStream_t st = s->stream;
-    if (!s->noalloc_call) {
-        ep_status gs = build_sweep_graph(s, sweep, graph);
-        if (gs != EP_OK) return gs;
-    }
     const long long limit = (long long)per_sweep * s->p.max_iter + 1;
     long long queued = 0;
-    for (int c = 0;; ++c) {
-        if (!s->noalloc_call && queued + kSweepChunk <= limit) {
-            CK(cudaGraphLaunch(*graph, st));
-            queued += kSweepChunk;
+    auto queue = [&](int size) -> ep_status {   // one graph of kSweepChunk[size] launches, or what is left to the limit
+        const int n = kSweepChunk[size];
+        if (!s->noalloc_call && queued + n <= limit) {
+            const ep_status gs = build_sweep_graph(s, sweep, n, &graphs->g[size]);
+            if (gs != EP_OK) return gs;
+            CK(cudaGraphLaunch(graphs->g[size], st));
+            queued += n;
         } else {
-            const long long stop = std::min(limit, queued + (long long)kSweepChunk);
+            const long long stop = std::min(limit, queued + (long long)n);
             for (; queued < stop; ++queued) sweep(st, (int)(queued & 7));
             CK(cudaGetLastError());
         }
+        return EP_OK;
+    };
+    const long long last = graphs->last;
+    for (int c = 0;; ++c) {
+        if (queued < limit) {
+            const bool near_end = queued + kSweepChunk[1] > last && queued < last + kSweepChunk[1];
+            const ep_status qs = queue((last > 0 ? near_end : c < 4) ? 0 : 1);
+            if (qs != EP_OK) return qs;
+        }
         CK(cudaMemcpyAsync(&s->ctl_host[c & 1], s->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, st));
         CK(cudaEventRecord(s->ev[c & 1], st));
-        if (queued >= limit) {   // everything up to the cap is queued; the last launch marks done
-            CK(cudaEventSynchronize(s->ev[c & 1]));
+        int look = c - 1;        // one graph behind keeps the GPU busy while the host checks
+        if (queued >= limit || (last > 0 && queued >= last && queued < last + kSweepChunk[1]))
+            look = c;            // everything is queued, or what should do
+        if (look < 0) continue;
+        CK(cudaEventSynchronize(s->ev[look & 1]));
+        const Ctl &h = s->ctl_host[look & 1];
+        if (h.done || queued >= limit) {   // at the limit the last launch marks done
+            graphs->last = (long long)per_sweep * h.iters;
             break;
-        }
-        if (c >= 1) {            // one chunk of look-ahead keeps the GPU busy while the host checks
-            CK(cudaEventSynchronize(s->ev[(c - 1) & 1]));
-            if (s->ctl_host[(c - 1) & 1].done) break;
         }
     }
     *queued_out = queued;
@@ -2123,8 +2144,8 @@ void ep_destroy(ep_sim *s)
 {
     if (!s) return;
     if (s->ready && s->stream) cudaStreamSynchronize(s->stream);
-    if (s->sweep_graph) cudaGraphExecDestroy(s->sweep_graph);
-    if (s->ie_graph) cudaGraphExecDestroy(s->ie_graph);
+    s->sweep_graph.drop();
+    s->ie_graph.drop();
     if (s->step_graph) cudaGraphExecDestroy(s->step_graph);
     for (auto &e : s->ev)
         if (e) cudaEventDestroy(e);
@@ -2218,14 +2239,8 @@ ep_status relayout_segments(ep_sim *s, int zseg)
     CK(cudaStreamSynchronize(s->stream));
     s->nseg = (int)segs.size();
     s->zseg = zseg;
-    if (s->sweep_graph) {
-        cudaGraphExecDestroy(s->sweep_graph);
-        s->sweep_graph = nullptr;
-    }
-    if (s->ie_graph) {
-        cudaGraphExecDestroy(s->ie_graph);
-        s->ie_graph = nullptr;
-    }
+    s->sweep_graph.drop();
+    s->ie_graph.drop();
     return EP_OK;
 }
 
