@@ -66,6 +66,9 @@ struct HostPlan {
     std::vector<Seg> segs_e, segs_e_z[4];   // the same over the domain (torso handles only)
     std::vector<Brick> bricks;          // tabulated operator: bricks over the tissue, and their lists' totals
     long long n_vert = 0, n_part = 0, n_bound = 0;
+    std::vector<uint8_t> walked;        // torso handles: voxels with nothing but torso around them, their number
+    std::vector<Seg> walk;              // and the work items over them
+    long long n_walked = 0;
 };
 
 constexpr int kZLens[4] = {8, 16, 24, 32};
@@ -145,6 +148,9 @@ struct ep_sim {
     Brick *bricks = nullptr;
     BrickLists lists{};
     unsigned *sweep_arrive = nullptr;
+    Seg *walk = nullptr;
+    void *walk_dinv = nullptr;
+    int nwalk = 0;
     bool noalloc_call = false;   // inside ep_step_noalloc: scratch is the static array, no graph
     // device-time accounting (ep_profile_enable)
     bool prof_on = false;
@@ -370,6 +376,38 @@ void build_bricks(const uint8_t *m, int nx, int ny, int nz, HostPlan &P)
     }
 }
 
+// Torso handles: the torso voxels whose neighbours in the grid, all 26, are torso too, and the work items over them
+// (the longest that still make two waves of CTAs, as for the other items).
+void plan_walk(const uint8_t *torso, const uint8_t *heart, int nx, int ny, int nz, HostPlan &P)
+{
+    const size_t n = (size_t)nx * ny * nz, plane = (size_t)nx * ny;
+    std::vector<uint8_t> a(n), b(n);
+    for (size_t q = 0; q < n; ++q) a[q] = torso[q] & (heart[q] ^ 1);
+    for (size_t r = 0; r < n; r += nx)   // along x, y and z in turn; off the grid counts as torso
+        for (int i = 0; i < nx; ++i) b[r + i] = a[r + i] & (i ? a[r + i - 1] : 1) & (i + 1 < nx ? a[r + i + 1] : 1);
+    for (int k = 0; k < nz; ++k)
+        for (int j = 0; j < ny; ++j) {
+            const size_t r = nx * (j + (size_t)ny * k);
+            const uint8_t *lo = &b[j ? r - nx : r], *hi = &b[j + 1 < ny ? r + nx : r];
+            for (int i = 0; i < nx; ++i) a[r + i] = b[r + i] & lo[i] & hi[i];
+        }
+    P.n_walked = 0;
+    for (int k = 0; k < nz; ++k) {
+        const uint8_t *lo = &a[plane * (k ? k - 1 : k)], *hi = &a[plane * (k + 1 < nz ? k + 1 : k)], *c = &a[plane * k];
+        unsigned s = 0;
+        for (size_t i = 0; i < plane; ++i) {
+            b[plane * k + i] = c[i] & lo[i] & hi[i];
+            s += b[plane * k + i];
+        }
+        P.n_walked += s;
+    }
+    for (int z : {32, 16, 8}) {
+        P.walk = build_segments(b.data(), nx, ny, nz, z);
+        if (P.walk.size() >= 2u * 152u * 4u) break;
+    }
+    P.walked = std::move(b);
+}
+
 // Marks the clear items of a list over mask m.
 void mark_clear(std::vector<Seg> &segs, const uint8_t *m, int nx, int ny, int nz)
 {
@@ -418,14 +456,22 @@ constexpr int kMaxRowCtas = 4096;
 constexpr size_t kArriveBytes = sizeof(unsigned) * kArriveStride * (kArriveGroups + 1);
 
 struct TabPlan {
-    int tab = 0, nbricks = 0, nsweep = 0, parts = 1;
+    int tab = 0, nbricks = 0, nsweep = 0, parts = 1, nwalk = 0;
     long long nrows = 0;
 };
 
 TabPlan tab_plan(const ep_sim *s)
 {
     TabPlan t;
-    if (s->lean || !s->have_params || !s->torso.empty() || s->n_tissue < kTabMin) return t;
+    if (s->lean || !s->have_params || s->n_tissue < kTabMin) return t;
+    if (!s->torso.empty()) {   // FP32: rows near the tissue, the walk through the torso away from it
+        if (s->d.precision != EP_FP32 || s->d.model != EP_BI || s->p.solver == EP_SOLVER_GAUSS_SEIDEL) return t;
+        t.tab = 1;
+        t.nrows = s->n_domain - s->plan.n_walked;
+        t.nwalk = (int)s->plan.walk.size();
+        t.nsweep = t.nwalk + (int)std::min<long long>(kMaxRowCtas, (t.nrows + kThreads - 1) / kThreads);
+        return t;
+    }
     const bool mono = s->d.model == EP_MONO;
     if (mono && s->d.precision == EP_FP32 && s->n_tissue > kRowsOnly) return t;
     const bool gs = !mono && s->p.solver == EP_SOLVER_GAUSS_SEIDEL;
@@ -454,6 +500,7 @@ size_t tab_bytes(const ep_sim *s, const TabPlan &t, size_t rb)
             abytes(sizeof(float2) * (size_t)s->n_tissue) + abytes((size_t)P.n_bound);
     else
         b = abytes(rb * kRowLen * (size_t)t.nrows);
+    if (!s->torso.empty()) b += abytes(sizeof(Seg) * (size_t)t.nwalk) + abytes(rb * (size_t)s->n);
     return b + abytes(rb * kChebTable) + abytes(kArriveBytes);
 }
 
@@ -587,6 +634,7 @@ ep_status plan_layout(ep_sim *s)
     s->nseg_e = torso ? (int)P.segs_e.size() : s->nseg;
     if (s->d.model == EP_BI && !torso && s->d.precision == EP_FP32 && s->n_tissue > kRowsOnly)
         build_bricks(mh, nx, ny, nz, P);
+    if (torso && s->d.precision == EP_FP32 && s->n_tissue >= kTabMin) plan_walk(s->torso.data(), mh, nx, ny, nz, P);
     // capacity of the item buffers: the largest item count of the z-lengths set-up and the batch use
     s->max_items = std::max<long long>(most, std::max(s->nseg, s->nseg_e));
     footprint(s, s->d.precision == EP_FP64 ? sizeof(double) : sizeof(float), &s->fp_resident, &s->fp_peak);
@@ -799,6 +847,12 @@ ep_status setup_typed(ep_sim *s)
             s->rows = dalloc(s, rb * kRowLen * (size_t)tp.nrows);
             got = got && s->rows;
         }
+        s->nwalk = tp.nwalk;
+        if (torso) {
+            take(s->walk, (size_t)tp.nwalk);
+            s->walk_dinv = dalloc(s, rb * (size_t)n);
+            got = got && s->walk_dinv;
+        }
         s->cheb_table = dalloc(s, rb * kChebTable);
         s->sweep_arrive = (unsigned *)dalloc(s, kArriveBytes);
         if (!got || !s->cheb_table || !s->sweep_arrive) return fail(s, EP_ENOMEM, "device allocation failed");
@@ -886,13 +940,19 @@ ep_status setup_typed(ep_sim *s)
                 s->row_colour[8] = (int)rowq.size();
             } else {
                 for (int q = 0; q < (int)n; ++q)
-                    if (m[q]) rowq.push_back(q);
+                    if (torso ? (m[q] || s->torso[q]) && !P.walked[q] : m[q] != 0) rowq.push_back(q);
             }
             int *d_rowq = (int *)tmp_fib;
             CK(cudaMemcpyAsync(d_rowq, rowq.data(), sizeof(int) * rowq.size(), cudaMemcpyHostToDevice, st));
-            k_build_rows<real><<<grid_for(tp.nrows, 128), 128, 0, st>>>(nx, ny, nz, tT, tL - tT, 0.0, C, s->rec, d_rowq,
+            k_build_rows<real><<<grid_for(tp.nrows, 128), 128, 0, st>>>(nx, ny, nz, tT, tL - tT, torso ? s->sig_o : 0.0, C, s->rec_e, d_rowq,
                                                                         tp.nrows, mono ? (const real *)s->ie_inv : nullptr,
                                                                         (real *)s->rows);
+            if (torso) {   // the masks staged for the records are read: their space takes the walked voxels
+                CK(cudaMemcpyAsync(tmp_torso, P.walked.data(), n, cudaMemcpyHostToDevice, st));
+                CK(cudaMemcpyAsync(s->walk, P.walk.data(), sizeof(Seg) * P.walk.size(), cudaMemcpyHostToDevice, st));
+                k_build_walk<real><<<grid_for(n, 256), 256, 0, st>>>(n, (const uint8_t *)tmp_torso, s->rec_e,
+                                                                     (real *)s->walk_dinv);
+            }
         }
         CK(cudaGetLastError());
     }
@@ -949,6 +1009,8 @@ ep_status setup_typed(ep_sim *s)
     s->plan.segs = std::vector<Seg>();
     s->plan.segs_e = std::vector<Seg>();
     s->plan.bricks = std::vector<Brick>();
+    s->plan.walked = std::vector<uint8_t>();
+    s->plan.walk = std::vector<Seg>();
     for (auto &v : s->plan.segs_z) v = std::vector<Seg>();
     for (auto &v : s->plan.segs_e_z) v = std::vector<Seg>();
     CK(cudaMallocHost((void **)&s->ctl_host, 2 * sizeof(Ctl)));
@@ -966,7 +1028,7 @@ void drop_tables(ep_sim *s)
     if (s->stream) cudaStreamSynchronize(s->stream);
     for (void *t : {(void *)s->rows, s->cheb_table, (void *)s->sweep_arrive, (void *)s->bricks, (void *)s->lists.k4,
                     (void *)s->lists.k2, (void *)s->lists.vloc, (void *)s->lists.vpair, (void *)s->lists.out,
-                    (void *)s->lists.oflag}) {
+                    (void *)s->lists.oflag, (void *)s->walk, s->walk_dinv}) {
         auto it = t ? std::find(s->allocs.begin(), s->allocs.end(), t) : s->allocs.end();
         if (it == s->allocs.end()) continue;
         if (s->d.dev_alloc && s->d.dev_free) s->d.dev_free(t, s->d.alloc_ctx);
@@ -974,7 +1036,7 @@ void drop_tables(ep_sim *s)
         s->allocs.erase(it);
     }
     s->dev_bytes -= s->tab_total;
-    s->tab = s->nrows = s->nbricks = s->nsweep = 0;
+    s->tab = s->nrows = s->nbricks = s->nsweep = s->nwalk = 0;
     s->lean = true;
     s->sweep_graph.drop();
     s->ie_graph.drop();
@@ -1066,6 +1128,10 @@ Inst<real> make_inst(const ep_sim *s)
     I.lists = s->lists;
     I.cheb_table = (const real *)s->cheb_table;
     I.sweep_arrive = s->sweep_arrive;
+    I.walk = s->walk;
+    I.walk_dinv = (const real *)s->walk_dinv;
+    I.nwalk = s->nwalk;
+    I.pad8 = 0;
     for (int i = 0; i < 9; ++i) I.row_colour[i] = s->row_colour[i];
     I.torso = s->torso.empty() ? 0 : 1;
     I.pad4 = 0;
@@ -1147,11 +1213,15 @@ struct TabSweep {
     {
         if constexpr (sizeof(real) == 4 && !kGS<MODE> && MODE != M_IE) {
             if (I.nbricks) {
-                launch(k_sweep<real, MODE, true>, I.nsweep, kSweepNT<true>, kSweepSmem<true>, q, I, phase);
+                launch(k_sweep<real, MODE, FORM_BRICKS>, I.nsweep, kSweepNT<FORM_BRICKS>, kSweepSmem<FORM_BRICKS>, q, I, phase);
+                return;
+            }
+            if (I.torso) {
+                launch(k_sweep<real, MODE, FORM_TORSO>, I.nsweep, kSweepNT<FORM_TORSO>, kSweepSmem<FORM_TORSO>, q, I, phase);
                 return;
             }
         }
-        launch(k_sweep<real, MODE, false>, I.nsweep, kSweepNT<false>, 0, q, I, phase);
+        launch(k_sweep<real, MODE, FORM_ROWS>, I.nsweep, kSweepNT<FORM_ROWS>, 0, q, I, phase);
     }
 };
 template <typename real, int MODE_FAR, int MODE_NEAR>
@@ -1283,14 +1353,14 @@ ep_status configure_kernels(ep_sim *s)
     if (e == cudaSuccess)
         e = allow_stencil_batch(std::integer_sequence<int, M_PAR_MONO, M_PAR_BI, M_RHS, M_JAC, M_JAC_CHEB>{});
     auto bricks = [&](auto *k) {
-        if (e == cudaSuccess) e = allow_smem(k, kSweepSmem<true>);
+        if (e == cudaSuccess) e = allow_smem(k, kSweepSmem<FORM_BRICKS>);
     };
-    bricks(k_sweep<float, M_JAC, true>);
-    bricks(k_sweep<float, M_JAC_CHEB, true>);
-    bricks(k_sweep_batch<float, M_JAC, true>);
-    bricks(k_sweep_batch<float, M_JAC_CHEB, true>);
-    bricks(k_sweep_active<float, M_JAC, true>);
-    bricks(k_sweep_active<float, M_JAC_CHEB, true>);
+    bricks(k_sweep<float, M_JAC, FORM_BRICKS>);
+    bricks(k_sweep<float, M_JAC_CHEB, FORM_BRICKS>);
+    bricks(k_sweep_batch<float, M_JAC, FORM_BRICKS>);
+    bricks(k_sweep_batch<float, M_JAC_CHEB, FORM_BRICKS>);
+    bricks(k_sweep_active<float, M_JAC, FORM_BRICKS>);
+    bricks(k_sweep_active<float, M_JAC_CHEB, FORM_BRICKS>);
     if (e == cudaSuccess) e = allow_stencil_active(std::integer_sequence<int, M_JAC, M_JAC_CHEB>{});
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -2476,7 +2546,7 @@ ep_status build_batch_graph(ep_batch *b)
             }
             // the other members: packed sweeps over the unfinished ones
             auto packed_sweep = [&](auto bricks, cudaStream_t a, int i) {
-                constexpr bool B = decltype(bricks)::value;
+                constexpr int B = decltype(bricks)::value ? FORM_BRICKS : FORM_ROWS;
                 const int gp = (int)gr.packed_tab[B];
                 if (gr.cheb) k_sweep_active<float, M_JAC_CHEB, B><<<gp, kSweepNT<B>, kSweepSmem<B>, a>>>(gi_inst, act_tab[B], gn, i & 1);
                 else k_sweep_active<float, M_JAC, B><<<gp, kSweepNT<B>, kSweepSmem<B>, a>>>(gi_inst, act_tab[B], gn, i & 1);
@@ -2746,7 +2816,7 @@ ep_status ep_batch_autotune(ep_batch *b, int trial_sweeps)
                     parity ^= 1;
                     const int gw = (int)gr.nsw;   // every member's items on the general path, the tabulated ones skipped there
                     auto tables = [&](auto bricks) {
-                        constexpr bool B = decltype(bricks)::value;
+                        constexpr int B = decltype(bricks)::value ? FORM_BRICKS : FORM_ROWS;
                         if (gr.cheb) k_sweep_batch<float, M_JAC_CHEB, B><<<gw, kSweepNT<B>, kSweepSmem<B>, s0>>>(b->d_inst, b->d_sweep + gr.sw0, parity);
                         else k_sweep_batch<float, M_JAC, B><<<gw, kSweepNT<B>, kSweepSmem<B>, s0>>>(b->d_inst, b->d_sweep + gr.sw0, parity);
                     };

@@ -201,6 +201,11 @@ struct Inst {
     const Brick *bricks;
     BrickLists lists;
     const real *cheb_table;
+    // torso handles: the voxels with nothing but torso around them are walked (nwalk items, 1/Dhat of such a voxel
+    // or -1), the others are rows
+    const Seg *walk;
+    const real *walk_dinv;
+    int nwalk, pad8;
     unsigned *sweep_arrive;   // arrivals of a checking sweep: kArriveGroups counters and the groups', 128 bytes apart
     int row_colour[9], pad6;
 };

@@ -41,6 +41,15 @@ __device__ __forceinline__ bool nonzero(double c) { return ((__double2hiint(c) &
 constexpr int kSweepThreads = 128;
 constexpr int kBrickThreads = 32 * kTileRows;
 
+// The forms of a tabulated sweep: rows; bricks; rows and the torso's walk.
+enum SweepForm { FORM_ROWS = 0, FORM_BRICKS = 1, FORM_TORSO = 2 };
+template <int FORM>
+constexpr int kSweepNT = FORM == FORM_BRICKS ? kBrickThreads : FORM == FORM_TORSO ? kThreads : kSweepThreads;
+// Resident CTAs asked for: 6 of rows (80 registers; 8 spill), 5 in a colour pass, whose gathers take more (176^3 heart:
+// 6.4 us a pass at 5, 6.9 at 6).
+template <typename real, int FORM, int MODE = M_JAC>
+constexpr int kSweepMinBlocks = sizeof(real) == 8 ? 2 : FORM == FORM_BRICKS ? EP_BRICK_BLOCKS : FORM == FORM_TORSO ? 3 : kGS<MODE> ? 5 : EP_SWEEP_BLOCKS;
+
 // What a sweep works on, from the control block and the descriptor.
 template <typename real>
 struct SweepOp {
@@ -328,24 +337,141 @@ __device__ __forceinline__ void sweep_brick(const Inst<float> &I, const SweepOp<
     }
 }
 
-// The work of CTA `cta` of the I.nsweep CTAs of a sweep, a brick or a share of the rows.  BRICKS: the handle's form,
-// and NT threads.
-template <typename real, int MODE, bool BRICKS>
-__device__ __forceinline__ void sweep_cta(const Inst<real> &I, int phase, int cta, BrickSmem *sm, double *sred,
+// One work item of the walk through the torso of a torso handle.  A voxel with nothing but torso around it (or the
+// grid's border) sees the isotropic operator sig_o I, which needs no record: F_a = C r_a^2 nT sig_o g_a with counts
+// that are constants of a lane, as in the walk over clear items (whose staging this shares: warp w copies voxel row w,
+// warp 0 also the ninth).  Every voxel of the grid is walked through; those that are not of this kind are not written
+// (walk_dinv < 0) and their values reach only vertices that no written voxel has.
+struct WalkSmem {
+    static constexpr int D = 4;
+    float u[D][kWarps + 1][32];
+    float b[D][kWarps][32], d[D][kWarps][32], p[D][kWarps][32];
+    float F[2][3][kWarps][32];
+};
+
+template <int MODE>
+__device__ __forceinline__ void sweep_walk(const Inst<float> &I, const SweepOp<float> &o, const float *src, float *out,
+                                           const Seg &sg, WalkSmem &sm, double &total)
+{
+    constexpr int D = WalkSmem::D;
+    const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
+    const int nx = I.nx, plane = I.nx * I.ny, nz = I.nz;
+    const int x = sg.x0 - 1 + lane, y = sg.by * kTileY + row - 1;
+    const bool own = x >= 0 && x < nx, left = x >= 1 && x - 1 < nx;
+    const bool yl = y >= 0 && y < I.ny, yh = y + 1 < I.ny;
+    const bool lo = own && yl, ninth = row == 0 && own && y + kWarps < I.ny;
+    const int q0 = x + nx * y, q8 = q0 + nx * kWarps;
+    const int cols = (left ? 1 : 0) + (own ? 1 : 0), rows = (yl ? 1 : 0) + (yh ? 1 : 0);
+    const float ax = rcp_count<float>((float)(cols == 2 ? rows : 0)), ay = rcp_count<float>((float)(rows == 2 ? cols : 0)),
+                az = rcp_count<float>((float)(cols * rows)), iso = I.C * I.sig_o * (float)(cols * rows);
+    const float kx = ax * ax * iso, ky = ay * ay * iso, kz = az * az * iso;   // one plane (kz: of two, half its voxels)
+    const int kbeg = sg.k0 - 1, kend = sg.k1;
+    auto issue = [&](int k, int slot) {
+        if (k <= kend) {
+            if ((unsigned)k < (unsigned)nz) {
+                if (lo) {
+                    const int q = q0 + k * plane;
+                    cp_async_n<4>(&sm.u[slot][row][lane], src + q);
+                    if (row > 0) {
+                        cp_async_n<4>(&sm.b[slot][row][lane], I.b + q);
+                        cp_async_n<4>(&sm.d[slot][row][lane], I.walk_dinv + q);
+                        if (kCheb<MODE> && o.cheb) cp_async_n<4>(&sm.p[slot][row][lane], out + q);
+                    }
+                }
+                if (ninth) cp_async_n<4>(&sm.u[slot][kWarps][lane], src + (q8 + k * plane));
+            } else {
+                sm.u[slot][row][lane] = 0.f;
+                if (row == 0) sm.u[slot][kWarps][lane] = 0.f;
+            }
+        }
+        cp_async_commit();
+    };
+#pragma unroll
+    for (int j = 0; j < D; ++j) {   // what no copy ever fills
+        if (!lo) sm.u[j][row][lane] = 0.f;
+        if (row == 0 && !ninth) sm.u[j][kWarps][lane] = 0.f;
+    }
+#pragma unroll
+    for (int j = 0; j < D - 1; ++j) issue(kbeg + j, j);
+    cp_async_wait<D - 2>();
+    __syncthreads();
+    const bool writes = row > 0 && lane >= 1 && lane <= kTileX && lo;
+    float X = 0.f, Y = 0.f, A = 0.f, S = 0.f, u = 0.f, b = 0.f, d = -1.f, pv = 0.f, acc = 0.f;
+    auto step = [&](int k, int slot) {
+        const int par = k & 1;
+        const float vl = sm.u[slot][row][lane], vh = sm.u[slot][row + 1][lane];
+        const float bn = sm.b[slot][row][lane], dn = sm.d[slot][row][lane];
+        const float pn = kCheb<MODE> ? sm.p[slot][row][lane] : 0.f;
+        const float s = vl + vh, t = vh - vl;
+        const float sl = __shfl_up_sync(kFull, s, 1), tl = __shfl_up_sync(kFull, t, 1);
+        const float Xn = s - sl, Yn = t + tl, An = s + sl;
+        float F0 = 0.f, F1 = 0.f, F2 = 0.f;
+        if (k > kbeg) {   // two planes: the squared counts' 1/4 times twice the voxels
+            const bool both = k > 0 && k < nz;
+            const float f = both ? 0.5f : 1.f;
+            F0 = kx * f * (X + Xn);
+            F1 = ky * f * (Y + Yn);
+            F2 = both ? 2.f * kz * (An - A) : 0.f;
+        }
+        X = Xn; Y = Yn; A = An;
+        sm.F[par][0][row][lane] = F0;
+        sm.F[par][1][row][lane] = F1;
+        sm.F[par][2][row][lane] = F2;
+        issue(k + D - 1, (slot + D - 1) % D);   // the slot of plane k - 1, which every warp has read
+        cp_async_wait<D - 2>();
+        __syncthreads();
+        const int below = row >= 1 ? row - 1 : 0;
+        const float p = sm.F[par][0][below][lane] + F0, q = sm.F[par][1][below][lane] - F1, r = sm.F[par][2][below][lane] + F2;
+        const float w = (p + q) + __shfl_down_sync(kFull, q - p, 1), z = r + __shfl_down_sync(kFull, r, 1);
+        if (k > kbeg + 1 && writes && d >= 0.f) {
+            const float res = sweep_out<float, MODE>(I, o, out, q0 + (k - 1) * plane, u, S + (w - z), b, d, pv);
+            acc += res * res;
+        }
+        S = w + z;
+        u = vl; b = bn; d = dn; pv = pn;
+    };
+    for (int k = kbeg;;) {
+        step(k, 0);
+        if (++k > kend) break;
+        step(k, 1);
+        if (++k > kend) break;
+        step(k, 2);
+        if (++k > kend) break;
+        step(k, 3);
+        if (++k > kend) break;
+    }
+    cp_async_wait<0>();
+    total += (double)acc;   // at most 32 planes in FP32, FP64 above
+}
+
+// The work of CTA `cta` of the I.nsweep CTAs of a sweep, a brick, an item of the torso's walk
+// or a share of the rows, after the handle's form.
+template <typename real, int MODE, int FORM>
+__device__ __forceinline__ void sweep_cta(const Inst<real> &I, int phase, int cta, unsigned char *smem, double *sred,
                                           int *sflag)
 {
-    constexpr int NT = BRICKS ? kBrickThreads : kSweepThreads;
+    constexpr int NT = kSweepNT<FORM>;
     const int parity = phase & 1;
     SweepOp<real> o;
     double acc = 0.0;
-    if constexpr (BRICKS) {
+    const int nwalk = FORM == FORM_TORSO ? I.nwalk : 0;
+    if (FORM == FORM_TORSO && cta < nwalk) {
+        if constexpr (FORM == FORM_TORSO) {
+            const Seg sg = I.walk[cta];
+            after_previous_launch();
+            if (!sweep_begin<real, MODE>(I, phase, o)) return;
+            sweep_walk<MODE>(I, o, sweep_src<real, MODE>(I, parity, o), sweep_dst<real, MODE>(I, parity), sg,
+                             *reinterpret_cast<WalkSmem *>(smem), acc);
+        }
+    } else if constexpr (FORM == FORM_BRICKS) {
         const Brick B = I.bricks[cta];
         after_previous_launch();
         if (!sweep_begin<real, MODE>(I, phase, o)) return;
-        sweep_brick<MODE>(I, o, sweep_src<real, MODE>(I, parity, o), sweep_dst<real, MODE>(I, parity), B, *sm, acc);
+        sweep_brick<MODE>(I, o, sweep_src<real, MODE>(I, parity, o), sweep_dst<real, MODE>(I, parity), B,
+                          *reinterpret_cast<BrickSmem *>(smem), acc);
     } else {
         const int r0 = kGS<MODE> ? I.row_colour[phase] : 0, r1 = kGS<MODE> ? I.row_colour[phase + 1] : I.nrows;
-        int i = r0 + cta * NT + threadIdx.x;
+        int i = r0 + (cta - nwalk) * NT + threadIdx.x;
         real c[kRowLen];
         if (i < r1) row_load(I, i, c);   // constants: read while the sweep before this one ends
         after_previous_launch();
@@ -358,7 +484,7 @@ __device__ __forceinline__ void sweep_cta(const Inst<real> &I, int phase, int ct
                 const float f = (float)r;
                 acc += (double)(f * f);
             }
-            i += I.nsweep * NT;
+            i += (I.nsweep - nwalk) * NT;
             if (i < r1) row_load(I, i, c);
         }
     }
@@ -393,49 +519,43 @@ __device__ __forceinline__ void sweep_cta(const Inst<real> &I, int phase, int ct
     }
 }
 
-// Bytes of dynamic shared memory and threads of a sweep CTA.
-template <bool BRICKS>
-constexpr size_t kSweepSmem = BRICKS ? sizeof(BrickSmem) : 0;
-template <bool BRICKS>
-constexpr int kSweepNT = BRICKS ? kBrickThreads : kSweepThreads;
-// Resident CTAs asked for: 6 of rows (80 registers; 8 spill), 5 in a colour pass, whose gathers take more (176^3 heart:
-// 6.4 us a pass at 5, 6.9 at 6).
-template <typename real, bool BRICKS, int MODE = M_JAC>
-constexpr int kSweepMinBlocks = sizeof(real) == 8 ? 2 : BRICKS ? EP_BRICK_BLOCKS : kGS<MODE> ? 5 : EP_SWEEP_BLOCKS;
+// Bytes of dynamic shared memory of a sweep CTA.
+template <int FORM>
+constexpr size_t kSweepSmem = FORM == FORM_BRICKS ? sizeof(BrickSmem) : FORM == FORM_TORSO ? sizeof(WalkSmem) : 0;
 
 // Single instance.
-template <typename real, int MODE, bool BRICKS>
-__global__ void __launch_bounds__(kSweepNT<BRICKS>, kSweepMinBlocks<real, BRICKS, MODE>) k_sweep(Inst<real> I, int phase)
+template <typename real, int MODE, int FORM>
+__global__ void __launch_bounds__(kSweepNT<FORM>, kSweepMinBlocks<real, FORM, MODE>) k_sweep(Inst<real> I, int phase)
 {
     extern __shared__ __align__(16) unsigned char ep_sweep_smem[];
-    __shared__ double sred[kSweepNT<BRICKS> / 32];
+    __shared__ double sred[kSweepNT<FORM> / 32];
     __shared__ int sflag;
-    sweep_cta<real, MODE, BRICKS>(I, phase, blockIdx.x, reinterpret_cast<BrickSmem *>(ep_sweep_smem), sred, &sflag);
+    sweep_cta<real, MODE, FORM>(I, phase, blockIdx.x, ep_sweep_smem, sred, &sflag);
 }
 
 // Batched: the sweep CTAs of all members of a list with this form (the batch's trial sweeps).
-template <typename real, int MODE, bool BRICKS>
-__global__ void __launch_bounds__(kSweepNT<BRICKS>, kSweepMinBlocks<real, BRICKS>)
+template <typename real, int MODE, int FORM>
+__global__ void __launch_bounds__(kSweepNT<FORM>, kSweepMinBlocks<real, FORM>)
 k_sweep_batch(const Inst<real> *insts, const BItem *items, int phase)
 {
     extern __shared__ __align__(16) unsigned char ep_sweep_smem[];
-    __shared__ double sred[kSweepNT<BRICKS> / 32];
+    __shared__ double sred[kSweepNT<FORM> / 32];
     __shared__ int sflag;
     __shared__ Inst<real> sI;
     const BItem it = items[blockIdx.x];
     const Inst<real> &I = stage_inst(insts + it.inst, sI);
-    if ((I.nbricks > 0) != BRICKS) return;
-    sweep_cta<real, MODE, BRICKS>(I, phase, it.item, reinterpret_cast<BrickSmem *>(ep_sweep_smem), sred, &sflag);
+    if ((I.nbricks > 0) != (FORM == FORM_BRICKS)) return;
+    sweep_cta<real, MODE, FORM>(I, phase, it.item, ep_sweep_smem, sred, &sflag);
 }
 
 // Batched: the unfinished members of a list (see k_stencil_active).  The descriptor is copied before the finished
 // flag is read, so a warp that leaves early has done its share.
-template <typename real, int MODE, bool BRICKS>
-__global__ void __launch_bounds__(kSweepNT<BRICKS>, kSweepMinBlocks<real, BRICKS>)
+template <typename real, int MODE, int FORM>
+__global__ void __launch_bounds__(kSweepNT<FORM>, kSweepMinBlocks<real, FORM>)
 k_sweep_active(const Inst<real> *insts, const ActRec *act, int n, int phase)
 {
     extern __shared__ __align__(16) unsigned char ep_sweep_smem[];
-    __shared__ double sred[kSweepNT<BRICKS> / 32];
+    __shared__ double sred[kSweepNT<FORM> / 32];
     __shared__ int sflag, sk;
     __shared__ Inst<real> sI;
     const int i = blockIdx.x;
@@ -449,7 +569,7 @@ k_sweep_active(const Inst<real> *insts, const ActRec *act, int n, int phase)
     if (sk < 0) return;
     const ActRec r = act[sk];
     const Inst<real> &I = stage_inst(insts + r.inst, sI);
-    sweep_cta<real, MODE, BRICKS>(I, phase, i - r.cum, reinterpret_cast<BrickSmem *>(ep_sweep_smem), sred, &sflag);
+    sweep_cta<real, MODE, FORM>(I, phase, i - r.cum, ep_sweep_smem, sred, &sflag);
 }
 
 // Explicit monodomain step over the rows, two launches: the reaction at every tissue voxel (v* into b, the new w),

@@ -107,6 +107,14 @@ __global__ void k_build_rows(int nx, int ny, int nz, double sT, double dS, doubl
     }
 }
 
+// 1/Dhat of the voxels of a torso handle that the walk takes, -1 elsewhere.
+template <typename real>
+__global__ void k_build_walk(long long n, const uint8_t *walked, const float4 *rec, real *dinv)
+{
+    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n; q += (long long)gridDim.x * blockDim.x)
+        dinv[q] = walked[q] ? (real)rec[q].w : real(-1);
+}
+
 // Lists of every brick, one CTA a brick: vertices in lattice order, the full ones (eight tissue voxels) first, then
 // the others that touch tissue; tissue voxels in window order, the inner ones (eight full vertices) first.  The
 // host counted them (struct Brick); a list that would pass its count is cut, and *bad is set.

@@ -127,6 +127,31 @@ def test_clear_items(kind, nx, ny, nz, diffusion):
     ref.close()
 
 
+# heart in a torso: rows near the tissue and around holes of the torso, the walk away from them (items of 30 x 7 x 8
+# at these sizes, cut by the box)
+@pytest.mark.parametrize("solver", [0, 1])
+@pytest.mark.parametrize("nx,ny,nz,fill", [(64, 47, 53, None), (91, 40, 61, 0.9995), (40, 38, 36, 0.9)])
+def test_torso_rows_and_walk(nx, ny, nz, fill, solver):
+    z, y, x = np.meshgrid(*[np.arange(n) + 0.5 - n / 2 for n in (nz, ny, nx)], indexing="ij")
+    r = np.sqrt(x * x + y * y + z * z)
+    c = W.random_case(11, nx, ny, nz, mask=((r < 14) & (r > 7)).astype(np.uint8)).fibres_as_float32()
+    c = W.with_torso(c, sig_o=0.8, fill=fill, seed=2)
+    p = c.params
+    p.solver, p.max_iter, p.rel_tol, p.check_every = solver, SWEEPS, 0.0, 2
+    p.cheb_lmin, p.cheb_lmax = (0.01, 6.0) if solver == 1 else (0.0, 0.0)
+    v, w, ve = W.random_state(11, c)
+    s, ref = ep.sim_from_case(c), oracle.Sim(c)
+    s.set_state(v, w, ve, 0)
+    ref.set_state(v, w, ve, 0)
+    assert s.step(1, allow_noconv=True).iters == SWEEPS
+    ref.step()
+    want = ref.state()["ve"]
+    tol = (32 * 6 * SWEEPS + 4 * 32) * 2.0 ** -24 * max(1.0, float(np.abs(want).max()))   # as for the rows
+    assert np.abs(s.read(ep.EP_VE) - want).max() <= tol
+    s.close()
+    ref.close()
+
+
 def test_tables_give_way_to_a_budget():
     """A batch budget that two handles meet without their tables, but not with them, admits both; they give the
     results of a handle that never had tables to the rounding of the operator's two forms."""
