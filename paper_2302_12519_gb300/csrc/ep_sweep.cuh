@@ -46,9 +46,9 @@ enum SweepForm { FORM_ROWS = 0, FORM_BRICKS = 1, FORM_TORSO = 2 };
 template <int FORM>
 constexpr int kSweepNT = FORM == FORM_BRICKS ? kBrickThreads : FORM == FORM_TORSO ? kThreads : kSweepThreads;
 // Resident CTAs asked for: 6 of rows (80 registers; 8 spill), 5 in a colour pass, whose gathers take more (176^3 heart:
-// 6.4 us a pass at 5, 6.9 at 6).
+// 6.4 us a pass at 5, 6.9 at 6), 4 of the torso's 256 threads (144^3 box: 36 us a sweep, 40 at 3).
 template <typename real, int FORM, int MODE = M_JAC>
-constexpr int kSweepMinBlocks = sizeof(real) == 8 ? 2 : FORM == FORM_BRICKS ? EP_BRICK_BLOCKS : FORM == FORM_TORSO ? 3 : kGS<MODE> ? 5 : EP_SWEEP_BLOCKS;
+constexpr int kSweepMinBlocks = sizeof(real) == 8 ? 2 : FORM == FORM_BRICKS ? EP_BRICK_BLOCKS : FORM == FORM_TORSO ? 4 : kGS<MODE> ? 5 : EP_SWEEP_BLOCKS;
 
 // What a sweep works on, from the control block and the descriptor.
 template <typename real>
@@ -341,7 +341,8 @@ __device__ __forceinline__ void sweep_brick(const Inst<float> &I, const SweepOp<
 // grid's border) sees the isotropic operator sig_o I, which needs no record: F_a = C r_a^2 nT sig_o g_a with counts
 // that are constants of a lane, as in the walk over clear items (whose staging this shares: warp w copies voxel row w,
 // warp 0 also the ninth).  Every voxel of the grid is walked through; those that are not of this kind are not written
-// (walk_dinv < 0) and their values reach only vertices that no written voxel has.
+// (walk_dinv < 0) and their values reach only vertices that no written voxel has.  With the rows beside it 36 us a sweep
+// of the 144^3 box (2.3 million voxels walked, 0.7 million rows); the two-term items and their single-term far ones 76.
 struct WalkSmem {
     static constexpr int D = 4;
     float u[D][kWarps + 1][32];
