@@ -340,12 +340,14 @@ typedef struct {
                                     each group takes about 1 ms of its sweeps, 8..64) */
     int zseg;                    /* z-planes per stencil work item (tuned) */
     size_t group_bytes;          /* members are swept in groups whose working sets total at most
-                                    this many bytes, so a group's sweeps stay in L2 (0 = one group; tuned) */
+                                    this many bytes, so a group's sweeps stay in L2 (0 = no limit; tuned); members with
+                                    operator tables also share at most 56 MB of them */
     int groups;                  /* number of such groups */
     int solo_members;            /* members whose Jacobi sweeps run as their own launches, concurrent
                                     with the packed launch of the others: those with at least half a
                                     wave of stencil items (3 CTAs per SM x SMs / 2, 228 on 152 SMs),
-                                    and every member of a group of at most 8 */
+                                    and every member of a group of at most 8 (of a group kept small by its members'
+                                    operator tables: those members) */
 } ep_batch_info;
 
 /* Create a batch of at most max_instances handles whose device memory may

@@ -41,6 +41,10 @@ constexpr int kZSeg = EP_ZSEG;     // default output planes per z-march segment
 constexpr int kZSegMin = 8;        // smallest segment length the batch autotuner tries
 constexpr int kSweepChunk[2] = {16, 64};   // launches of the queued graphs (multiples of 8: launches know their phase)
 constexpr int kSoloAllMembers = 8; // batch groups this small sweep every member in its own launches
+// Tables of a batch group's members together: what stays in the L2 cache from one sweep to the next.  Ten shells of 48^3
+// to 160^3 (160 MB of rows), two steps: one group 93 ms, groups of about 100 MB 74, 50 MB 70, 25 MB 80; forty of up to
+// 128^3: one group 153, 50 MB 106.
+constexpr size_t kGroupTables = EP_GROUP_TABLES;
 constexpr double kDivFactor = 1e16;
 constexpr int kNoAllocMaxPartials = 32768;   // ep_step_noalloc: stencil work items and reduction chunks
 
@@ -1037,6 +1041,7 @@ void drop_tables(ep_sim *s)
         s->allocs.erase(it);
     }
     s->dev_bytes -= s->tab_total;
+    s->tab_total = 0;
     s->tab = s->nrows = s->nbricks = s->nsweep = s->nwalk = 0;
     s->lean = true;
     s->sweep_graph.drop();
@@ -2352,13 +2357,16 @@ ep_status rebuild_tables(ep_batch *b)
     b->groups.clear();
     for (int r = 0; r < b->ninst;) {
         int r1 = r;
-        size_t bytes = 0;
+        size_t bytes = 0, tables = 0;
         const bool cheb = is_cheb(b->order[r]);
+        auto next = [&] { return b->slot[b->order[r1]]; };
         do {
-            bytes += 20 * (size_t)b->slot[b->order[r1]]->n;
+            bytes += 20 * (size_t)next()->n;
+            tables += next()->tab_total;
             ++r1;
         } while (r1 < b->ninst && is_cheb(b->order[r1]) == cheb &&
-                 (b->group_bytes == 0 || bytes + 20 * (size_t)b->slot[b->order[r1]]->n <= b->group_bytes));
+                 (b->group_bytes == 0 || bytes + 20 * (size_t)next()->n <= b->group_bytes) &&
+                 tables + next()->tab_total <= kGroupTables);
         ep_batch::Group g;
         g.cheb = cheb;
         g.sw0 = (long long)sweeps.size();
@@ -2384,10 +2392,14 @@ ep_status rebuild_tables(ep_batch *b)
         g.nsw = (long long)sweeps.size() - g.sw0;
         g.packed_tab[0] = g.packed_tab[1] = 0;
         g.packed_items = 0;
-        const bool few = r1 - r <= kSoloAllMembers;
+        // few members, each in its own launches: a whole solver's few, or the tabulated ones of a group that is small
+        // because of their tables
+        int same = 0;
+        for (int q : b->order) same += is_cheb(q) == cheb;
+        const bool small = r1 - r <= kSoloAllMembers, few = (b->group_bytes ? r1 - r : same) <= kSoloAllMembers;
         for (int q = r; q < r1; ++q) {
             ep_sim *s = b->slot[b->order[q]];
-            if (few || s->nseg >= b->solo_items) g.solo.push_back(q);
+            if (few || (small && s->tab) || s->nseg >= b->solo_items) g.solo.push_back(q);
             else if (s->tab) g.packed_tab[s->nbricks > 0] += s->nsweep;
             else g.packed_items += s->nseg;
         }
