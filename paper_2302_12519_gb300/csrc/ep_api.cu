@@ -1188,7 +1188,7 @@ struct OneSweep {
 // A kernel over the tabulated operator in the order of the stream.  In FP32 the launch may start while the one before
 // it still runs (the kernel waits for that one itself, after_previous_launch, before it touches what changes): 6.7 to
 // 5.7 us a sweep of the 128^3 shell, 3.2 to 2.6 of the 48^3 one.  Not in FP64, whose long kernels share the few FP64
-// lanes with the early one: 15 against 10 us a step of the 32^3 slab.
+// lanes with the early one: 15 against 10 us a step of the 32^3 slab (reaction and diffusion as two launches).
 template <typename real, typename... A>
 void launch_after(void (*kernel)(Inst<real>, A...), int grid, int block, size_t smem, cudaStream_t q, const Inst<real> &I, A... args)
 {
@@ -1502,7 +1502,7 @@ ep_status solve_elliptic(ep_sim *s, const Inst<real> &I, int &iters, double &rel
     return EP_OK;
 }
 
-// Explicit monodomain steps over the tabulated operator: two launches a step, replayed in graphs of kStepChunk steps.
+// Explicit monodomain steps over the tabulated operator: a launch a step, replayed in graphs of kStepChunk steps.
 constexpr int kStepChunk = 32;   // even: a graph starts on an even step
 
 template <typename real>
@@ -1511,11 +1511,11 @@ ep_status mono_steps(ep_sim *s, const Inst<real> &I, int n_steps)
     cudaStream_t st = s->stream;
     const int gr = grid_for(s->n_tissue, kSweepThreads);
     auto one = [&](int parity) {
-        launch_after(k_react<real>, gr, kSweepThreads, 0, st, I, parity);
-        launch_after(k_diffuse_rows<real>, gr, kSweepThreads, 0, st, I, parity);
+        launch_after(k_mono_step<real>, gr, kSweepThreads, 0, st, I, parity);
     };
     const long long tick[2] = {s->step, s->step};
     CK(cudaMemcpyAsync((char *)s->ctl + offsetof(Ctl, tick), tick, sizeof(tick), cudaMemcpyHostToDevice, st));
+    if (n_steps > 0) k_react<real><<<gr, kSweepThreads, 0, st>>>(I, (int)(s->step & 1));
     for (int it = 0; it < n_steps;) {
         if (!s->noalloc_call && !(s->step & 1) && n_steps - it >= kStepChunk) {
             if (!s->step_graph) {
@@ -1577,7 +1577,7 @@ ep_status step_typed(ep_sim *s, int n_steps, ep_step_stats *stats)
             float ms = 0.f;
             CK(cudaEventElapsedTime(&ms, s->pev[0], s->pev[1]));
             s->prof.other_ms += ms;
-            s->prof.other_launches += 2LL * n_steps;
+            s->prof.other_launches += n_steps + (n_steps > 0);
             s->prof.steps += n_steps;
         }
     }

@@ -573,13 +573,21 @@ k_sweep_active(const Inst<real> *insts, const ActRec *act, int n, int phase)
     sweep_cta<real, MODE, FORM>(I, phase, i - r.cum, ep_sweep_smem, sred, &sflag);
 }
 
-// Explicit monodomain step over the rows, two launches: the reaction at every tissue voxel (v* into b, the new w),
-// then the diffusion of v* (the new v, activation times, the non-finite flag).  The fused walk recomputes the
-// reaction of its halo and rebuilds the tensors; in FP64, where this GPU does two operations a clock and SM, that is
-// most of its time: 121 us a step of the 32^3 slab against 10 here.  In FP32 small grids are bound by latency: 61 x 45
-// x 53, 19.5 us a step in the walk, 7.3 here (two launches).  Launches of step parity p read the step from tick[p]; the second writes tick[p ^ 1].
+// Explicit monodomain steps over the rows.  A step is one launch: the diffusion of v* (the new v, activation times, the
+// non-finite flag), then the reaction of the next step at the same voxel (its v*, into the other of two buffers, and
+// its w, into the buffer of the w that this step used up); the first step of a call is led by the reaction alone.
+// The fused walk recomputes the reaction of its halo and rebuilds the tensors; in FP64, where this GPU does two
+// operations a clock and SM, that is most of its time: 121 us a step of the 32^3 slab against 8.5 here.  In FP32 small
+// grids are bound by latency: 61 x 45 x 53, 19.5 us a step in the walk, 7.1 with reaction and diffusion as two
+// launches, 5.2 here.  Launches of step parity p read the step from tick[p] and leave tick[p ^ 1].
 template <typename real>
-__device__ __forceinline__ void react_voxels(const Inst<real> &I, long long step, int first, int end, int stride)
+__device__ __forceinline__ real *vstar(const Inst<real> &I, int parity)
+{
+    return parity ? I.x1 : I.b;   // scratch between steps
+}
+
+template <typename real>
+__device__ __forceinline__ void react_voxels(const Inst<real> &I, long long step, real *vs_out, int first, int end, int stride)
 {
     const int parity = (int)(step & 1);
     const double tn = (double)step * I.dt_d;
@@ -596,49 +604,62 @@ __device__ __forceinline__ void react_voxels(const Inst<real> &I, long long step
         }
         real vs, ws;
         ms_step(I, stim, v[q], w[q], x, y, z, vs, ws);
-        I.b[q] = vs;
+        vs_out[q] = vs;
         wn[q] = ws;
     }
 }
 
-template <typename real>
-__device__ __forceinline__ void diffuse_rows(const Inst<real> &I, long long step, int first, int end, int stride)
+template <typename real, bool NEXT>
+__device__ __forceinline__ long long diffuse_rows(const Inst<real> &I, const long long *counter, const real *vs_in,
+                                                  real *vs_out, int first, int end, int stride)
 {
+    real c[kRowLen];
+    if (first < end) row_load(I, first, c);
+    after_previous_launch();
+    const long long step = *counter;
     const int parity = (int)(step & 1);
     const double tn = (double)step * I.dt_d;
     const real *v = I.v[parity];
     real *vn = I.v[parity ^ 1];
+    const unsigned stim = NEXT ? active_stimuli(I, (double)(step + 1) * I.dt_d) : 0u;
     for (int i = first; i < end; i += stride) {
-        real c[kRowLen];
-        row_load(I, i, c);
+        if (i != first) row_load(I, i, c);
         const int q = row_index(c[27]);
-        const real u = I.b[q], vold = v[q];
-        const real vnew = u - I.coef_par * row_apply(I, c, I.b + q, u);
+        const real u = vs_in[q], vold = v[q], w = NEXT ? I.w[parity ^ 1][q] : real(0);
+        const real vnew = u - I.coef_par * row_apply(I, c, vs_in + q, u);
         vn[q] = vnew;
         if (vold < real(0.5) && vnew >= real(0.5) && I.tact[q] < real(0))
             I.tact[q] = (real)(tn + I.dt_d * (0.5 - (double)vold) / ((double)vnew - (double)vold));
         if (!isfinite(vnew)) atomicOr(&I.ctl->nonfinite, 1);
+        if (NEXT) {
+            real vs, ws;
+            ms_step(I, stim, vnew, w, q % I.nx, (q / I.nx) % I.ny, q / (I.nx * I.ny), vs, ws);
+            vs_out[q] = vs;
+            I.w[parity][q] = ws;
+        }
     }
+    return step;
 }
 
 template <typename real>
 __global__ void __launch_bounds__(kSweepThreads) k_react(Inst<real> I, int parity)
 {
     after_previous_launch();
-    react_voxels(I, I.ctl->tick[parity], blockIdx.x * kSweepThreads + threadIdx.x, I.nrows, gridDim.x * kSweepThreads);
+    react_voxels(I, I.ctl->tick[parity], vstar(I, parity), blockIdx.x * kSweepThreads + threadIdx.x, I.nrows,
+                 gridDim.x * kSweepThreads);
 }
 
 template <typename real>
-__global__ void __launch_bounds__(kSweepThreads, sizeof(real) == 8 ? 2 : EP_SWEEP_BLOCKS) k_diffuse_rows(Inst<real> I, int parity)
+__global__ void __launch_bounds__(kSweepThreads, sizeof(real) == 8 ? 2 : EP_SWEEP_BLOCKS) k_mono_step(Inst<real> I, int parity)
 {
-    after_previous_launch();
-    const long long step = I.ctl->tick[parity];
-    diffuse_rows(I, step, blockIdx.x * kSweepThreads + threadIdx.x, I.nrows, gridDim.x * kSweepThreads);
+    const long long step = diffuse_rows<real, true>(I, &I.ctl->tick[parity], vstar(I, parity), vstar(I, parity ^ 1),
+                                                    blockIdx.x * kSweepThreads + threadIdx.x, I.nrows,
+                                                    gridDim.x * kSweepThreads);
     if (blockIdx.x == 0 && threadIdx.x == 0) I.ctl->tick[parity ^ 1] = step + 1;
 }
 
-// Batched: a share of a member's rows per entry of the packed reduction-chunk list (members with rows only); the
-// step counter moves at the end of the batched step.
+// Batched: a share of a member's rows per entry of the packed reduction-chunk list (members with rows only), reaction
+// and diffusion as two launches; the step counter moves at the end of the batched step.
 template <typename real, bool DIFFUSE>
 __global__ void __launch_bounds__(kSweepThreads, EP_SWEEP_BLOCKS) k_mono_batch(const Inst<real> *insts, const BItem *items)
 {
@@ -647,8 +668,8 @@ __global__ void __launch_bounds__(kSweepThreads, EP_SWEEP_BLOCKS) k_mono_batch(c
     const Inst<real> &I = stage_inst(insts + it.inst, sI);
     if (!I.tab) return;
     const int r0 = (int)((long long)I.nrows * it.item / it.nitems), r1 = (int)((long long)I.nrows * (it.item + 1) / it.nitems);
-    if (DIFFUSE) diffuse_rows(I, I.ctl->step, r0 + threadIdx.x, r1, kSweepThreads);
-    else react_voxels(I, I.ctl->step, r0 + threadIdx.x, r1, kSweepThreads);
+    if (DIFFUSE) diffuse_rows<real, false>(I, &I.ctl->step, I.b, nullptr, r0 + threadIdx.x, r1, kSweepThreads);
+    else react_voxels(I, I.ctl->step, I.b, r0 + threadIdx.x, r1, kSweepThreads);
 }
 
 // cheb_weight(k) for k < kChebTable - 1; the last entry is the weights' limit 2 e^-theta / rho.
