@@ -976,7 +976,7 @@ ep_status setup_typed(ep_sim *s)
         // for the estimate's error), the fastest contraction of the slow modes that stays stable
         if (s->p.jacobi_omega < 0.0) s->omega = std::min(1.0, 1.9 / s->cheb_lmax);
     }
-    if (tp.tab && s->p.solver == EP_SOLVER_CHEBYSHEV) {
+    if (tp.tab && s->p.solver == EP_SOLVER_CHEBYSHEV && s->cheb_lmax > 0.0) {
         const double rho = (s->cheb_lmax - s->cheb_lmin) / (s->cheb_lmax + s->cheb_lmin);
         k_cheb_table<real><<<1, 1024, 0, st>>>(rho, std::acosh(1.0 / rho), (real *)s->cheb_table);
     }
@@ -3059,6 +3059,7 @@ void serve_loop(ep_server *v)
             if (budget && r->peak > budget && !r->sim->ready && !r->sim->lean) {   // without its tables it may fit
                 r->sim->lean = true;
                 if (plan_layout(r->sim) == EP_OK) r->peak = r->sim->fp_peak;
+                if (r->peak > budget) r->sim->lean = false;   // rejected all the same: the handle goes back as it came
             }
             if (budget && r->peak > budget) {
                 srv_erase(v->queue, r);
