@@ -542,14 +542,14 @@ __device__ __forceinline__ void ring_plane(const Inst<real> &I, const Op<real> &
 
 // The walk over a clear item (kClearItem).  The mask there is the grid itself, so a lane's pair counts are constants
 // of its column and rows, and off the grid u and the records are 0: no flag or count is formed in the loop, and the
-// sums s and differences d of a column's two voxels carry the gradient (g_x: s - s_left over both planes, g_y:
-// d + d_left, g_z: the change of s + s_left) and, transposed, the scatter.  Bound by instruction issue and the shared
+// differences of a column's two voxels from the left ones, from one another and from the plane below carry the gradient
+// (differences first: of neighbours they are all but exact) and sums and differences, transposed, the scatter.  Bound by instruction issue and the shared
 // memory pipe (shuffles, records); 164 instructions a plane and warp of the implicit sweep instead of 230 before the
 // rows were shared.  256^3 monodomain slab: 298 us a step without, 217 with rings of each thread's own, 189 with the
 // shared one.
 template <typename real>
 struct ClearState {
-    real X, Y, A;       // gradient sums of this plane
+    real X, Y, h;       // gradient sums of this plane; the voxel (x, hi)
     real M[6];          // sum of f f^T over the four voxels of this plane
     real S;             // what the vertex plane below leaves to this plane's output
     real u, e0, e1, e2; // output voxel (x, lo)
@@ -661,17 +661,17 @@ struct ClearWalk {
                            a0 * a1 + b0 * b1, a0 * a2 + b0 * b2, a1 * a2 + b1 * b2};
 #pragma unroll
         for (int j = 0; j < 6; ++j) C.M[j] = Z[j] + __shfl_up_sync(kFull, Z[j], 1);
-        const real s = lo + hi, d = hi - lo;
-        const real sl = __shfl_up_sync(kFull, s, 1), dl = __shfl_up_sync(kFull, d, 1);
-        C.X = s - sl;
-        C.Y = d + dl;
-        C.A = s + sl;
+        const real ll = __shfl_up_sync(kFull, lo, 1), lh = __shfl_up_sync(kFull, hi, 1);
+        const real up = (lo - P.u) + (hi - P.h), upl = __shfl_up_sync(kFull, up, 1);
+        C.X = (lo - ll) + (hi - lh);
+        C.Y = (hi - lo) + (lh - ll);
+        C.h = hi;
         real F0 = real(0), F1 = real(0), F2 = real(0);
         if (k > kbeg) {
             const bool both = k < o.nz && k > 0;   // planes of the vertex plane in the grid: two, or one at its ends
             const real f = both ? real(0.5) : real(1), iso = both ? c.iso + c.iso : c.iso;
             const real rx = c.ax * f, ry = c.ay * f, rz = both ? c.az : real(0);
-            const real hx = (P.X + C.X) * rx, hy = (P.Y + C.Y) * ry, hz = (C.A - P.A) * rz;
+            const real hx = (P.X + C.X) * rx, hy = (P.Y + C.Y) * ry, hz = (up + upl) * rz;
             const real M0 = P.M[0] + C.M[0], M1 = P.M[1] + C.M[1], M2 = P.M[2] + C.M[2];
             const real M3 = P.M[3] + C.M[3], M4 = P.M[4] + C.M[4], M5 = P.M[5] + C.M[5];
             F0 = rx * (iso * hx + o.dS * (M0 * hx + M3 * hy + M4 * hz));
@@ -697,7 +697,7 @@ struct ClearWalk {
     __device__ __forceinline__ void walk()
     {
         ClearState<real> S0, S1;
-        S0.X = S0.Y = S0.A = S0.S = S0.u = S0.e0 = S0.e1 = S0.e2 = real(0);
+        S0.X = S0.Y = S0.h = S0.S = S0.u = S0.e0 = S0.e1 = S0.e2 = real(0);
 #pragma unroll
         for (int j = 0; j < 6; ++j) S0.M[j] = real(0);
         S1 = S0;

@@ -273,10 +273,10 @@ __device__ __forceinline__ void sweep_brick(const Inst<float> &I, const SweepOp<
         const float u4 = v[0], u5 = v[1], u6 = v[32], u7 = v[33];
         float gx, gy, gz;
         if (t < B.nfull) {
-            const float s0 = u0 + u1, s1 = u2 + u3, s2 = u4 + u5, s3 = u6 + u7;
+            // differences first: of neighbours they are all but exact, where sums would round at the iterate's own size
             gx = ((u1 - u0) + (u3 - u2)) + ((u5 - u4) + (u7 - u6));
-            gy = (s1 - s0) + (s3 - s2);
-            gz = (s2 - s0) + (s3 - s1);
+            gy = ((u2 - u0) + (u3 - u1)) + ((u6 - u4) + (u7 - u5));
+            gz = ((u4 - u0) + (u5 - u1)) + ((u6 - u2) + (u7 - u3));
         } else {
             const unsigned w = I.lists.vpair[B.pbase + t - B.nfull];
             auto pair = [&](int bit, float lo, float hi) { return (w >> bit) & 1u ? hi - lo : 0.f; };
@@ -397,24 +397,26 @@ __device__ __forceinline__ void sweep_walk(const Inst<float> &I, const SweepOp<f
     cp_async_wait<D - 2>();
     __syncthreads();
     const bool writes = row > 0 && lane >= 1 && lane <= kTileX && lo;
-    float X = 0.f, Y = 0.f, A = 0.f, S = 0.f, u = 0.f, b = 0.f, d = -1.f, pv = 0.f, acc = 0.f;
+    float X = 0.f, Y = 0.f, S = 0.f, u = 0.f, h = 0.f, b = 0.f, d = -1.f, pv = 0.f, acc = 0.f;
     auto step = [&](int k, int slot) {
         const int par = k & 1;
         const float vl = sm.u[slot][row][lane], vh = sm.u[slot][row + 1][lane];
         const float bn = sm.b[slot][row][lane], dn = sm.d[slot][row][lane];
         const float pn = kCheb<MODE> ? sm.p[slot][row][lane] : 0.f;
-        const float s = vl + vh, t = vh - vl;
-        const float sl = __shfl_up_sync(kFull, s, 1), tl = __shfl_up_sync(kFull, t, 1);
-        const float Xn = s - sl, Yn = t + tl, An = s + sl;
+        // differences first: of neighbours they are all but exact, where sums would round at the iterate's own size
+        // (the 144^3 box took 5 to 9 % more sweeps to a residual of 1e-6 over sums)
+        const float ll = __shfl_up_sync(kFull, vl, 1), lh = __shfl_up_sync(kFull, vh, 1);
+        const float c = (vl - u) + (vh - h), cl = __shfl_up_sync(kFull, c, 1);
+        const float Xn = (vl - ll) + (vh - lh), Yn = (vh - vl) + (lh - ll);
         float F0 = 0.f, F1 = 0.f, F2 = 0.f;
         if (k > kbeg) {   // two planes: the squared counts' 1/4 times twice the voxels
             const bool both = k > 0 && k < nz;
             const float f = both ? 0.5f : 1.f;
             F0 = kx * f * (X + Xn);
             F1 = ky * f * (Y + Yn);
-            F2 = both ? 2.f * kz * (An - A) : 0.f;
+            F2 = both ? 2.f * kz * (c + cl) : 0.f;
         }
-        X = Xn; Y = Yn; A = An;
+        X = Xn; Y = Yn;
         sm.F[par][0][row][lane] = F0;
         sm.F[par][1][row][lane] = F1;
         sm.F[par][2][row][lane] = F2;
@@ -429,7 +431,7 @@ __device__ __forceinline__ void sweep_walk(const Inst<float> &I, const SweepOp<f
             acc += res * res;
         }
         S = w + z;
-        u = vl; b = bn; d = dn; pv = pn;
+        u = vl; h = vh; b = bn; d = dn; pv = pn;
     };
     for (int k = kbeg;;) {
         step(k, 0);

@@ -152,6 +152,36 @@ def test_torso_rows_and_walk(nx, ny, nz, fill, solver):
     ref.close()
 
 
+@pytest.mark.parametrize("kind,nx,ny,nz", [("torso", 64, 47, 53), ("full", 91, 91, 89), ("full", 33, 31, 29)])
+def test_differences_of_large_values(kind, nx, ny, nz):
+    """The residual of a start that is large against its differences (2^14 and 0 to 4 units in the last place) is the
+    FP64 operator's on the same start and the same new v: neighbours are subtracted before anything is added."""
+    mask = np.ones((nz, ny, nx), np.uint8)
+    if kind == "torso":
+        z, y, x = np.meshgrid(*[np.arange(n) + 0.5 - n / 2 for n in (nz, ny, nx)], indexing="ij")
+        r = np.sqrt(x * x + y * y + z * z)
+        mask = ((r < 14) & (r > 7)).astype(np.uint8)
+    h = []
+    for precision in (W.FP32, W.FP64):
+        c = W.random_case(13, nx, ny, nz, mask=mask, precision=precision).fibres_as_float32()
+        if kind == "torso":
+            c = W.with_torso(c, sig_o=0.8)
+        c.params.max_iter, c.params.rel_tol, c.params.check_every = 1, 0.0, 1
+        h.append(ep.sim_from_case(c))
+    v, w, ve = W.random_state(13, c)
+    far = 2.0 ** 14 + 2.0 ** -9 * np.random.default_rng(13).integers(0, 5, ve.size)
+    far = np.where(ve != 0.0, far, 0.0)
+    h[0].set_state(2.0 ** -10 * v, w, far, 0)
+    got = h[0].step(1, allow_noconv=True).rel_res
+    b = -h[1].apply_operator(c.params.sig_iL, c.params.sig_iT, h[0].read(ep.EP_V))
+    want = np.linalg.norm(b - h[1].apply_elliptic(far)) / np.linalg.norm(b)
+    for s in h:
+        s.close()
+    # the rounding of a residual, as above, is under 32 x 6 of 2^-24 of its terms, in norm far less; sums of values
+    # would be off by one unit of 2^14 in every second one, a tenth of the residual
+    assert abs(got / want - 1.0) <= 1e-4
+
+
 def test_tables_give_way_to_a_budget():
     """A batch budget that two handles meet without their tables, but not with them, admits both; they give the
     results of a handle that never had tables to the rounding of the operator's two forms."""
