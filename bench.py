@@ -148,14 +148,25 @@ def _peaks():
 
 
 def _kernel_hash():
-    """Identity of the stencil kernels' code: SHA-256 of ep_common.cuh and
-    ep_stencil.cuh with their line comments and blank lines removed, so that an
-    edit of comments alone keeps a profile record current."""
+    """Identity of the stencil and sweep kernels' code: SHA-256 of their
+    headers with line comments and blank lines removed, so that an edit of
+    comments alone keeps a profile record current."""
     h = hashlib.sha256()
-    for p in ("paper_2302_12519_gb300/csrc/ep_common.cuh", "paper_2302_12519_gb300/csrc/ep_stencil.cuh"):
-        code = [ln.split("//", 1)[0].rstrip() for ln in open(os.path.join(ROOT, p)).read().splitlines()]
+    for p in ("ep_common.cuh", "ep_stencil.cuh", "ep_tables.cuh", "ep_sweep.cuh"):
+        path = os.path.join(ROOT, "paper_2302_12519_gb300/csrc", p)
+        code = [ln.split("//", 1)[0].rstrip() for ln in open(path).read().splitlines()]
         h.update(("\n".join(c for c in code if c.strip()) + "\n").encode())
     return h.hexdigest()[:16]
+
+
+def _sweep_kernel(mode, n_tissue):
+    """Name of the FP32 elliptic sweep kernel without a torso: over assembled
+    rows up to 720 thousand tissue voxels (the colour sweeps always), over
+    vertex lists in bricks above, the z-march where no tables are kept."""
+    if n_tissue < 4096:
+        return f"k_stencil<float,{mode}>"
+    rows = mode == "M_JAC_GS" or n_tissue <= 720000
+    return f"k_sweep<float,{mode},{'FORM_ROWS' if rows else 'FORM_BRICKS'}>"
 
 
 def _traffic_record(stem):
@@ -483,8 +494,8 @@ def solver_legs(ep, case, a, blob0, stream, flush, end_state, peak):
         total_s = sum(ms) / 1e3
         d = {"value": M * a.steps / total_s, "unit": "tissue voxel-steps/s", "ms_per_step": 1e3 * total_s / a.steps,
              "sweeps_per_step": iters, "step_status": statuses,
-             "kernel": ("k_stencil<float,M_JAC_CHEB> (correction form)" if solver == 1 else
-                        "k_stencil<float,M_JAC_GS> (one colour pass; 8 a sweep)"),
+             "kernel": (_sweep_kernel("M_JAC_CHEB", M) + " (correction form)" if solver == 1 else
+                        _sweep_kernel("M_JAC_GS", M) + " (one colour pass; 8 a sweep)"),
              "avg_launch_us": launch_s * 1e6, "algorithmic_bytes_per_voxel": per,
              "traffic_bytes_per_voxel": _traffic_record(("chebyshev_sweep_" if solver == 1 else "gauss_seidel_pass_")
                                                         + a.workload),
@@ -670,13 +681,17 @@ def run_ours(a):
         # the implicit sweeps dominate the step
         launch_s = prof.ie_sweep_ms / 1e3 / max(prof.ie_sweeps, 1)
         alg_bytes = BYTES_PER_IE_SWEEP_VOXEL * M
-        kname, share = "k_stencil<float,M_IE> (implicit-Euler Jacobi sweep)", prof.ie_sweep_ms / 1e3 / total_s
+        kname = (_sweep_kernel("M_IE", M) if M <= 720000 else "k_stencil<float,M_IE>") + " (implicit-Euler Jacobi sweep)"
+        share = prof.ie_sweep_ms / 1e3 / total_s
     elif mono:
         # the fused reaction + diffusion launch is the step (plus a one-thread step-counter kernel)
         launch_s = prof.other_ms / 1e3 / max(prof.steps, 1)
         # v, w read and written at the state precision, fibre 6, mask 1
         alg_bytes = (BYTES_PER_MONO_VOXEL if case.precision == 0 else 4 * 8 + 16) * M
-        kname = "k_stencil<%s,M_PAR_MONO> (fused reaction + diffusion)" % ("float" if case.precision == 0 else "double")
+        kname = ("%s<%s%s> (fused reaction + diffusion)" %
+                 (("k_mono_step", "float" if case.precision == 0 else "double", "")
+                  if M >= 4096 and (case.precision != 0 or M <= 720000) else
+                  ("k_stencil", "float" if case.precision == 0 else "double", ",M_PAR_MONO")))
         share = prof.other_ms / 1e3 / total_s
     else:
         sweep_s = prof.sweep_ms / 1e3
@@ -684,13 +699,12 @@ def run_ours(a):
         per_voxel = (BYTES_PER_CHEB_SWEEP_VOXEL if a.solver == "chebyshev" else
                      BYTES_PER_GS_PASS_VOXEL if a.solver == "gs" else BYTES_PER_SWEEP_VOXEL)
         alg_bytes = per_voxel * n_dom   # over tissue + torso when a torso is set
-        kname = ("k_stencil<float,M_JAC(_CHEB)> over the torso items away from the tissue + "
-                 "k_stencil<float,M_JAC_BATH(_CHEB)> over the rest (one elliptic sweep over tissue + torso)"
-                 if torso else "k_stencil<float,M_JAC> (damped Jacobi sweep)")
+        kname = ("k_sweep<float,M_JAC(_CHEB),FORM_TORSO> (one elliptic sweep over tissue + torso)"
+                 if torso else _sweep_kernel("M_JAC", M) + " (damped Jacobi sweep)")
         if a.solver == "chebyshev":
             kname += ", Chebyshev-accelerated"
         if a.solver == "gs":
-            kname = "k_stencil<float,M_JAC_GS> (one colour pass of the eight-colour Gauss-Seidel sweep)"
+            kname = _sweep_kernel("M_JAC_GS", M) + " (one colour pass of the eight-colour Gauss-Seidel sweep)"
         share = sweep_s / total_s
     achieved = alg_bytes / launch_s / 1e9 if launch_s > 0 else 0.0
     stem = (f"ie_sweep_slab{a.slab_n}_mono" if mono and implicit else

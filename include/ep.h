@@ -154,8 +154,8 @@ typedef struct {
                                       an estimated jacobi_omega; 0 when neither needs one */
     long long n_domain;      /* voxels of the elliptic equation: tissue, plus the torso if set */
     int n_segments_elliptic; /* work items of the elliptic sweeps (n_segments without a torso) */
-    int n_segments_far;      /* of those, items whose voxels and halo hold no tissue (swept by the
-                                single-term kernel: there the operator is the torso's alone) */
+    int n_segments_far;      /* of those, items whose voxels and halo hold no tissue (there the operator is the
+                                torso's alone: without operator tables the single-term kernel sweeps them) */
 } ep_info;
 
 typedef struct ep_sim ep_sim;
@@ -213,7 +213,8 @@ ep_status ep_write_state(ep_sim *s, const void *host, size_t bytes);
 /* Apply the diffusion operator L_{sL,sT} = G'^T S G' of the handle's mask and
  * fibres to a host field u (n doubles), writing L u (n doubles; zero off the
  * tissue).  L u approximates -div(Sigma grad u) (Sec. "Operators / Laplacian",
- * Eq. ass3).  Uses the same stencil kernel as the time step. */
+ * Eq. ass3).  Uses the stencil kernel of the steps and sweeps that keep no
+ * operator tables. */
 ep_status ep_apply_operator(ep_sim *s, double sig_L, double sig_T,
                             const double *u_host, double *out_host, size_t n);
 
@@ -259,7 +260,8 @@ ep_status ep_read_ecg(ep_sim *s, ep_ecg_sample *out, int max_samples, int *n_out
 
 /* Apply the elliptic operator of the handle (L_i + L_e, plus the torso's
  * sig_o I if set) to a host field u (n doubles), writing n doubles (zero
- * outside tissue + torso), with the same kernel as the solve's sweeps.
+ * outside tissue + torso), with the stencil kernels of a solve without
+ * operator tables.
  * Diagnostic. */
 ep_status ep_apply_elliptic(ep_sim *s, const double *u_host, double *out_host, size_t n);
 
@@ -277,7 +279,8 @@ ep_status ep_apply_elliptic(ep_sim *s, const double *u_host, double *out_host, s
  * or ep_get_info call, which allocate), else EP_ESTATE.  Limits: at most
  * 32768 stencil work items (ep_info.n_segments) and 32768 reduction chunks
  * (2048 tissue voxels each), at most 4096 tissue components; larger problems
- * get EP_EINVAL with a message.  The first call on a device looks up the
+ * get EP_EINVAL with a message.  A handle whose table sweeps would need more
+ * than 32768 partial sums takes the stencil kernels instead.  The first call on a device looks up the
  * array's device address (cudaGetSymbolAddress) with that device current,
  * and looks it up again when the device's context has changed since (after
  * a cudaDeviceReset the handle itself must be created anew: its device
@@ -307,7 +310,13 @@ typedef struct {
  * connected components, reduction chunks, work items) made without touching
  * the device: resident_bytes is what the handle holds once set up, peak_bytes
  * the most it holds during set-up (staging of fibres, mask and records).
- * After set-up both equal the bytes held.  EP_ESTATE without a mask,
+ * After set-up both equal the bytes held.  From 4096 tissue voxels on they
+ * include the operator tables, known once the parameters are set: 112 bytes
+ * a tissue voxel in FP32 (224 in FP64), about 90 for FP32 bidomain handles
+ * above 720 thousand tissue voxels, none for FP32 monodomain ones of that
+ * size; with a torso, for the voxels at the tissue only.  A handle runs
+ * without them where they do not fit: if their allocation fails, or a batch
+ * or server would else refuse it for its budget.  EP_ESTATE without a mask,
  * EP_EINVAL if the mask has no tissue.  Host-only; needs no GPU.  No
  * counterpart in the paper: admission control of the served form. */
 ep_status ep_footprint(ep_sim *s, size_t *resident_bytes, size_t *peak_bytes);

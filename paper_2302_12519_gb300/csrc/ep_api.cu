@@ -449,13 +449,13 @@ bool needs_spectrum(const ep_sim *s)
     return s->p.solver == EP_SOLVER_CHEBYSHEV || (s->p.solver == EP_SOLVER_JACOBI && s->p.jacobi_omega < 0.0);
 }
 
-// The elliptic sweeps of a bidomain handle without a torso, and the diffusion of a monodomain one, run over the
-// tabulated operator.  Below kTabMin tissue
-// voxels a sweep is a launch's latency on either path, and the handle stays as small as its fields.
+// The elliptic sweeps of a bidomain handle (with a torso in FP32), and the diffusion of a monodomain one, run over the
+// tabulated operator.  Below kTabMin tissue voxels a sweep is a launch's latency on either path, and the handle stays
+// as small as its fields.
 constexpr long long kTabMin = 4096;
 // Assembled rows for every tissue voxel (112 bytes a row in FP32) up to this many: the rows then stay in the L2
 // cache.  Above it the bricks: 671 thousand voxels (192^3 shell) take 15.5 us a sweep in rows and 18.3 in bricks, 831
-// thousand (160^3 heart) 23.1 and 19.8, 3.41 million (256^3 heart) 91 and 55.6.
+// thousand (160^3 heart) 23.1 and 19.8, 3.41 million (256^3 heart) 91 and 56.2.
 constexpr long long kRowsOnly = EP_ROWS_ONLY;
 constexpr int kMaxRowCtas = 4096;
 constexpr size_t kArriveBytes = sizeof(unsigned) * kArriveStride * (kArriveGroups + 1);
@@ -1263,8 +1263,8 @@ ep_status build_sweep_graph(ep_sim *s, const Sweep &sweep, int n, cudaGraphExec_
 // never waits for the host.  Around the number that the solve before needed the graphs have 16 launches, and from that
 // number on each graph's own flag is waited for: queued launches after the end return at once, but in 1.5 us each (a
 // solve of 11 sweeps under two graphs of 64 spent 175 us of its 950 us step on them).  At most max_iter sweeps
-// (per_sweep launches each) do work; the launch
-// after them marks a capped solve done.  Returns the launches queued in *queued_out.
+// (per_sweep launches each) do work; the launch after them marks a capped solve done.  Returns the launches queued in
+// *queued_out.
 template <typename Sweep>
 ep_status run_sweeps(ep_sim *s, const Sweep &sweep, ep_sim::SweepGraphs *graphs, long long *queued_out, int per_sweep = 1)
 {

@@ -545,8 +545,8 @@ __device__ __forceinline__ void ring_plane(const Inst<real> &I, const Op<real> &
 // differences of a column's two voxels from the left ones, from one another and from the plane below carry the gradient
 // (differences first: of neighbours they are all but exact) and sums and differences, transposed, the scatter.  Bound by instruction issue and the shared
 // memory pipe (shuffles, records); 164 instructions a plane and warp of the implicit sweep instead of 230 before the
-// rows were shared.  256^3 monodomain slab: 298 us a step without, 217 with rings of each thread's own, 189 with the
-// shared one.
+// rows were shared.  256^3 monodomain slab: 298 us a step without, 217 with rings of each thread's own, 193 with the
+// shared one (189 with sums of neighbours before differences, which lost digits of the iterate).
 template <typename real>
 struct ClearState {
     real X, Y, h;       // gradient sums of this plane; the voxel (x, hi)

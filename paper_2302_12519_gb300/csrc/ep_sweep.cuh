@@ -6,8 +6,8 @@
 // A colour pass of Gauss-Seidel reads its own eighth of the rows only: 6.4 us a pass on 1.10 million voxels, where
 // the march forms every flux for one voxel in eight, 32 us.
 // Bricks: 36 bytes of K and place a voxel (30 x 6 x 8 bricks share their lattices' faces), 16 of fields.  Bound by
-// memory latency: the lists alone stream in 32 us of the 256^3 heart's 55.6 (3.41 million voxels; the march 69.9, bound
-// by its instructions, 53 million against 33).  Measured against it and dropped: a z-march over K with packed columns
+// memory latency: the lists alone stream in 32 us of the 256^3 heart's 56.2 (3.41 million voxels; the march 69.9, bound
+// by its instructions, 53 million against 35).  Measured against it and dropped: a z-march over K with packed columns
 // and masked loads (54 us with the surface voxels as rows; its loads wait on one another), the same with a cp.async
 // ring (65 us), bricks of 6 x 6 (58.7) and 8 x 12 (91), two bricks in flight a CTA (58), all loads of a brick at
 // once (61).
