@@ -143,6 +143,8 @@ struct ep_sim {
     void *x2 = nullptr;          // second correction buffer of the FP32 elliptic solve (correction form)
     long long ie_seen = 0;                // implicit sweeps counted by earlier calls
     long long step = 0;
+    // times that its work items or tables changed since set-up: what a batch keeps of them is stale then
+    long long layout = 0;
     // tabulated elliptic operator (ep_tables.cuh); lean: left out, where its memory is not to be had
     bool lean = false;
     size_t tab_total = 0;   // its device bytes
@@ -1044,6 +1046,7 @@ void drop_tables(ep_sim *s)
     s->tab_total = 0;
     s->tab = s->nrows = s->nbricks = s->nsweep = s->nwalk = 0;
     s->lean = true;
+    ++s->layout;
     s->sweep_graph.drop();
     s->ie_graph.drop();
     if (s->step_graph) cudaGraphExecDestroy(s->step_graph);
@@ -2265,6 +2268,7 @@ struct ep_batch {
     int ninst = 0;
     long long nseg_items = 0, nchunk_items = 0;
     std::vector<int> order;        // slot of each table row
+    std::vector<long long> layouts;   // its handle's layout when the tables were built
     cudaGraphExec_t graph = nullptr;
     bool dirty = true;
     int nsm = 152, sweeps_per_check = 16, zseg = kZSeg;
@@ -2315,6 +2319,7 @@ ep_status relayout_segments(ep_sim *s, int zseg)
     CK(cudaStreamSynchronize(s->stream));
     s->nseg = (int)segs.size();
     s->zseg = zseg;
+    ++s->layout;
     s->sweep_graph.drop();
     s->ie_graph.drop();
     return EP_OK;
@@ -2436,8 +2441,20 @@ ep_status rebuild_tables(ep_batch *b)
         b->graph = nullptr;
     }
     b->last.assign(b->ninst, Ctl{});
+    b->layouts.clear();
+    for (int i : b->order) b->layouts.push_back(b->slot[i]->layout);
     b->dirty = false;
     return EP_OK;
+}
+
+// The tables as the members stand now: a member that another batch holds too may have lost its operator tables, or
+// got other work items, there.
+ep_status current_tables(ep_batch *b)
+{
+    bool stale = b->dirty;
+    for (size_t r = 0; r < b->layouts.size() && !stale; ++r) stale = b->slot[b->order[r]]->layout != b->layouts[r];
+    b->dirty = stale;
+    return stale ? rebuild_tables(b) : EP_OK;
 }
 
 int grid_of(long long items, int cap) { return (int)std::max<long long>(1, std::min<long long>(items, cap)); }
@@ -2689,7 +2706,6 @@ ep_status ep_batch_add(ep_batch *b, ep_sim *s, int *slot)
                 if (t && t->tab && used + s->dev_bytes > b->budget) {
                     used -= t->tab_total;
                     drop_tables(t);
-                    b->dirty = true;
                 }
         }
     }
@@ -2724,7 +2740,7 @@ ep_status ep_batch_step(ep_batch *b, int n_steps)
     if (!b) return EP_EINVAL;
     if (n_steps < 0) return bfail(b, EP_EINVAL, "n_steps must be >= 0");
     ep_status st;
-    if (b->dirty && (st = rebuild_tables(b)) != EP_OK) return st;
+    if ((st = current_tables(b)) != EP_OK) return st;
     if (b->ninst == 0 || n_steps == 0) return EP_OK;
     if ((st = build_batch_graph(b)) != EP_OK) return st;
     cudaStream_t s0 = b->stream;
@@ -2773,7 +2789,7 @@ ep_status ep_batch_autotune(ep_batch *b, int trial_sweeps)
 {
     if (!b || trial_sweeps < 1) return EP_EINVAL;
     ep_status st;
-    if (b->dirty && (st = rebuild_tables(b)) != EP_OK) return st;
+    if ((st = current_tables(b)) != EP_OK) return st;
     if (b->ninst == 0) return EP_OK;
     cudaStream_t s0 = b->stream;
     // snapshot the solve state of every member: v_e (x0) and the control block
@@ -2905,7 +2921,7 @@ ep_status ep_batch_get_info(ep_batch *b, ep_batch_info *info)
 {
     if (!b || !info) return EP_EINVAL;
     ep_status st;
-    if (b->dirty && (st = rebuild_tables(b)) != EP_OK) return st;
+    if ((st = current_tables(b)) != EP_OK) return st;
     info->instances = b->ninst;
     info->stencil_items = b->nseg_items;
     info->chunk_items = b->nchunk_items;

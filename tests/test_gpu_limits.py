@@ -1,0 +1,63 @@
+"""Where memory or the stream sets a limit: budgets and allocators that hold a handle's fields but not its operator
+tables, a handle held by two batches, streams that cannot be captured.  None of it faults the GPU: budgets and
+allocators refuse on the host."""
+import numpy as np
+import pytest
+
+import oracle
+import paper_2302_12519_gb300 as ep
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+FIELDS = (ep.EP_V, ep.EP_W, ep.EP_VE, ep.EP_TACT)
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_2302_12519_gb300 import build
+    build.build()
+    ep.load()
+
+
+@pytest.mark.parametrize("change", ["budget", "work items"])
+def test_a_handle_in_two_batches(change):
+    """A handle that another batch strips of its operator tables (a budget that only bare handles meet), or gives other
+    work items, is stepped right by the batch that held it before, whose lists were built on what it had."""
+    tabulated = change == "budget"
+    nx, ny, nz = (40, 30, 20) if tabulated else (12, 10, 30)   # 3 600 voxels have no tables
+    cases = [W.random_case(14 + i, nx - i, ny, nz, mask=np.ones((nz, ny, nx - i), np.uint8)) for i in range(2)]
+    for c in cases:
+        c.params.max_iter, c.params.rel_tol, c.params.check_every = 4, 0.0, 2
+    hs = [[ep.sim_from_case(c) for c in cases] for _ in range(2)]
+    for pair in hs:
+        for i, (h, c) in enumerate(zip(pair, cases)):
+            h.set_state(*W.random_state(14 + i, c), 0)
+    (a, other), alone = hs[0], hs[1][0]
+    first = ep.Batch(1)
+    first.set_schedule(0, 64, 0)
+    first.add(a)
+    first.step(2, allow_noconv=True)
+    budget = 0
+    if tabulated:   # room for the other handle's tables at most
+        rows = 112 * cases[0].n_tissue
+        budget = a.info().device_bytes + other.info().device_bytes - rows
+    second = ep.Batch(2, hbm_budget_bytes=budget)
+    second.set_schedule(0, 64 if tabulated else 8, 0)
+    second.add(other)
+    held = a.info().device_bytes
+    second.add(a)
+    assert (a.info().device_bytes < held) == tabulated
+    first.step(2, allow_noconv=True)
+    second.step(1, allow_noconv=True)
+    alone.step(5, allow_noconv=True)
+    # five steps of four sweeps over the operator's other form: 32 roundings of 2^-24 of 6 max|x| a sweep, four more a
+    # step for v and the right-hand side, carried at most exp(5 dt 0.25 / tau_in)
+    p = cases[0].params
+    tol = 5 * (32 * 6 * 4 + 4 * 32) * 2.0 ** -24 * np.exp(5 * p.dt * 0.25 / p.tau_in)
+    for f in FIELDS[:3]:
+        assert np.abs(a.read(f) - alone.read(f)).max() <= tol * max(1.0, float(np.abs(alone.read(f)).max()))
+    first.close()
+    second.close()
+    for h in hs[0] + hs[1]:
+        h.close()
