@@ -24,7 +24,8 @@
  *    keeps no pointer to caller memory.
  *  - Device memory is owned by the handle.  It is allocated with
  *    ep_grid_desc.dev_alloc / dev_free when both are set (e.g. a framework's
- *    caching allocator), otherwise with cudaMalloc / cudaFree.
+ *    caching allocator; at least 16-byte aligned), otherwise with cudaMalloc /
+ *    cudaFree.
  *  - All work is issued on ep_grid_desc.cuda_stream (NULL = the legacy
  *    default stream).  Calls that return host data synchronise that stream.
  *  - A handle is not thread safe: use it from one host thread at a time.

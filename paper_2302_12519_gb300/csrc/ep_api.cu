@@ -12,6 +12,7 @@
 // never stalls the GPU between sweeps.
 #include <algorithm>
 #include <cmath>
+#include <cstdint>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -150,7 +151,7 @@ struct ep_sim {
     size_t tab_total = 0;   // its device bytes
     int tab = 0, nrows = 0, nbricks = 0, nsweep = 0;
     int row_colour[9] = {};
-    void *rows = nullptr, *cheb_table = nullptr;
+    void *rows_mem = nullptr, *rows = nullptr, *cheb_table = nullptr;   // rows: where rows_mem is aligned as they are read
     Brick *bricks = nullptr;
     BrickLists lists{};
     unsigned *sweep_arrive = nullptr;
@@ -496,6 +497,10 @@ TabPlan tab_plan(const ep_sim *s)
     return t;
 }
 
+// FP64 rows are read in 32 bytes, twice what the rest of a handle asks of a device allocator's alignment: 16 bytes to
+// round up with.
+size_t rows_bytes(size_t rb, long long nrows) { return abytes(rb * kRowLen * (size_t)nrows + (rb == 8 ? 16 : 0)); }
+
 size_t tab_bytes(const ep_sim *s, const TabPlan &t, size_t rb)
 {
     if (!t.tab) return 0;
@@ -506,7 +511,7 @@ size_t tab_bytes(const ep_sim *s, const TabPlan &t, size_t rb)
             abytes(sizeof(float2) * (size_t)P.n_vert) + abytes(2 * (size_t)P.n_vert) + abytes(2 * (size_t)P.n_part) +
             abytes(sizeof(float2) * (size_t)s->n_tissue) + abytes((size_t)P.n_bound);
     else
-        b = abytes(rb * kRowLen * (size_t)t.nrows);
+        b = rows_bytes(rb, t.nrows);
     if (!s->torso.empty()) b += abytes(sizeof(Seg) * (size_t)t.nwalk) + abytes(rb * (size_t)s->n);
     return b + abytes(rb * kChebTable) + abytes(kArriveBytes);
 }
@@ -832,7 +837,7 @@ ep_status setup_typed(ep_sim *s)
     s->nbricks = tp.nbricks;
     s->nsweep = tp.nsweep;
     s->tab_total = tab_bytes(s, tp, rb);
-    s->rows = nullptr;
+    s->rows_mem = s->rows = nullptr;
     s->bricks = nullptr;
     if (tp.tab) {
         bool got = true;
@@ -851,8 +856,9 @@ ep_status setup_typed(ep_sim *s)
             take(s->lists.out, nt);
             take(s->lists.oflag, (size_t)P.n_bound);
         } else {
-            s->rows = dalloc(s, rb * kRowLen * (size_t)tp.nrows);
-            got = got && s->rows;
+            s->rows_mem = dalloc(s, rows_bytes(rb, tp.nrows));
+            s->rows = (void *)(((uintptr_t)s->rows_mem + 4 * rb - 1) / (4 * rb) * (4 * rb));
+            got = got && s->rows_mem;
         }
         s->nwalk = tp.nwalk;
         if (torso) {
@@ -1033,7 +1039,7 @@ void drop_tables(ep_sim *s)
 {
     if (!s->tab) return;
     if (s->stream) cudaStreamSynchronize(s->stream);
-    for (void *t : {(void *)s->rows, s->cheb_table, (void *)s->sweep_arrive, (void *)s->bricks, (void *)s->lists.k4,
+    for (void *t : {s->rows_mem, s->cheb_table, (void *)s->sweep_arrive, (void *)s->bricks, (void *)s->lists.k4,
                     (void *)s->lists.k2, (void *)s->lists.vloc, (void *)s->lists.vpair, (void *)s->lists.out,
                     (void *)s->lists.oflag, (void *)s->walk, s->walk_dinv}) {
         auto it = t ? std::find(s->allocs.begin(), s->allocs.end(), t) : s->allocs.end();

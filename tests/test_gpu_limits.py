@@ -61,3 +61,23 @@ def test_a_handle_in_two_batches(change):
     second.close()
     for h in hs[0] + hs[1]:
         h.close()
+
+
+@pytest.mark.parametrize("model,precision", [(W.BI, W.FP64), (W.MONO, W.FP64), (W.BI, W.FP32)])
+def test_an_allocator_that_aligns_to_16_bytes(model, precision):
+    """Every block lies 16 bytes past a 32-byte boundary: the results are those of well aligned memory, bit for bit."""
+    alloc, free = ep.torch_allocator()
+    c = W.random_case(33, 17, 16, 16, model=model, mask=np.ones((16, 16, 17), np.uint8), precision=precision)
+    c.params.max_iter, c.params.rel_tol, c.params.check_every = 5, 0.0, 2
+    v, w, ve = W.random_state(33, c)
+    out = []
+    for pair in ((alloc, free), (lambda n: alloc(n + 16) + 16, lambda p: free(p - 16))):
+        s = ep.sim_from_case(c, allocator=pair)
+        s.set_state(v, w, ve, 0)
+        s.step(2, allow_noconv=True)
+        resident = s.info().device_bytes
+        assert resident == s.footprint()[0]
+        out.append([s.read(f) for f in FIELDS])
+        s.close()
+    for a, b in zip(*out):
+        np.testing.assert_array_equal(a, b)
