@@ -1514,39 +1514,48 @@ ep_status solve_elliptic(ep_sim *s, const Inst<real> &I, int &iters, double &rel
 // Explicit monodomain steps over the tabulated operator: a launch a step, replayed in graphs of kStepChunk steps.
 constexpr int kStepChunk = 32;   // even: a graph starts on an even step
 
+// The graph is captured on a stream of its own: the handle's may be one that cannot be captured (the legacy default
+// stream), or a blocking one, whose capture would make another thread's calls on the default stream fail.
+template <typename Step>
+bool build_step_graph(ep_sim *s, const Step &one)
+{
+    cudaStream_t q = nullptr;
+    cudaGraph_t g = nullptr;
+    cudaError_t e = cudaStreamCreateWithFlags(&q, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaStreamBeginCapture(q, cudaStreamCaptureModeThreadLocal);
+    if (e == cudaSuccess) {
+        for (int i = 0; i < kStepChunk; ++i) one(q, i & 1);
+        e = cudaStreamEndCapture(q, &g);
+    }
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&s->step_graph, g, 0);
+    if (g) cudaGraphDestroy(g);
+    if (q) cudaStreamDestroy(q);
+    if (e != cudaSuccess) s->step_graph = nullptr;
+    cudaGetLastError();
+    return e == cudaSuccess;
+}
+
 template <typename real>
 ep_status mono_steps(ep_sim *s, const Inst<real> &I, int n_steps)
 {
     cudaStream_t st = s->stream;
     const int gr = grid_for(s->n_tissue, kSweepThreads);
-    auto one = [&](int parity) {
-        launch_after(k_mono_step<real>, gr, kSweepThreads, 0, st, I, parity);
-    };
+    auto one = [&](cudaStream_t q, int parity) { launch_after(k_mono_step<real>, gr, kSweepThreads, 0, q, I, parity); };
     const long long tick[2] = {s->step, s->step};
     CK(cudaMemcpyAsync((char *)s->ctl + offsetof(Ctl, tick), tick, sizeof(tick), cudaMemcpyHostToDevice, st));
     if (n_steps > 0) k_react<real><<<gr, kSweepThreads, 0, st>>>(I, (int)(s->step & 1));
+    bool graphs = !s->noalloc_call;
     for (int it = 0; it < n_steps;) {
-        if (!s->noalloc_call && !(s->step & 1) && n_steps - it >= kStepChunk) {
-            if (!s->step_graph) {
-                cudaGraph_t g = nullptr;
-                CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-                for (int i = 0; i < kStepChunk; ++i) one(i & 1);
-                cudaError_t e = cudaStreamEndCapture(st, &g);
-                if (e == cudaSuccess) {
-                    e = cudaGraphInstantiate(&s->step_graph, g, 0);
-                    cudaGraphDestroy(g);
-                }
-                if (e != cudaSuccess) {
-                    cudaGetLastError();
-                    s->step_graph = nullptr;
-                    return fail(s, EP_ECUDA, std::string("step graph: ") + cudaGetErrorString(e));
-                }
+        if (graphs && !(s->step & 1) && n_steps - it >= kStepChunk) {
+            if (!s->step_graph && !build_step_graph(s, one)) {
+                graphs = false;   // single launches do as well
+                continue;
             }
             CK(cudaGraphLaunch(s->step_graph, st));
             it += kStepChunk;
             s->step += kStepChunk;
         } else {
-            one((int)(s->step & 1));
+            one(st, (int)(s->step & 1));
             CK(cudaGetLastError());
             ++it;
             ++s->step;

@@ -81,3 +81,25 @@ def test_an_allocator_that_aligns_to_16_bytes(model, precision):
         s.close()
     for a, b in zip(*out):
         np.testing.assert_array_equal(a, b)
+
+
+CUDA_STREAM_LEGACY = 1   # cudaStreamLegacy: the default stream, which cannot be captured
+
+
+# 70 steps: two graphs of 32 and six single launches
+@pytest.mark.parametrize("precision", [W.FP32, W.FP64])
+def test_monodomain_steps_on_a_stream_that_cannot_be_captured(precision):
+    c = W.random_case(31, 17, 16, 16, model=W.MONO, mask=np.ones((16, 16, 17), np.uint8), precision=precision)
+    v, w, _ = W.random_state(31, c)
+    out = []
+    for stream in (None, CUDA_STREAM_LEGACY):
+        s = ep.Sim(c.nx, c.ny, c.nz, c.dx, ep.EP_MONO, precision, use_torch=False, stream=stream)
+        s.set_mask(c.mask_flat())
+        s.set_fibres(c.fib_flat())
+        s.set_params(c.params)
+        s.set_state(v, w, None, 0)
+        assert s.step(70).step == 70
+        out.append([s.read(f) for f in FIELDS])
+        s.close()
+    for a, b in zip(*out):
+        np.testing.assert_array_equal(a, b)
