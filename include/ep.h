@@ -408,12 +408,15 @@ void ep_batch_destroy(ep_batch *b);
  * optional) plus a step count and a release time.  Released requests are
  * admitted in release order while a slot is free and the request's set-up
  * peak (ep_footprint) fits the budget next to the bytes of every request the
- * server holds (running or finished and not yet collected); a request whose
- * peak alone exceeds the budget finishes with EP_EREJECTED.  Admitted
+ * server holds (running or finished and not yet collected).  Where operator
+ * tables alone keep it out they are given up: the request's own, then those of
+ * finished and of running requests, as many as it takes.  A request whose
+ * peak without tables exceeds the budget finishes with EP_EREJECTED.  Admitted
  * requests are set up on the device and stepped with the other members in
  * chunks of at most chunk_steps steps; a chunk never takes a member past its
  * step count, and requests join or leave only between chunks.  Each request
- * computes exactly what ep_step on the handle alone computes.
+ * computes exactly what ep_step on the handle alone computes (one that gave
+ * its tables up: to the rounding of the operator's other form).
  *
  * Ownership: ep_server_submit hands the handle to the server; it comes back
  * in the ep_request_result of ep_server_collect (state on the device, read

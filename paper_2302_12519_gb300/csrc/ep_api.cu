@@ -2999,7 +2999,7 @@ struct SrvReq {
     ep_sim *sim = nullptr;
     int n_steps = 0, steps_done = 0, slot = -1, model = 0;
     int status = EP_OK, plan_status = EP_OK;
-    bool cancel = false, busy = false, planned = false;
+    bool cancel = false, busy = false, planned = false, lean0 = false;
     double release = 0, t_admit = -1, t_done = -1;
     long long iters_base = 0, total_iters = 0;
     size_t peak = 0, bytes = 0;
@@ -3059,6 +3059,46 @@ void srv_erase(std::deque<SrvReq *> &q, SrvReq *r)
     if (it != q.end()) q.erase(it);
 }
 
+// Set-up peak of a planned request (what it holds, once set up) without its operator tables.
+size_t srv_bare(const SrvReq *r)
+{
+    ep_sim *s = r->sim;
+    if (s->ready) return s->dev_bytes - s->tab_total;
+    const bool lean = s->lean;
+    size_t resident = 0, peak = 0;
+    s->lean = true;
+    footprint(s, sizeof(float), &resident, &peak);
+    s->lean = lean;
+    return peak;
+}
+
+// mu held.  Whether the request fits the budget beside what the server holds.  Where operator tables alone keep it out
+// they give way, as in a batch: its own first (a request that is not set up leaves them out), then those of results
+// not yet collected, then those of the running requests, as many as it takes.
+bool srv_make_room(ep_server *v, SrvReq *r, size_t bare, size_t budget)
+{
+    if (v->hbm_in_use + r->peak <= budget) return true;
+    std::vector<SrvReq *> held;   // that were admitted: what a refused or cancelled handle has is not the server's
+    for (SrvReq *q : v->finished)
+        if (q->bytes && q->sim->tab) held.push_back(q);
+    for (SrvReq *q : v->active)
+        if (q->sim->tab) held.push_back(q);
+    size_t tables = 0;
+    for (const SrvReq *q : held) tables += q->sim->tab_total;
+    if (v->hbm_in_use - tables + bare > budget) return false;
+    if (r->sim->ready) drop_tables(r->sim);
+    else r->sim->lean = true;
+    r->peak = bare;
+    for (SrvReq *q : held) {
+        if (v->hbm_in_use + r->peak <= budget) break;
+        const size_t b = q->sim->tab_total;
+        drop_tables(q->sim);
+        q->bytes -= b;
+        v->hbm_in_use -= b;
+    }
+    return true;
+}
+
 void serve_loop(ep_server *v)
 {
     cudaSetDevice(v->device);
@@ -3087,12 +3127,8 @@ void serve_loop(ep_server *v)
                 srv_finish(v, r, r->plan_status);
                 continue;
             }
-            if (budget && r->peak > budget && !r->sim->ready && !r->sim->lean) {   // without its tables it may fit
-                r->sim->lean = true;
-                if (plan_layout(r->sim) == EP_OK) r->peak = r->sim->fp_peak;
-                if (r->peak > budget) r->sim->lean = false;   // rejected all the same: the handle goes back as it came
-            }
-            if (budget && r->peak > budget) {
+            const size_t bare = srv_bare(r);
+            if (budget && bare > budget) {
                 srv_erase(v->queue, r);
                 ++v->st.rejected;
                 srv_finish(v, r, EP_EREJECTED);
@@ -3109,7 +3145,8 @@ void serve_loop(ep_server *v)
                 for (const SrvReq *q : v->active) items += q->sim->nseg;
                 if (items > v->cfg.max_active_items) break;
             }
-            if (budget && v->hbm_in_use + r->peak > budget) {   // wait for memory to be released
+            r->lean0 = r->sim->lean;
+            if (budget && !srv_make_room(v, r, bare, budget)) {   // wait for memory to be released
                 if (v->active.empty() && !v->finished.empty() && !v->blocked_on_results) {
                     v->blocked_on_results = true;
                     v->cv_done.notify_all();
@@ -3141,6 +3178,7 @@ void serve_loop(ep_server *v)
             v->hbm_in_use += r->bytes;
             if (as != EP_OK) {
                 if (slot >= 0) ep_batch_remove(v->batch[r->model], slot);
+                if (!r->sim->ready) r->sim->lean = r->lean0;   // the handle goes back as it came
                 v->err = std::string("admission of request ") + std::to_string(r->id) + " failed: " + r->sim->err +
                          " " + ep_batch_last_error(v->batch[r->model]);
                 srv_finish(v, r, as);

@@ -103,3 +103,83 @@ def test_monodomain_steps_on_a_stream_that_cannot_be_captured(precision):
         s.close()
     for a, b in zip(*out):
         np.testing.assert_array_equal(a, b)
+
+
+def _shell(seed):
+    """Few tissue voxels in a large box: its tables (112 bytes a tissue voxel) are less than the set-up's staging."""
+    c = W.sampled_shell(np.random.default_rng(seed), 48, 10, f"shell{seed}")
+    c.params.max_iter, c.params.rel_tol = 50, 0.0
+    return c, ep.sim_from_case(c, use_torch=False)
+
+
+def _sizes():
+    """Device bytes of such a handle and the peak of its set-up, with tables and without."""
+    c, s = _shell(0)
+    resident, peak = s.footprint()
+    s.close()
+    tables = 112 * c.n_tissue
+    assert c.n_tissue >= 4096 and peak - resident > tables   # so that one handle alone fits every budget below
+    return resident, peak, resident - tables, peak - tables
+
+
+SLACK = 1 << 17   # the Chebyshev weights, counters and partial sums that belong to the tables
+
+
+# What two requests need at once: the second without its tables; both without; the first a result not yet collected.
+@pytest.mark.parametrize("who", ["second", "both", "result"])
+def test_server_gives_tables_up_to_admit(who):
+    resident, peak, bare, bare_peak = _sizes()
+    budget = (resident if who == "second" else bare) + bare_peak + SLACK
+    assert peak <= budget < resident + peak
+    srv = ep.Server(max_slots=4, chunk_steps=2, hbm_budget_bytes=budget)
+    first = srv.submit(_shell(0)[1], 2 if who == "result" else 400)
+    if who == "result":
+        srv.drain(timeout_s=60)
+    second = srv.submit(_shell(0)[1], 2)
+    srv.drain(timeout_s=60)   # EP_EBUSY if the second request waits for the first one's memory
+    got = {r.id: (r, s) for r, s in srv.collect(max_results=4)}
+    assert {first, second} == set(got)
+    for r, s in got.values():
+        assert r.status in (ep.EP_OK, ep.EP_ENOCONV) and r.device_bytes == s.info().device_bytes
+    if who != "result":
+        assert got[second][0].t_admit_s < got[first][0].t_done_s
+    assert (got[first][0].device_bytes < resident) == (who != "second") and got[second][0].device_bytes < resident
+    assert srv.stats().hbm_peak <= budget and srv.stats().hbm_in_use == 0
+    srv.close()
+    if who != "both":
+        return
+    c, alone = _shell(0)   # both ran on without tables: two steps against a handle that has them
+    alone.step(2, allow_noconv=True)
+    # 50 sweeps a step, 32 roundings of 2^-24 of 6 max|x| a sweep and four more a step for v and the right-hand side
+    tol = 2 * (32 * 6 * 50 + 4 * 32) * 2.0 ** -24
+    for f in FIELDS[:3]:
+        assert np.abs(got[second][1].read(f) - alone.read(f)).max() <= tol * max(1.0, float(np.abs(alone.read(f)).max()))
+    alone.close()
+
+
+def test_server_takes_a_set_up_handle_without_its_tables():
+    """A handle that comes with its tables, for a budget that it meets without them."""
+    resident, _, bare, _ = _sizes()
+    s = _shell(0)[1]
+    assert s.info().device_bytes == resident
+    srv = ep.Server(max_slots=1, hbm_budget_bytes=bare + SLACK)
+    srv.submit(s, 2)
+    srv.drain(timeout_s=60)
+    (r, s), = srv.collect()
+    assert r.status in (ep.EP_OK, ep.EP_ENOCONV) and r.steps_done == 2 and r.device_bytes <= bare + SLACK
+    s.close()
+    srv.close()
+
+
+def test_server_leaves_a_rejected_handle_its_tables():
+    _, _, bare, bare_peak = _sizes()
+    fresh, ready = _shell(0)[1], _shell(0)[1]
+    held = ready.info().device_bytes
+    plan = fresh.footprint()
+    srv = ep.Server(max_slots=2, hbm_budget_bytes=bare - SLACK)
+    ids = [srv.submit(fresh, 2), srv.submit(ready, 2)]
+    srv.drain(timeout_s=60)
+    got = {r.id: (r, s) for r, s in srv.collect()}
+    assert all(got[i][0].status == ep.EP_EREJECTED for i in ids)
+    assert got[ids[0]][1].footprint() == plan and got[ids[1]][1].info().device_bytes == held
+    srv.close()
