@@ -1423,6 +1423,7 @@ ep_status ensure_ready(ep_sim *s)
         dfree_all(s);
         s->lean = true;
         st = setup();
+        if (st != EP_OK) s->lean = false;   // the next attempt may find room for them
     }
     if (st != EP_OK) {
         dfree_all(s);

@@ -183,3 +183,83 @@ def test_server_leaves_a_rejected_handle_its_tables():
     assert all(got[i][0].status == ep.EP_EREJECTED for i in ids)
     assert got[ids[0]][1].footprint() == plan and got[ids[1]][1].info().device_bytes == held
     srv.close()
+
+
+class CappedAllocator:
+    """torch's caching allocator behind the dev_alloc / dev_free hooks, up to `cap` bytes at a time."""
+
+    def __init__(self, cap):
+        self.alloc, self.free = ep.torch_allocator()
+        self.cap, self.size = cap, {}
+
+    def pair(self):
+        def alloc(nbytes):
+            if sum(self.size.values()) + nbytes > self.cap:
+                return 0
+            p = self.alloc(nbytes)
+            self.size[p] = nbytes
+            return p
+
+        def free(ptr):
+            del self.size[ptr]
+            self.free(ptr)
+
+        return alloc, free
+
+
+# the last row: a colour pass over rows, bricks (737 thousand voxels), rows and the torso's walk
+@pytest.mark.parametrize("kind,model,precision,solver", [("box", W.BI, W.FP32, 1), ("box", W.BI, W.FP64, 0),
+                                                         ("box", W.MONO, W.FP32, 0), ("box", W.MONO, W.FP64, 0),
+                                                         ("box", W.BI, W.FP32, 2), ("big", W.BI, W.FP32, 0),
+                                                         ("torso", W.BI, W.FP32, 1)])
+def test_tables_that_do_not_fit_are_left_out(kind, model, precision, solver):
+    """Memory for a handle's fields and staging but not its tables: it steps without them, to the rounding of the
+    operator's two forms of the oracle; and after an attempt that had no room at all, a later one gets its tables."""
+    nx, ny, nz = {"box": (23, 20, 19), "big": (91, 91, 89), "torso": (47, 40, 41)}[kind]
+    mask = np.ones((nz, ny, nx), np.uint8)
+    if kind == "torso":
+        z, y, x = np.meshgrid(*[np.arange(n) + 0.5 - n / 2 for n in (nz, ny, nx)], indexing="ij")
+        r = np.sqrt(x * x + y * y + z * z)
+        mask = ((r < 14) & (r > 7)).astype(np.uint8)
+    c = W.random_case(35, nx, ny, nz, model=model, mask=mask, precision=precision).fibres_as_float32()
+    if kind == "torso":
+        c = W.with_torso(c, sig_o=0.8)
+    p = c.params
+    p.solver, p.max_iter, p.rel_tol, p.check_every = solver, 4, 0.0, 2
+    p.cheb_lmin, p.cheb_lmax = (0.01, 6.0) if solver == 1 else (0.0, 0.0)
+    p.omega = 1.3 if solver == 2 else 0.0
+    probe = ep.sim_from_case(c)
+    full = probe.footprint()
+    probe.close()
+    mem = CappedAllocator(full[1] // 8)
+    s = ep.sim_from_case(c, allocator=mem.pair())
+    with pytest.raises(ep.EPError) as e:
+        s.info()
+    assert e.value.status == ep.EP_ENOMEM and not mem.size
+    assert s.footprint() == full
+    mem.cap = full[1] - 1   # one byte short of the tables
+    held = s.info().device_bytes
+    assert held == sum(mem.size.values()) < full[0]
+    v, w, ve = W.random_state(35, c)
+    ref = oracle.Sim(c)
+    s.set_state(v, w, ve, 0)
+    ref.set_state(v, w, ve, 0)
+    s.step(1, allow_noconv=True)
+    ref.step()
+    want = ref.state()
+    # four sweeps of 32 roundings of 2^-24 (FP64: 1/D is stored in FP32) of 6 max|x|, and v and the right-hand side
+    for f, k in ((ep.EP_V, "v"), (ep.EP_W, "w")) + (((ep.EP_VE, "ve"),) if model == W.BI else ()):
+        x = max(1.0, float(np.abs(want[k]).max()))
+        tol = (32 * 6 * 4 + 4 * 32) * 2.0 ** -24 * x if precision == W.FP32 else 6 * 4 * 2.0 ** -24 * x
+        assert np.abs(s.read(f) - want[k]).max() <= tol
+    s.close()
+    ref.close()
+    assert not mem.size
+    mem.cap = full[1]
+    s = ep.sim_from_case(c, allocator=mem.pair())
+    mem.cap = full[1] // 8
+    with pytest.raises(ep.EPError):
+        s.info()
+    mem.cap = full[1]
+    assert s.info().device_bytes == full[0]
+    s.close()
