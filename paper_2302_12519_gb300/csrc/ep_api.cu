@@ -2475,6 +2475,17 @@ ep_status current_tables(ep_batch *b)
 
 int grid_of(long long items, int cap) { return (int)std::max<long long>(1, std::min<long long>(items, cap)); }
 
+// Monodomain members with tables, and the grid of their launches.
+bool mono_tables(const ep_batch *b)
+{
+    return b->model == EP_MONO && std::any_of(b->order.begin(), b->order.end(), [&](int i) { return b->slot[i]->tab != 0; });
+}
+dim3 mono_shares(const ep_batch *b)
+{
+    const int nc = std::max(1, (int)b->nchunk_items);
+    return dim3(nc, std::max(1, std::min(kChunk / kSweepThreads, 3 * EP_SWEEP_BLOCKS * b->nsm / nc)));
+}
+
 // One graph runs a whole chunk of steps: an outer loop over the steps left
 // (device counter) whose body is one step; inside it, the sweeps of all
 // unfinished solves repeat until every member has converged (or hit its cap).
@@ -2520,13 +2531,10 @@ ep_status build_batch_graph(ep_batch *b)
 
     CKB(cudaStreamBeginCaptureToGraph(st, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
     if (b->model == EP_MONO) {
-        bool any = false, general = false;
-        for (int r = 0; r < b->ninst; ++r) (b->slot[b->order[r]]->tab ? any : general) = true;
+        bool general = false;
+        for (int r = 0; r < b->ninst; ++r) general = general || !b->slot[b->order[r]]->tab;
         if (general) k_stencil_batch<float, M_PAR_MONO><<<gs, kThreads, kSmemBytes<float, M_PAR_MONO>, st>>>(b->d_inst, b->d_seg);
-        if (any) {
-            k_mono_batch<float, false><<<nc, kSweepThreads, 0, st>>>(b->d_inst, b->d_chunk);
-            k_mono_batch<float, true><<<nc, kSweepThreads, 0, st>>>(b->d_inst, b->d_chunk);
-        }
+        if (mono_tables(b)) k_mono_batch<float, true><<<mono_shares(b), kSweepThreads, 0, st>>>(b->d_inst, b->d_chunk);
     }
     else k_stencil_batch<float, M_PAR_BI><<<gs, kThreads, kSmemBytes<float, M_PAR_BI>, st>>>(b->d_inst, b->d_seg);
     if (b->model == EP_BI) {
@@ -2770,6 +2778,10 @@ ep_status ep_batch_step(ep_batch *b, int n_steps)
     }
     const long long n = n_steps;
     CKB(cudaMemcpyAsync(b->d_steps_left, &n, sizeof(n), cudaMemcpyHostToDevice, s0));
+    if (mono_tables(b)) {   // a step's launch ends with the reaction of the next
+        k_mono_batch<float, false><<<mono_shares(b), kSweepThreads, 0, s0>>>(b->d_inst, b->d_chunk);
+        CKB(cudaGetLastError());
+    }
     CKB(cudaGraphLaunch(b->graph, s0));
     for (int r = 0; r < b->ninst; ++r)
         CKB(cudaMemcpyAsync(&b->last[r], b->slot[b->order[r]]->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s0));

@@ -611,9 +611,9 @@ __device__ __forceinline__ void react_voxels(const Inst<real> &I, long long step
     }
 }
 
-template <typename real, bool NEXT>
-__device__ __forceinline__ long long diffuse_rows(const Inst<real> &I, const long long *counter, const real *vs_in,
-                                                  real *vs_out, int first, int end, int stride)
+template <typename real>
+__device__ __forceinline__ long long diffuse_react_rows(const Inst<real> &I, const long long *counter, const real *vs_in,
+                                                        real *vs_out, int first, int end, int stride)
 {
     real c[kRowLen];
     if (first < end) row_load(I, first, c);
@@ -623,22 +623,20 @@ __device__ __forceinline__ long long diffuse_rows(const Inst<real> &I, const lon
     const double tn = (double)step * I.dt_d;
     const real *v = I.v[parity];
     real *vn = I.v[parity ^ 1];
-    const unsigned stim = NEXT ? active_stimuli(I, (double)(step + 1) * I.dt_d) : 0u;
+    const unsigned stim = active_stimuli(I, (double)(step + 1) * I.dt_d);
     for (int i = first; i < end; i += stride) {
         if (i != first) row_load(I, i, c);
         const int q = row_index(c[27]);
-        const real u = vs_in[q], vold = v[q], w = NEXT ? I.w[parity ^ 1][q] : real(0);
+        const real u = vs_in[q], vold = v[q], w = I.w[parity ^ 1][q];
         const real vnew = u - I.coef_par * row_apply(I, c, vs_in + q, u);
         vn[q] = vnew;
         if (vold < real(0.5) && vnew >= real(0.5) && I.tact[q] < real(0))
             I.tact[q] = (real)(tn + I.dt_d * (0.5 - (double)vold) / ((double)vnew - (double)vold));
         if (!isfinite(vnew)) atomicOr(&I.ctl->nonfinite, 1);
-        if (NEXT) {
-            real vs, ws;
-            ms_step(I, stim, vnew, w, q % I.nx, (q / I.nx) % I.ny, q / (I.nx * I.ny), vs, ws);
-            vs_out[q] = vs;
-            I.w[parity][q] = ws;
-        }
+        real vs, ws;
+        ms_step(I, stim, vnew, w, q % I.nx, (q / I.nx) % I.ny, q / (I.nx * I.ny), vs, ws);
+        vs_out[q] = vs;
+        I.w[parity][q] = ws;
     }
     return step;
 }
@@ -654,24 +652,31 @@ __global__ void __launch_bounds__(kSweepThreads) k_react(Inst<real> I, int parit
 template <typename real>
 __global__ void __launch_bounds__(kSweepThreads, sizeof(real) == 8 ? 2 : EP_SWEEP_BLOCKS) k_mono_step(Inst<real> I, int parity)
 {
-    const long long step = diffuse_rows<real, true>(I, &I.ctl->tick[parity], vstar(I, parity), vstar(I, parity ^ 1),
-                                                    blockIdx.x * kSweepThreads + threadIdx.x, I.nrows,
-                                                    gridDim.x * kSweepThreads);
+    const long long step = diffuse_react_rows(I, &I.ctl->tick[parity], vstar(I, parity), vstar(I, parity ^ 1),
+                                              blockIdx.x * kSweepThreads + threadIdx.x, I.nrows,
+                                              gridDim.x * kSweepThreads);
     if (blockIdx.x == 0 && threadIdx.x == 0) I.ctl->tick[parity ^ 1] = step + 1;
 }
 
-// Batched: a share of a member's rows per entry of the packed reduction-chunk list (members with rows only), reaction
-// and diffusion as two launches; the step counter moves at the end of the batched step.
-template <typename real, bool DIFFUSE>
+// Batched: the same two launches over the members with rows; blockIdx.x an entry of the packed reduction-chunk list
+// (2 048 rows), blockIdx.y a share of it, as many shares as give the GPU three rounds of resident CTAs (mono_shares):
+// bound by latency, a small batch needs all its rows in flight, while in a large one each CTA's copy of the descriptor
+// counts.  The reaction alone leads the launches of a call (STEP false); the step counter moves at the end of the
+// batched step.  us a step in the march over recomputed tensors, in reaction and diffusion as two launches of whole
+// chunks, and here: 64 slabs of 24^3 54, 65, 46; four of 24^3 33, 32, 12; four of 88^3 96, 100, 88; sixteen of 88^3
+// 338, 320, 295; 32 shells of 128^3 432, 274, 240.
+template <typename real, bool STEP>
 __global__ void __launch_bounds__(kSweepThreads, EP_SWEEP_BLOCKS) k_mono_batch(const Inst<real> *insts, const BItem *items)
 {
     __shared__ Inst<real> sI;
     const BItem it = items[blockIdx.x];
     const Inst<real> &I = stage_inst(insts + it.inst, sI);
     if (!I.tab) return;
-    const int r0 = (int)((long long)I.nrows * it.item / it.nitems), r1 = (int)((long long)I.nrows * (it.item + 1) / it.nitems);
-    if (DIFFUSE) diffuse_rows<real, false>(I, &I.ctl->step, I.b, nullptr, r0 + threadIdx.x, r1, kSweepThreads);
-    else react_voxels(I, I.ctl->step, I.b, r0 + threadIdx.x, r1, kSweepThreads);
+    const long long part = (long long)it.item * gridDim.y + blockIdx.y, parts = (long long)it.nitems * gridDim.y;
+    const int r0 = (int)(I.nrows * part / parts), r1 = (int)(I.nrows * (part + 1) / parts);
+    const int parity = (int)(I.ctl->step & 1);
+    if (STEP) diffuse_react_rows(I, &I.ctl->step, vstar(I, parity), vstar(I, parity ^ 1), r0 + threadIdx.x, r1, kSweepThreads);
+    else react_voxels(I, I.ctl->step, vstar(I, parity), r0 + threadIdx.x, r1, kSweepThreads);
 }
 
 // cheb_weight(k) for k < kChebTable - 1; the last entry is the weights' limit 2 e^-theta / rho.
