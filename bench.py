@@ -159,13 +159,24 @@ def _kernel_hash():
     return h.hexdigest()[:16]
 
 
-def _sweep_kernel(mode, n_tissue):
-    """Name of the FP32 elliptic sweep kernel without a torso: over assembled
-    rows up to 720 thousand tissue voxels (the colour sweeps always), over
-    vertex lists in bricks above, the z-march where no tables are kept."""
-    if n_tissue < 4096:
+def _table_limits():
+    """Tissue voxels from which a handle has operator tables, and up to which
+    they are assembled rows, as the library's source has them."""
+    import re
+    src = {p: open(os.path.join(ROOT, "paper_2302_12519_gb300/csrc", p)).read() for p in ("ep_api.cu", "ep_common.cuh")}
+    return (int(re.search(r"kTabMin = (\d+);", src["ep_api.cu"]).group(1)),
+            int(re.search(r"#define EP_ROWS_ONLY (\d+)", src["ep_common.cuh"]).group(1)))
+
+
+def _sweep_kernel(mode, n_tissue, bare):
+    """Name of the FP32 sweep kernel without a torso: over assembled rows, over
+    vertex lists in bricks above the rows' limit (the colour sweeps: rows
+    always), the z-march where no tables are kept: on small handles, on large
+    monodomain ones and on bare ones, whose tables did not fit."""
+    tab_min, rows_only = _table_limits()
+    if bare or n_tissue < tab_min or (mode == "M_IE" and n_tissue > rows_only):
         return f"k_stencil<float,{mode}>"
-    rows = mode == "M_JAC_GS" or n_tissue <= 720000
+    rows = mode == "M_JAC_GS" or n_tissue <= rows_only
     return f"k_sweep<float,{mode},{'FORM_ROWS' if rows else 'FORM_BRICKS'}>"
 
 
@@ -472,8 +483,10 @@ def solver_legs(ep, case, a, blob0, stream, flush, end_state, peak):
         h.set_params(c.params)
         for st in c.stimuli:
             h.add_stimulus(st.lo, st.hi, st.t_start, st.dur, st.amp)
+        planned = h.footprint()[0]
         h.write_state(blob0)
         info = h.info()
+        bare = info.device_bytes < planned
         h.profile_enable(True)
         ms, iters, statuses = [], [], []
         for _ in range(a.steps):
@@ -494,8 +507,8 @@ def solver_legs(ep, case, a, blob0, stream, flush, end_state, peak):
         total_s = sum(ms) / 1e3
         d = {"value": M * a.steps / total_s, "unit": "tissue voxel-steps/s", "ms_per_step": 1e3 * total_s / a.steps,
              "sweeps_per_step": iters, "step_status": statuses,
-             "kernel": (_sweep_kernel("M_JAC_CHEB", M) + " (correction form)" if solver == 1 else
-                        _sweep_kernel("M_JAC_GS", M) + " (one colour pass; 8 a sweep)"),
+             "kernel": (_sweep_kernel("M_JAC_CHEB", M, bare) + " (correction form)" if solver == 1 else
+                        _sweep_kernel("M_JAC_GS", M, bare) + " (one colour pass; 8 a sweep)"),
              "avg_launch_us": launch_s * 1e6, "algorithmic_bytes_per_voxel": per,
              "traffic_bytes_per_voxel": _traffic_record(("chebyshev_sweep_" if solver == 1 else "gauss_seidel_pass_")
                                                         + a.workload),
@@ -619,6 +632,7 @@ def run_ours(a):
     ecg = case.electrodes is not None and case.model == 1
     if ecg:   # room for the warm-up, the timed window and its end-to-end replay
         sim.set_ecg(case.electrodes, a.warmup + 2 * a.steps + 1)
+    planned = sim.footprint()[0]
     if a.solver == "chebyshev":   # the oracle baseline runs the same semi-iteration on the same interval
         info = sim.info()
         case.params.cheb_lmin, case.params.cheb_lmax = info.cheb_lmin, info.cheb_lmax
@@ -632,6 +646,7 @@ def run_ours(a):
         sim.step(1, allow_noconv=True)
     torch.cuda.synchronize()
     n_dom = sim.info().n_domain   # voxels of the elliptic sweeps (tissue + torso)
+    bare = sim.info().device_bytes < planned   # the operator tables did not fit
     # snapshot of the state that starts the timed window (the e2e leg replays the same steps)
     nb = sim.state_bytes()
     blobs = [torch.empty(nb, dtype=torch.uint8, pin_memory=True).numpy() for _ in range(2)]
@@ -681,17 +696,17 @@ def run_ours(a):
         # the implicit sweeps dominate the step
         launch_s = prof.ie_sweep_ms / 1e3 / max(prof.ie_sweeps, 1)
         alg_bytes = BYTES_PER_IE_SWEEP_VOXEL * M
-        kname = (_sweep_kernel("M_IE", M) if M <= 720000 else "k_stencil<float,M_IE>") + " (implicit-Euler Jacobi sweep)"
+        kname = _sweep_kernel("M_IE", M, bare) + " (implicit-Euler Jacobi sweep)"
         share = prof.ie_sweep_ms / 1e3 / total_s
     elif mono:
         # the fused reaction + diffusion launch is the step (plus a one-thread step-counter kernel)
         launch_s = prof.other_ms / 1e3 / max(prof.steps, 1)
         # v, w read and written at the state precision, fibre 6, mask 1
         alg_bytes = (BYTES_PER_MONO_VOXEL if case.precision == 0 else 4 * 8 + 16) * M
-        kname = ("%s<%s%s> (fused reaction + diffusion)" %
-                 (("k_mono_step", "float" if case.precision == 0 else "double", "")
-                  if M >= 4096 and (case.precision != 0 or M <= 720000) else
-                  ("k_stencil", "float" if case.precision == 0 else "double", ",M_PAR_MONO")))
+        tab_min, rows_only = _table_limits()
+        real = "float" if case.precision == 0 else "double"
+        rows = not bare and M >= tab_min and (case.precision != 0 or M <= rows_only)
+        kname = (f"k_mono_step<{real}>" if rows else f"k_stencil<{real},M_PAR_MONO>") + " (fused reaction + diffusion)"
         share = prof.other_ms / 1e3 / total_s
     else:
         sweep_s = prof.sweep_ms / 1e3
@@ -699,12 +714,15 @@ def run_ours(a):
         per_voxel = (BYTES_PER_CHEB_SWEEP_VOXEL if a.solver == "chebyshev" else
                      BYTES_PER_GS_PASS_VOXEL if a.solver == "gs" else BYTES_PER_SWEEP_VOXEL)
         alg_bytes = per_voxel * n_dom   # over tissue + torso when a torso is set
-        kname = ("k_sweep<float,M_JAC(_CHEB),FORM_TORSO> (one elliptic sweep over tissue + torso)"
-                 if torso else _sweep_kernel("M_JAC", M) + " (damped Jacobi sweep)")
+        kname = ("k_stencil<float,M_JAC(_CHEB)> over the torso items away from the tissue + "
+                 "k_stencil<float,M_JAC_BATH(_CHEB)> over the rest (one elliptic sweep over tissue + torso)"
+                 if torso and (bare or M < _table_limits()[0]) else
+                 "k_sweep<float,M_JAC(_CHEB),FORM_TORSO> (one elliptic sweep over tissue + torso)"
+                 if torso else _sweep_kernel("M_JAC", M, bare) + " (damped Jacobi sweep)")
         if a.solver == "chebyshev":
             kname += ", Chebyshev-accelerated"
         if a.solver == "gs":
-            kname = _sweep_kernel("M_JAC_GS", M) + " (one colour pass of the eight-colour Gauss-Seidel sweep)"
+            kname = _sweep_kernel("M_JAC_GS", M, bare) + " (one colour pass of the eight-colour Gauss-Seidel sweep)"
         share = sweep_s / total_s
     achieved = alg_bytes / launch_s / 1e9 if launch_s > 0 else 0.0
     stem = (f"ie_sweep_slab{a.slab_n}_mono" if mono and implicit else

@@ -384,8 +384,8 @@ void build_bricks(const uint8_t *m, int nx, int ny, int nz, HostPlan &P)
 }
 
 // Torso handles: the torso voxels whose neighbours in the grid, all 26, are torso too, and the work items over them
-// (the longest that still give each SM three; the rows fill the rest.  144^3 box: 525 items of 32 planes 36 us a
-// sweep, 945 of 16 38, 1890 of 8 42).
+// (the longest that still give each of 152 SMs three, a number and not the device's, since a plan needs no device; the
+// rows fill the rest.  144^3 box: 525 items of 32 planes 36 us a sweep, 945 of 16 38, 1890 of 8 42).
 void plan_walk(const uint8_t *torso, const uint8_t *heart, int nx, int ny, int nz, HostPlan &P)
 {
     const size_t n = (size_t)nx * ny * nz, plane = (size_t)nx * ny;
@@ -472,7 +472,10 @@ TabPlan tab_plan(const ep_sim *s)
 {
     TabPlan t;
     if (s->lean || !s->have_params || s->n_tissue < kTabMin) return t;
-    if (!s->torso.empty()) {   // FP32: rows near the tissue, the walk through the torso away from it
+    // FP32: rows near the tissue, the walk through the torso away from it.  Above kRowsOnly too, where the march is its
+    // only alternative (two-term items): Chebyshev 200^3 box, 1.62 million tissue voxels, 92 us a sweep against 184;
+    // 256^3, 3.41 million, 178 against 317.
+    if (!s->torso.empty()) {
         if (s->d.precision != EP_FP32 || s->d.model != EP_BI || s->p.solver == EP_SOLVER_GAUSS_SEIDEL) return t;
         t.tab = 1;
         t.nrows = s->n_domain - s->plan.n_walked;
@@ -1197,7 +1200,8 @@ struct OneSweep {
 // A kernel over the tabulated operator in the order of the stream.  In FP32 the launch may start while the one before
 // it still runs (the kernel waits for that one itself, after_previous_launch, before it touches what changes): 6.7 to
 // 5.7 us a sweep of the 128^3 shell, 3.2 to 2.6 of the 48^3 one.  Not in FP64, whose long kernels share the few FP64
-// lanes with the early one: 15 against 10 us a step of the 32^3 slab (reaction and diffusion as two launches).
+// lanes with the early one: 9.9 against 8.3 us a step of the 32^3 slab, 8.4 against 5.9 a sweep of the 48^3 shell,
+// where the 128^3 one would gain 4 % (33.8 to 32.6).
 template <typename real, typename... A>
 void launch_after(void (*kernel)(Inst<real>, A...), int grid, int block, size_t smem, cudaStream_t q, const Inst<real> &I, A... args)
 {
