@@ -431,6 +431,15 @@ void mark_clear(std::vector<Seg> &segs, const uint8_t *m, int nx, int ny, int nz
     }
 }
 
+// Whether a handle's clear items take the walk of their own.  Its sums are in another order than the march's, and which
+// voxels lie in clear items depends on the planes an item has.  So a handle that a batch can hold, where these change,
+// has the walk where every item is clear whatever its planes: results do not depend on the schedule.
+bool clear_items(const ep_sim *s)
+{
+    const bool batched = s->d.precision == EP_FP32 && s->torso.empty() && s->p.diffusion == EP_EXPLICIT;
+    return !batched || s->n_tissue == s->n;
+}
+
 // ---------------------------------------------------------------------------
 // set-up: layout built on the host from the mask, records on the device
 // ---------------------------------------------------------------------------
@@ -785,7 +794,7 @@ ep_status setup_typed(ep_sim *s)
         s->nseg_e = tor ? (int)s->plan.segs_e.size() : s->nseg;
         s->nseg_far = tor ? partition_far(s->plan.segs_e, s->mask.data(), s->d.nx, s->d.ny, s->d.nz) : 0;
         s->zseg = kZLens[pick];
-        mark_clear(s->plan.segs, m, nx, ny, nz);
+        if (clear_items(s)) mark_clear(s->plan.segs, m, nx, ny, nz);
         if (tor) {
             std::vector<uint8_t> dom(s->mask);
             for (long long q = 0; q < n; ++q) dom[q] |= s->torso[q];
@@ -2334,7 +2343,7 @@ ep_status relayout_segments(ep_sim *s, int zseg)
     if (zseg == s->zseg) return EP_OK;
     std::vector<Seg> segs = build_segments(s->mask.data(), s->d.nx, s->d.ny, s->d.nz, zseg);
     if ((long long)segs.size() > s->max_items) return fail(s, EP_EINVAL, "segment capacity exceeded");
-    mark_clear(segs, s->mask.data(), s->d.nx, s->d.ny, s->d.nz);
+    if (clear_items(s)) mark_clear(segs, s->mask.data(), s->d.nx, s->d.ny, s->d.nz);
     CK(cudaMemcpyAsync(s->segs, segs.data(), sizeof(Seg) * segs.size(), cudaMemcpyHostToDevice, s->stream));
     CK(cudaStreamSynchronize(s->stream));
     s->nseg = (int)segs.size();

@@ -43,3 +43,31 @@ def test_monodomain_members_same_alone_and_in_the_mix(sizes):
     b.close()
     for s in alone + mixed:
         s.close()
+
+
+# Blocks above the 720 thousand voxels up to which they have tables, one full and one with a cavity: the planes of a work
+# item change with the schedule (8 to 32 of 40), and with them which voxels lie in items without a hole
+@pytest.mark.parametrize("cavity", [False, True])
+def test_results_do_not_depend_on_the_planes_of_a_work_item(cavity):
+    mask = np.ones((40, 150, 150), np.uint8)
+    if cavity:
+        mask[18:22, 60:63, 70:90] = 0
+    c = W.random_case(81, 150, 150, 40, model=W.MONO, mask=mask)
+    v, w, _ = W.random_state(81, c)
+    out = []
+    for zseg in (None, 8, 16, 32):
+        s = ep.sim_from_case(c)
+        s.set_state(v, w, None, 0)
+        if zseg is None:
+            s.step(3)
+        else:
+            b = ep.Batch(1)
+            b.set_schedule(0, zseg, -1)
+            b.add(s)
+            b.step(3)
+            b.close()
+        out.append([s.read(f) for f in (ep.EP_V, ep.EP_W, ep.EP_TACT)])
+        s.close()
+    for other in out[1:]:
+        for a, b in zip(out[0], other):
+            np.testing.assert_array_equal(a, b)
