@@ -103,6 +103,7 @@ struct ep_sim {
     int nseg_e = 0;              // work items of the elliptic sweeps (nseg without a torso)
     int nseg_far = 0;            // the first of them, whose cells and halo hold no tissue
     int zseg = kZSeg;            // z-planes per stencil work item
+    int nclear = 0;              // clear items of the elliptic sweeps
     long long max_items = 0;     // segment capacity of the segs / partials buffers
     double omega = 0.0;
     double cheb_lmin = 0.0, cheb_lmax = 0.0;   // Chebyshev interval in use
@@ -416,9 +417,10 @@ void plan_walk(const uint8_t *torso, const uint8_t *heart, int nx, int ny, int n
     P.walked = std::move(b);
 }
 
-// Marks the clear items of a list over mask m.
-void mark_clear(std::vector<Seg> &segs, const uint8_t *m, int nx, int ny, int nz)
+// Marks the clear items of a list over mask m and returns their number.
+int mark_clear(std::vector<Seg> &segs, const uint8_t *m, int nx, int ny, int nz)
 {
+    int found = 0;
     for (Seg &g : segs) {
         const int xa = std::max(0, g.x0 - 1), xb = std::min(nx, g.x0 + kTileX + 1);
         const int ya = std::max(0, g.by * kTileY - 1), yb = std::min(ny, g.by * kTileY + kTileY + 1);
@@ -428,7 +430,9 @@ void mark_clear(std::vector<Seg> &segs, const uint8_t *m, int nx, int ny, int nz
             for (int j = ya; j < yb && clear; ++j)
                 clear = !std::memchr(m + (size_t)nx * (j + (size_t)ny * k) + xa, 0, (size_t)(xb - xa));
         if (clear) g.by |= kClearItem;
+        found += clear;
     }
+    return found;
 }
 
 // Whether a handle's clear items take the walk of their own.  Its sums are in another order than the march's, and which
@@ -794,11 +798,11 @@ ep_status setup_typed(ep_sim *s)
         s->nseg_e = tor ? (int)s->plan.segs_e.size() : s->nseg;
         s->nseg_far = tor ? partition_far(s->plan.segs_e, s->mask.data(), s->d.nx, s->d.ny, s->d.nz) : 0;
         s->zseg = kZLens[pick];
-        if (clear_items(s)) mark_clear(s->plan.segs, m, nx, ny, nz);
+        s->nclear = clear_items(s) ? mark_clear(s->plan.segs, m, nx, ny, nz) : 0;
         if (tor) {
             std::vector<uint8_t> dom(s->mask);
             for (long long q = 0; q < n; ++q) dom[q] |= s->torso[q];
-            mark_clear(s->plan.segs_e, dom.data(), nx, ny, nz);
+            s->nclear = mark_clear(s->plan.segs_e, dom.data(), nx, ny, nz);   // of the elliptic sweeps
         }
     }
     const HostPlan &P = s->plan;
@@ -1252,6 +1256,16 @@ struct TabSweep {
         launch(k_sweep<real, MODE, FORM_ROWS>, I.nsweep, kSweepNT<FORM_ROWS>, 0, q, I, phase);
     }
 };
+// Calls f with the mode of the march's Jacobi or Chebyshev sweeps, for launches with clear items or without.
+template <typename F>
+auto jacobi_mode(bool cheb, bool clear, F &&f)
+{
+    if (cheb && clear) return f(std::integral_constant<int, M_JAC_CHEB_CLEAR>{});
+    if (cheb) return f(std::integral_constant<int, M_JAC_CHEB>{});
+    if (clear) return f(std::integral_constant<int, M_JAC_CLEAR>{});
+    return f(std::integral_constant<int, M_JAC>{});
+}
+
 template <typename real, int MODE_FAR, int MODE_NEAR>
 struct SplitSweep {
     Inst<real> far, near;   // far.nseg or near.nseg may be 0
@@ -1375,11 +1389,11 @@ cudaError_t allow_stencil_active(std::integer_sequence<int, MODES...>)
 ep_status configure_kernels(ep_sim *s)
 {
     using Modes = std::integer_sequence<int, M_APPLY, M_RHS, M_PAR_MONO, M_PAR_BI, M_JAC, M_IE_RHS, M_IE, M_JAC_BATH,
-                                        M_APPLY_BATH, M_JAC_CHEB, M_JAC_BATH_CHEB, M_JAC_GS>;
+                                        M_APPLY_BATH, M_JAC_CHEB, M_JAC_BATH_CHEB, M_JAC_GS, M_JAC_CLEAR, M_JAC_CHEB_CLEAR>;
     cudaError_t e = allow_stencil<float>(Modes{});
     if (e == cudaSuccess) e = allow_stencil<double>(Modes{});
     if (e == cudaSuccess)
-        e = allow_stencil_batch(std::integer_sequence<int, M_PAR_MONO, M_PAR_BI, M_RHS, M_JAC, M_JAC_CHEB>{});
+        e = allow_stencil_batch(std::integer_sequence<int, M_PAR_MONO, M_PAR_BI, M_RHS, M_JAC, M_JAC_CHEB, M_JAC_CLEAR, M_JAC_CHEB_CLEAR>{});
     auto bricks = [&](auto *k) {
         if (e == cudaSuccess) e = allow_smem(k, kSweepSmem<FORM_BRICKS>);
     };
@@ -1389,7 +1403,7 @@ ep_status configure_kernels(ep_sim *s)
     bricks(k_sweep_batch<float, M_JAC_CHEB, FORM_BRICKS>);
     bricks(k_sweep_active<float, M_JAC, FORM_BRICKS>);
     bricks(k_sweep_active<float, M_JAC_CHEB, FORM_BRICKS>);
-    if (e == cudaSuccess) e = allow_stencil_active(std::integer_sequence<int, M_JAC, M_JAC_CHEB>{});
+    if (e == cudaSuccess) e = allow_stencil_active(std::integer_sequence<int, M_JAC, M_JAC_CHEB, M_JAC_CLEAR, M_JAC_CHEB_CLEAR>{});
     if (e != cudaSuccess) {
         cudaGetLastError();
         return fail(s, EP_ECUDA, std::string("cudaFuncSetAttribute(shared memory): ") + cudaGetErrorString(e));
@@ -1479,8 +1493,9 @@ ep_status solve_elliptic(ep_sim *s, const Inst<real> &I, int &iters, double &rel
     } else if (I.solver == 2) {   // eight colour passes a sweep
         rs = run_sweeps(s, OneSweep<real, M_JAC_GS>{I}, &s->sweep_graph, &queued, 8);
     } else if (s->torso.empty()) {
-        rs = cheb ? run_sweeps(s, OneSweep<real, M_JAC_CHEB>{I}, &s->sweep_graph, &queued)
-                  : run_sweeps(s, OneSweep<real, M_JAC>{I}, &s->sweep_graph, &queued);
+        rs = jacobi_mode(cheb, s->nclear > 0, [&](auto m) {
+            return run_sweeps(s, OneSweep<real, decltype(m)::value>{I}, &s->sweep_graph, &queued);
+        });
     } else {   // tissue + torso: the domain's items and records, split by distance from the tissue
         const Inst<real> Ie = make_elliptic_inst<real>(s);
         Inst<real> far = Ie, near = Ie;
@@ -1491,8 +1506,10 @@ ep_status solve_elliptic(ep_sim *s, const Inst<real> &I, int &iters, double &rel
         near.segs = s->segs_e + s->nseg_far;
         near.nseg = s->nseg_e - s->nseg_far;
         near.item0 = s->nseg_far;
-        rs = cheb ? run_sweeps(s, SplitSweep<real, M_JAC_CHEB, M_JAC_BATH_CHEB>{far, near}, &s->sweep_graph, &queued)
-                  : run_sweeps(s, SplitSweep<real, M_JAC, M_JAC_BATH>{far, near}, &s->sweep_graph, &queued);
+        rs = jacobi_mode(cheb, s->nclear > 0, [&](auto m) {
+            constexpr int F = decltype(m)::value, N = kCheb<F> ? M_JAC_BATH_CHEB : M_JAC_BATH;
+            return run_sweeps(s, SplitSweep<real, F, N>{far, near}, &s->sweep_graph, &queued);
+        });
     }
     if (rs != EP_OK) return rs;
     if (s->prof_on) {
@@ -2311,6 +2328,7 @@ struct ep_batch {
         std::vector<int> solo;    // rows swept in their own launches
         long long packed_items;   // items of the other rows without a tabulated operator (packed sweep launches)
         bool cheb;                // its members' solver: Chebyshev-accelerated (else damped Jacobi)
+        bool clear;               // a member without a tabulated operator has clear items
         long long packed_tab[2];  // sweep CTAs of those with a tabulated operator, rows and bricks (packed launches each)
         long long sw0, nsw;       // range of its tabulated members' sweep CTAs in d_sweep
     };
@@ -2343,7 +2361,7 @@ ep_status relayout_segments(ep_sim *s, int zseg)
     if (zseg == s->zseg) return EP_OK;
     std::vector<Seg> segs = build_segments(s->mask.data(), s->d.nx, s->d.ny, s->d.nz, zseg);
     if ((long long)segs.size() > s->max_items) return fail(s, EP_EINVAL, "segment capacity exceeded");
-    if (clear_items(s)) mark_clear(segs, s->mask.data(), s->d.nx, s->d.ny, s->d.nz);
+    s->nclear = clear_items(s) ? mark_clear(segs, s->mask.data(), s->d.nx, s->d.ny, s->d.nz) : 0;
     CK(cudaMemcpyAsync(s->segs, segs.data(), sizeof(Seg) * segs.size(), cudaMemcpyHostToDevice, s->stream));
     CK(cudaStreamSynchronize(s->stream));
     s->nseg = (int)segs.size();
@@ -2426,6 +2444,7 @@ ep_status rebuild_tables(ep_batch *b)
         g.nsw = (long long)sweeps.size() - g.sw0;
         g.packed_tab[0] = g.packed_tab[1] = 0;
         g.packed_items = 0;
+        g.clear = false;
         // few members, each in its own launches: a whole solver's few, or the tabulated ones of a group that is small
         // because of their tables
         int same = 0;
@@ -2433,6 +2452,7 @@ ep_status rebuild_tables(ep_batch *b)
         const bool small = r1 - r <= kSoloAllMembers, few = (b->group_bytes ? r1 - r : same) <= kSoloAllMembers;
         for (int q = r; q < r1; ++q) {
             ep_sim *s = b->slot[b->order[q]];
+            g.clear = g.clear || (!s->tab && s->nclear > 0);
             if (few || (small && s->tab) || s->nseg >= b->solo_items) g.solo.push_back(q);
             else if (s->tab) g.packed_tab[s->nbricks > 0] += s->nsweep;
             else g.packed_items += s->nseg;
@@ -2602,12 +2622,12 @@ ep_status build_batch_graph(ep_batch *b)
             for (int j = 0; j < nsolo; ++j) {
                 cudaStream_t a = b->aux[j];
                 CKB(cudaStreamWaitEvent(a, b->ev_fork, 0));
-                const Inst<float> I = make_inst<float>(b->slot[b->order[gr.solo[j]]]);
+                const ep_sim *member = b->slot[b->order[gr.solo[j]]];
+                const Inst<float> I = make_inst<float>(member);
                 for (int i = 0; i < spc; ++i) {
                     if (I.tab && gr.cheb) TabSweep<float, M_JAC_CHEB, false>{I}(a, i & 1);
                     else if (I.tab) TabSweep<float, M_JAC, false>{I}(a, i & 1);
-                    else if (gr.cheb) k_stencil<float, M_JAC_CHEB><<<I.nseg, kThreads, kSmemBytes<float, M_JAC_CHEB>, a>>>(I, no_io<float>());
-                    else k_stencil<float, M_JAC><<<I.nseg, kThreads, kSmemBytes<float, M_JAC>, a>>>(I, no_io<float>());
+                    else jacobi_mode(gr.cheb, member->nclear > 0, [&](auto m) { OneSweep<float, decltype(m)::value>{I}(a, i); });
                 }
                 CKB(cudaEventRecord(b->ev_join[j], a));
             }
@@ -2631,8 +2651,10 @@ ep_status build_batch_graph(ep_batch *b)
             if (gr.packed_items > 0)
                 for (int i = 0; i < spc; ++i) {
                     const int gp = grid_of(gr.packed_items, 1 << 30);
-                    if (gr.cheb) k_stencil_active<float, M_JAC_CHEB><<<gp, kThreads, kSmemBytes<float, M_JAC_CHEB>, b->side>>>(gi_inst, b->d_act, gn);
-                    else k_stencil_active<float, M_JAC><<<gp, kThreads, kSmemBytes<float, M_JAC>, b->side>>>(gi_inst, b->d_act, gn);
+                    jacobi_mode(gr.cheb, gr.clear, [&](auto m) {
+                        constexpr int MODE = decltype(m)::value;
+                        k_stencil_active<float, MODE><<<gp, kThreads, kSmemBytes<float, MODE>, b->side>>>(gi_inst, b->d_act, gn);
+                    });
                 }
             for (int j = 0; j < nbranch; ++j) CKB(cudaStreamWaitEvent(b->side, b->ev_join[j], 0));
             active_lists(b->side);
@@ -2894,8 +2916,10 @@ ep_status ep_batch_autotune(ep_batch *b, int trial_sweeps)
                         tables(std::true_type{});
                         tables(std::false_type{});
                     }
-                    if (gl && gr.cheb) k_stencil_batch<float, M_JAC_CHEB><<<gs, kThreads, kSmemBytes<float, M_JAC_CHEB>, s0>>>(b->d_inst, b->d_seg + gr.seg0);
-                    else if (gl) k_stencil_batch<float, M_JAC><<<gs, kThreads, kSmemBytes<float, M_JAC>, s0>>>(b->d_inst, b->d_seg + gr.seg0);
+                    if (gl) jacobi_mode(gr.cheb, gr.clear, [&](auto m) {
+                        constexpr int MODE = decltype(m)::value;
+                        k_stencil_batch<float, MODE><<<gs, kThreads, kSmemBytes<float, MODE>, s0>>>(b->d_inst, b->d_seg + gr.seg0);
+                    });
                 };
                 sweep();
                 CKB(cudaEventRecord(e0, s0));

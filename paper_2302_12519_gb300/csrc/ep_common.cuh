@@ -56,17 +56,19 @@ constexpr int kChunk = 2048;                // tissue voxels per reduction chunk
 // semi-iteration (separate instances, so the plain sweeps carry none of it).
 // M_JAC_GS: one colour pass of the eight-colour Gauss-Seidel / SOR sweep, in
 // place on x0 (a sweep is eight launches, colours 0..7).
+// M_JAC_CLEAR, M_JAC_CHEB_CLEAR: M_JAC and M_JAC_CHEB with the walk over clear
+// items, for launches that have any (an instance with both forms spills more).
 enum Mode { M_APPLY = 0, M_RHS = 1, M_PAR_MONO = 2, M_PAR_BI = 3, M_JAC = 4, M_IE_RHS = 5, M_IE = 6, M_JAC_BATH = 7,
-            M_APPLY_BATH = 8, M_JAC_CHEB = 9, M_JAC_BATH_CHEB = 10, M_JAC_GS = 11 };
+            M_APPLY_BATH = 8, M_JAC_CHEB = 9, M_JAC_BATH_CHEB = 10, M_JAC_GS = 11, M_JAC_CLEAR = 12, M_JAC_CHEB_CLEAR = 13 };
 enum Diffusion { DIFF_EXPLICIT = 0, DIFF_IMPLICIT = 1 };
 
 // Modes that run a solve sweep (Jacobi of the elliptic or the implicit parabolic system).
 template <int MODE>
-constexpr bool kCheb = MODE == M_JAC_CHEB || MODE == M_JAC_BATH_CHEB;
+constexpr bool kCheb = MODE == M_JAC_CHEB || MODE == M_JAC_BATH_CHEB || MODE == M_JAC_CHEB_CLEAR;
 template <int MODE>
 constexpr bool kGS = MODE == M_JAC_GS;
 template <int MODE>
-constexpr bool kJac = MODE == M_JAC || MODE == M_JAC_BATH || kCheb<MODE> || kGS<MODE>;
+constexpr bool kJac = MODE == M_JAC || MODE == M_JAC_BATH || MODE == M_JAC_CLEAR || kCheb<MODE> || kGS<MODE>;
 template <int MODE>
 constexpr bool kTwoTerm = MODE == M_JAC_BATH || MODE == M_APPLY_BATH || MODE == M_JAC_BATH_CHEB;
 template <int MODE>

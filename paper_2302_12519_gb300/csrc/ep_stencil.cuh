@@ -418,11 +418,11 @@ template <typename real, int MODE>
 constexpr bool kRinged = (kJac<MODE> || MODE == M_IE || MODE == M_PAR_MONO) &&
                          !(kTwoTerm<MODE> && sizeof(real) == 8);
 
-// Modes whose clear items take the walk of their own.  Not the FP32 Chebyshev sweeps: they reach it on handles without
-// tables only, and the instance that holds both spills more (32^3 shell, 3 080 voxels: 11.7 us a sweep, 11.2 without;
-// a box of 17 x 16 x 15, all of it clear, 9.5 with the walk, 10.8 without).
-template <typename real, int MODE>
-constexpr bool kClearWalk = MODE == M_JAC || (MODE == M_JAC_CHEB && sizeof(real) == 8) || MODE == M_IE || MODE == M_PAR_MONO;
+// Modes whose clear items take the walk of their own.  The Jacobi and Chebyshev sweeps have instances without it: with
+// both forms in one, a 32^3 shell of 3 080 voxels took 11.7 us a Chebyshev sweep, 11.2 without (FP64: 100.8 and 99.5).
+// A box of 17 x 16 x 15, all of it clear, takes 9.5 with the walk and 10.8 without (FP64: 66 and 99).
+template <int MODE>
+constexpr bool kClearWalk = MODE == M_JAC_CLEAR || MODE == M_JAC_CHEB_CLEAR || MODE == M_IE || MODE == M_PAR_MONO;
 
 template <typename real, int MODE>
 struct Ring {
@@ -948,8 +948,8 @@ __device__ __forceinline__ void stencil_item(const Inst<real> &I, int seg_index,
         // unrolled by 4 so that every ring slot is a compile-time constant
         constexpr int D = Ring<real, MODE>::D;
         Ring<real, MODE> &R = sm.ring;
-        const bool walked = kClearWalk<real, MODE> && clear;
-        if constexpr (kClearWalk<real, MODE>)
+        const bool walked = kClearWalk<MODE> && clear;
+        if constexpr (kClearWalk<MODE>)
             if (clear) clear_walk<real, MODE>(I, o, g, lo_in, kbeg, kend, reinterpret_cast<ClearRing<real, MODE> &>(R), sF, check, acc);
 #pragma unroll
         for (int j = 0; j < D - 1; ++j) {

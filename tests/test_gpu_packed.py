@@ -42,7 +42,7 @@ def _handles(cases):
 def test_packed_members_same_alone_and_in_the_mix(bricks, solver, capped):
     cases = [_case(40, 16, 16, 16, "full"), _case(41, 31, 17, 8, "full"), _case(42, 96, 96, 1, "full")]
     cases += [_case(43 + i, 18 + i, 20 + i, 15 - i % 3, "holes") for i in range(7)]
-    cases += [_case(51, 13, 11, 9, "full"), _case(52, 4095, 1, 1, "full")]
+    cases += [_case(51, 13, 11, 9, "full"), _case(52, 15, 14, 13, "holes")]   # clear items only, none
     if bricks:
         cases.append(_case(53, 91, 91, 89, "full"))
     for c in cases:
