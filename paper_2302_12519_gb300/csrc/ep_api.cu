@@ -42,10 +42,12 @@ constexpr int kZSeg = EP_ZSEG;     // default output planes per z-march segment
 constexpr int kZSegMin = 8;        // smallest segment length the batch autotuner tries
 constexpr int kSweepChunk[2] = {16, 64};   // launches of the queued graphs (multiples of 8: launches know their phase)
 constexpr int kSoloAllMembers = 8; // batch groups this small sweep every member in its own launches
-// Tables of a batch group's members together: what stays in the L2 cache from one sweep to the next.  Ten shells of 48^3
-// to 160^3 (160 MB of rows), two steps: one group 93 ms, groups of about 100 MB 74, 50 MB 70, 25 MB 80; forty of up to
-// 128^3: one group 153, 50 MB 106.
-constexpr size_t kGroupTables = EP_GROUP_TABLES;
+// Tables of a batch group's members together: what stays in the L2 cache from one sweep to the next, where bricks, which
+// stream, count half; two members may share a group up to a quarter more, since a member alone leaves the GPU idle at
+// the ends of its sweeps.  us a sweep of all members, with 56 MB and as here: 16 blocks of 64^3 (29 MB of rows each) 140
+// and 109, four hearts of 176^3 (50 MB of bricks) 107 and 81, six shells of 150^3 (36 MB of rows) 50 and 45; four of
+// 128^3 (22 MB) 22.5 in pairs, 25.7 in a group of three and one, 28 together.
+constexpr size_t kGroupTables = (size_t)60 << 20;
 constexpr double kDivFactor = 1e16;
 constexpr int kNoAllocMaxPartials = 32768;   // ep_step_noalloc: stencil work items and reduction chunks
 
@@ -2385,6 +2387,9 @@ ep_status grow(ep_batch *b, T **p, size_t *cap, size_t need)
     return EP_OK;
 }
 
+// What a member's tables count towards a group's (kGroupTables).
+size_t group_share(const ep_sim *s) { return s->nbricks ? s->tab_total / 2 : s->tab_total; }
+
 ep_status rebuild_tables(ep_batch *b)
 {
     b->order.clear();
@@ -2414,11 +2419,11 @@ ep_status rebuild_tables(ep_batch *b)
         auto next = [&] { return b->slot[b->order[r1]]; };
         do {
             bytes += 20 * (size_t)next()->n;
-            tables += next()->tab_total;
+            tables += group_share(next());
             ++r1;
         } while (r1 < b->ninst && is_cheb(b->order[r1]) == cheb &&
                  (b->group_bytes == 0 || bytes + 20 * (size_t)next()->n <= b->group_bytes) &&
-                 tables + next()->tab_total <= kGroupTables);
+                 tables + group_share(next()) <= (r1 - r == 1 ? kGroupTables + kGroupTables / 4 : kGroupTables));
         ep_batch::Group g;
         g.cheb = cheb;
         g.sw0 = (long long)sweeps.size();

@@ -31,9 +31,6 @@ constexpr int kTileY = kWarps - 1;          // output rows per CTA (warps 1..kWa
 #ifndef EP_BRICK_BLOCKS
 #define EP_BRICK_BLOCKS 4
 #endif
-#ifndef EP_GROUP_TABLES
-#define EP_GROUP_TABLES ((size_t)56 << 20)
-#endif
 #ifndef EP_ROWS_ONLY
 #define EP_ROWS_ONLY 720000
 #endif

@@ -21,6 +21,9 @@ def _built():
 def _case(seed, nx, ny, nz, kind):
     rng = np.random.default_rng(seed)
     mask = np.ones((nz, ny, nx), np.uint8) if kind == "full" else (rng.random((nz, ny, nx)) > 0.03).astype(np.uint8)
+    if kind == "layers":
+        z, y, x = np.meshgrid(np.arange(nz), np.arange(ny), np.arange(nx), indexing="ij")
+        mask = ((x + 0.7 * y + 0.4 * z) / 6.0 % 1.0 < 0.57).astype(np.uint8)
     return W.random_case(seed, nx, ny, nz, model=W.BI, mask=mask)
 
 
@@ -90,4 +93,27 @@ def test_autotune_with_tables_keeps_the_solve():
     assert all(b.slot_stats(i).iters == 5 and b.slot_stats(i).step == 5 for i in range(3))
     b.close()
     for s in hs:
+        s.close()
+
+
+# Two blocks of 64^3 (29 MB of rows each) share a group of at most 60 MB; so do two members with 57 MB of bricks, which
+# count half, and two with 37 MB of rows (up to 75 MB a pair); a third joins none of them
+@pytest.mark.parametrize("n,size,kind,groups", [(4, (64, 64, 64), "full", 2), (2, (90, 98, 160), "layers", 1),
+                                                (3, (90, 98, 160), "layers", 2), (3, (75, 90, 85), "layers", 2)])
+def test_members_that_share_a_group(n, size, kind, groups):
+    cases = [_case(80 + i, *size, kind) for i in range(n)]
+    for c in cases:
+        c.params.solver, c.params.max_iter, c.params.rel_tol, c.params.check_every = 1, 6, 0.0, 4
+    alone, mixed = _handles(cases), _handles(cases)
+    b = ep.Batch(n)
+    for s in mixed:
+        b.add(s)
+    assert b.info().groups == groups
+    b.step(2, allow_noconv=True)
+    for a, m in zip(alone, mixed):
+        a.step(2, allow_noconv=True)
+        for f in FIELDS:
+            np.testing.assert_array_equal(m.read(f), a.read(f))
+    b.close()
+    for s in alone + mixed:
         s.close()
