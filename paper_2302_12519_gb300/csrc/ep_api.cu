@@ -2317,6 +2317,7 @@ struct ep_batch {
     long long nseg_items = 0, nchunk_items = 0;
     std::vector<int> order;        // slot of each table row
     std::vector<long long> layouts;   // its handle's layout when the tables were built
+    std::vector<int> packed;       // how its sweeps are launched
     cudaGraphExec_t graph = nullptr;
     bool dirty = true;
     int nsm = 152, sweeps_per_check = 16, zseg = kZSeg;
@@ -2465,7 +2466,8 @@ ep_status rebuild_tables(ep_batch *b)
         b->groups.push_back(g);
         r = r1;
     }
-    std::vector<int> packed(b->ninst, 1);   // 0 solo, 1 packed, 2 and 3 packed over rows and bricks
+    std::vector<int> &packed = b->packed;   // 0 solo, 1 packed, 2 and 3 packed over rows and bricks
+    packed.assign(b->ninst, 1);
     for (int r = 0; r < b->ninst; ++r)
         if (b->slot[b->order[r]]->tab) packed[r] = b->slot[b->order[r]]->nbricks > 0 ? 3 : 2;
     for (const ep_batch::Group &g : b->groups)
@@ -2584,12 +2586,14 @@ ep_status build_batch_graph(ep_batch *b)
             const int gn = gr.inst1 - gr.inst0;
             const Inst<float> *gi_inst = b->d_inst + gr.inst0;
             const int *gi_packed = b->d_packed + gr.inst0;
+            // rows: up to three of a member's sweep CTAs in one of a packed launch that has more than the GPU holds
+            const int share[2] = {(int)std::max<long long>(1, std::min<long long>(3, gr.packed_tab[0] / (EP_SWEEP_BLOCKS * b->nsm))), 1};
             ActRec *act_tab[2] = {b->d_act + (b->ninst + 1), b->d_act + 2 * (b->ninst + 1)};
             auto active_lists = [&](cudaStream_t q) {   // of the packed members; the loop's condition
-                k_active_list<float><<<1, kActThreads, 0, q>>>(gi_inst, gi_packed, gn, 1, b->d_act, b->d_counts, hg[gi]);
+                k_active_list<float><<<1, kActThreads, 0, q>>>(gi_inst, gi_packed, gn, 1, 1, b->d_act, b->d_counts, hg[gi]);
                 for (int f = 0; f < 2; ++f)
                     if (gr.packed_tab[f] > 0)
-                        k_active_list<float><<<1, kActThreads, 0, q>>>(gi_inst, gi_packed, gn, 2 + f, act_tab[f], b->d_counts, hg[gi]);
+                        k_active_list<float><<<1, kActThreads, 0, q>>>(gi_inst, gi_packed, gn, 2 + f, share[f], act_tab[f], b->d_counts, hg[gi]);
             };
             active_lists(st);
             // inner loop: sweeps of the unfinished members until every solve of the group is finished
@@ -2637,11 +2641,15 @@ ep_status build_batch_graph(ep_batch *b)
                 CKB(cudaEventRecord(b->ev_join[j], a));
             }
             // the other members: packed sweeps over the unfinished ones
+            int packed_ctas[2] = {0, 0};
+            for (int q = gr.inst0; q < gr.inst1; ++q)
+                if (b->packed[q] >= 2)
+                    packed_ctas[b->packed[q] - 2] += (b->slot[b->order[q]]->nsweep + share[b->packed[q] - 2] - 1) / share[b->packed[q] - 2];
             auto packed_sweep = [&](auto bricks, cudaStream_t a, int i) {
                 constexpr int B = decltype(bricks)::value ? FORM_BRICKS : FORM_ROWS;
-                const int gp = (int)gr.packed_tab[B];
-                if (gr.cheb) k_sweep_active<float, M_JAC_CHEB, B><<<gp, kSweepNT<B>, kSweepSmem<B>, a>>>(gi_inst, act_tab[B], gn, i & 1);
-                else k_sweep_active<float, M_JAC, B><<<gp, kSweepNT<B>, kSweepSmem<B>, a>>>(gi_inst, act_tab[B], gn, i & 1);
+                const int gp = packed_ctas[B];
+                if (gr.cheb) k_sweep_active<float, M_JAC_CHEB, B><<<gp, kSweepNT<B>, kSweepSmem<B>, a>>>(gi_inst, act_tab[B], gn, share[B], i & 1);
+                else k_sweep_active<float, M_JAC, B><<<gp, kSweepNT<B>, kSweepSmem<B>, a>>>(gi_inst, act_tab[B], gn, share[B], i & 1);
             };
             for (int f = 0; f < 2; ++f) {
                 if (gr.packed_tab[f] == 0) continue;

@@ -608,7 +608,7 @@ constexpr int kActThreads = 1024;
 
 template <typename real>
 __global__ void __launch_bounds__(kActThreads)
-k_active_list(const Inst<real> *insts, const int *packed, int n, int kind, ActRec *act, int *counts,
+k_active_list(const Inst<real> *insts, const int *packed, int n, int kind, int share, ActRec *act, int *counts,
               cudaGraphConditionalHandle h)
 {
     __shared__ int swa[32], swc[32];
@@ -625,7 +625,7 @@ k_active_list(const Inst<real> *insts, const int *packed, int n, int kind, ActRe
         running |= live ? 1 : 0;
         if (live && packed[i] == kind) {
             a = 1;
-            c = insts[i].tab ? insts[i].nsweep : insts[i].nseg;
+            c = insts[i].tab ? (insts[i].nsweep + share - 1) / share : insts[i].nseg;
         }
         int sa = a, sc = c;   // inclusive scans within the warp
         for (int o = 1; o < 32; o <<= 1) {

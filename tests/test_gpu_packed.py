@@ -117,3 +117,25 @@ def test_members_that_share_a_group(n, size, kind, groups):
     b.close()
     for s in alone + mixed:
         s.close()
+
+
+# Members of 32 and 34 sweep CTAs of rows go one, two and three to a CTA of the packed launch; 912 CTAs are resident on
+# 152 SMs
+@pytest.mark.parametrize("n", [40, 60, 100])
+def test_packed_ctas_that_take_several_sweep_ctas(n):
+    cases = [_case(100 + i % 7, 32, 8, 16 + i % 2, "full") for i in range(n)]
+    for i, c in enumerate(cases):
+        c.params.max_iter, c.params.rel_tol, c.params.check_every = 5 + 3 * (i % 3), 0.0, 4
+    alone, mixed = _handles(cases), _handles(cases)
+    b = ep.Batch(n)
+    for s in mixed:
+        b.add(s)
+    assert b.info().solo_members == 0 and b.info().groups == 1
+    b.step(2, allow_noconv=True)
+    for a, m in zip(alone, mixed):
+        a.step(2, allow_noconv=True)
+        for f in FIELDS:
+            np.testing.assert_array_equal(m.read(f), a.read(f))
+    b.close()
+    for s in alone + mixed:
+        s.close()
