@@ -73,6 +73,7 @@ struct HostPlan {
     std::vector<Seg> segs_e, segs_e_z[4];   // the same over the domain (torso handles only)
     std::vector<Brick> bricks;          // tabulated operator: bricks over the tissue, and their lists' totals
     long long n_vert = 0, n_part = 0, n_bound = 0;
+    long long planes[2] = {0, 0};       // planes that the march's items of 32 walk, of clear items in [1]
     std::vector<uint8_t> walked;        // torso handles: voxels with nothing but torso around them, their number
     std::vector<Seg> walk;              // and the work items over them
     long long n_walked = 0;
@@ -478,6 +479,42 @@ constexpr long long kRowsOnly = EP_ROWS_ONLY;
 constexpr int kMaxRowCtas = 4096;
 constexpr size_t kArriveBytes = sizeof(unsigned) * kArriveStride * (kArriveGroups + 1);
 
+// FP64 rows are read in 32 bytes, twice what the rest of a handle asks of a device allocator's alignment: 16 bytes to
+// round up with.
+size_t rows_bytes(size_t rb, long long nrows) { return abytes(rb * kRowLen * (size_t)nrows + (rb == 8 ? 16 : 0)); }
+
+// Rows that no second member like this one would share a batch's group with.
+bool lone_rows(const ep_sim *s) { return rows_bytes(sizeof(float), s->n_tissue) > kGroupTables / 2; }
+
+// Whether the march's items of 32 planes are filled well: 125 voxels a plane and more (210 at most; hearts and shells 80
+// to 120).
+bool dense_items(const ep_sim *s) { return 125 * (s->plan.planes[0] + s->plan.planes[1]) < s->n_tissue; }
+
+// The form of an FP32 Jacobi or Chebyshev sweep without a torso: what should cost least in us of the whole GPU.  Rows 22
+// ps a voxel; bricks 11 ps a vertex and 4 more a voxel at the surface, and 5 us; the march 2.6 ns a plane of an item (1.8
+// of a clear one; Chebyshev 2.9 and 2.0), and 4.5 us (12).  These are the costs beside other work: densely filled items
+// march well, and rows that have a batch's group to themselves (kGroupTables) leave the GPU idle at its ends, 30 ps a
+// voxel.  Alone a member is bound by latency as well, and where the forms change places rows would be faster by up to a
+// quarter there; but the choice holds alone and in a batch, which give the same results, and neither is slower than
+// without tables.
+// us a sweep before the tables, with tables whatever the mask, and by this rule, Jacobi / Chebyshev: 256^3 block 235 /
+// 266, 239 / 247, 167 / 195; 300^3 347 / 394, 377 / 388, 247 / 289; eight blocks of 80^3 in a batch 66 / 78, 110 / 114,
+// 49 / 61; of 110^3 164 / 193, 212 / 212, 122 / 152; one of 80^3 15.7 / 19.1, 11.0 / 11.5, 12.3 / 12.9.
+enum SweepForm32 { USE_ROWS, USE_BRICKS, USE_MARCH };
+SweepForm32 choose_form(const ep_sim *s)
+{
+    const HostPlan &P = s->plan;
+    const bool cheb = s->p.solver == EP_SOLVER_CHEBYSHEV, walk = clear_items(s);
+    const double general = (double)(P.planes[0] + (walk ? 0 : P.planes[1])), clear = walk ? (double)P.planes[1] : 0.0;
+    const double march = cheb ? 12.0 + 2.9e-3 * general + 2.0e-3 * clear : 4.5 + 2.6e-3 * general + 1.8e-3 * clear;
+    const double none = 1e300, n = (double)s->n_tissue;
+    const double rows = s->n_tissue > kRowsOnly ? none : (lone_rows(s) && dense_items(s) ? 3.0e-5 : 2.2e-5) * n;
+    const double bricks = P.bricks.empty() || P.n_vert > 2147483647LL   // the lists are indexed in 32 bits
+                              ? none : 5.0 + 1.1e-5 * (double)P.n_vert + 4e-6 * (double)P.n_bound;
+    if (march < std::min(rows, bricks)) return USE_MARCH;
+    return rows <= bricks ? USE_ROWS : USE_BRICKS;
+}
+
 struct TabPlan {
     int tab = 0, nbricks = 0, nsweep = 0, parts = 1, nwalk = 0;
     long long nrows = 0;
@@ -503,21 +540,20 @@ TabPlan tab_plan(const ep_sim *s)
     const bool gs = !mono && s->p.solver == EP_SOLVER_GAUSS_SEIDEL;
     t.tab = 1;
     t.parts = gs ? 8 : 1;
-    if (!gs && s->d.precision == EP_FP32 && s->n_tissue > kRowsOnly) {
-        if (s->plan.n_vert > 2147483647LL) return TabPlan();   // the lists are indexed in 32 bits
-        t.nbricks = (int)s->plan.bricks.size();
-        t.nsweep = t.nbricks;
-        return t;
+    if (!mono && !gs && s->d.precision == EP_FP32) {
+        const SweepForm32 c = choose_form(s);
+        if (c == USE_MARCH) return TabPlan();
+        if (c == USE_BRICKS) {
+            t.nbricks = (int)s->plan.bricks.size();
+            t.nsweep = t.nbricks;
+            return t;
+        }
     }
     t.nrows = s->n_tissue;
     const long long per = gs ? (t.nrows + 7) / 8 + (t.nrows + 15) / 16 : t.nrows;   // a colour's rows, or thereabouts
     t.nsweep = (int)std::min<long long>(kMaxRowCtas, (per + kSweepThreads - 1) / kSweepThreads);
     return t;
 }
-
-// FP64 rows are read in 32 bytes, twice what the rest of a handle asks of a device allocator's alignment: 16 bytes to
-// round up with.
-size_t rows_bytes(size_t rb, long long nrows) { return abytes(rb * kRowLen * (size_t)nrows + (rb == 8 ? 16 : 0)); }
 
 size_t tab_bytes(const ep_sim *s, const TabPlan &t, size_t rb)
 {
@@ -662,8 +698,13 @@ ep_status plan_layout(ep_sim *s)
     s->nchunk = (int)P.chunks.size();
     s->nseg = (int)P.segs.size();
     s->nseg_e = torso ? (int)P.segs_e.size() : s->nseg;
-    if (s->d.model == EP_BI && !torso && s->d.precision == EP_FP32 && s->n_tissue > kRowsOnly)
-        build_bricks(mh, nx, ny, nz, P);
+    if (s->d.model == EP_BI && !torso && s->d.precision == EP_FP32 && s->n_tissue >= kTabMin) {   // what choose_form weighs
+        std::vector<Seg> items = P.segs_z[3];
+        mark_clear(items, mh, nx, ny, nz);
+        P.planes[0] = P.planes[1] = 0;
+        for (const Seg &g : items) P.planes[(g.by & kClearItem) != 0] += g.k1 - g.k0 + 2;
+        if (s->n_tissue > kRowsOnly || (dense_items(s) && lone_rows(s))) build_bricks(mh, nx, ny, nz, P);
+    }
     if (torso && s->d.precision == EP_FP32 && s->n_tissue >= kTabMin) plan_walk(s->torso.data(), mh, nx, ny, nz, P);
     // capacity of the item buffers: the largest item count of the z-lengths set-up and the batch use
     s->max_items = std::max<long long>(most, std::max(s->nseg, s->nseg_e));

@@ -42,6 +42,7 @@ def test_row_tables(lib, model, precision, solver, per):
 @pytest.mark.parametrize("kind", ["box", "heart"])
 def test_brick_tables(lib, kind):
     c = W.random_case(3, 91, 91, 89, mask=np.ones((89, 91, 91), np.uint8)) if kind == "box" else W.config2(n=160)
+    c.params.solver = 1 if kind == "box" else 0   # the Jacobi sweeps of a box that large take the march
     assert 43.0 < _tables(c) / c.n_tissue < 50.0
 
 
@@ -49,6 +50,25 @@ def test_no_tables(lib):
     for c in (W.random_case(3, 16, 16, 15, mask=np.ones((15, 16, 16), np.uint8)),
               W.random_case(3, 91, 91, 89, model=W.MONO, mask=np.ones((89, 91, 91), np.uint8))):
         assert _tables(c) == 0
+
+
+@pytest.mark.parametrize("n,fill,jacobi,chebyshev", [(64, 1.0, 112, 112), (74, 1.0, 0, 45), (88, 1.0, 0, 45), (150, 1.0, 0, 0),
+                                                     (80, 0.97, 0, 45)])
+def test_form_of_a_dense_block(lib, n, fill, jacobi, chebyshev):
+    """Bytes a tissue voxel: rows, none (the march), bricks."""
+    mask = (np.random.default_rng(1).random((n, n, n)) < fill).astype(np.uint8)
+    for solver, per in ((0, jacobi), (1, chebyshev)):
+        c = W.random_case(3, n, n, n, mask=mask)
+        c.params.solver = solver
+        assert abs(_tables(c) / c.n_tissue - per) <= (6 if per else 0)
+
+
+@pytest.mark.parametrize("case,per", [(W.config1(), 112), (W.config2(n=144), 112), (W.config2(), 45), (W.sampled_shell(np.random.default_rng(0), 204, 1, "s"), 45)],
+                         ids=["shell128", "heart144", "heart256", "shell204"])
+def test_form_of_shells_and_hearts(lib, case, per):
+    for solver in (0, 1):
+        case.params.solver = solver
+        assert abs(_tables(case) / case.n_tissue - per) <= 5
 
 
 def test_torso_tables(lib):

@@ -210,7 +210,7 @@ class CappedAllocator:
 # the last row: a colour pass over rows, bricks (737 thousand voxels), rows and the torso's walk
 @pytest.mark.parametrize("kind,model,precision,solver", [("box", W.BI, W.FP32, 1), ("box", W.BI, W.FP64, 0),
                                                          ("box", W.MONO, W.FP32, 0), ("box", W.MONO, W.FP64, 0),
-                                                         ("box", W.BI, W.FP32, 2), ("big", W.BI, W.FP32, 0),
+                                                         ("box", W.BI, W.FP32, 2), ("big", W.BI, W.FP32, 1),
                                                          ("torso", W.BI, W.FP32, 1)])
 def test_tables_that_do_not_fit_are_left_out(kind, model, precision, solver):
     """Memory for a handle's fields and staging but not its tables: it steps without them, to the rounding of the
