@@ -159,25 +159,25 @@ def _kernel_hash():
     return h.hexdigest()[:16]
 
 
-def _table_limits():
-    """Tissue voxels from which a handle has operator tables, and up to which
-    they are assembled rows, as the library's source has them."""
-    import re
-    src = {p: open(os.path.join(ROOT, "paper_2302_12519_gb300/csrc", p)).read() for p in ("ep_api.cu", "ep_common.cuh")}
-    return (int(re.search(r"kTabMin = (\d+);", src["ep_api.cu"]).group(1)),
-            int(re.search(r"#define EP_ROWS_ONLY (\d+)", src["ep_common.cuh"]).group(1)))
+def _set_params(sim, case):
+    """Sets the case's parameters on a handle whose mask is set and returns the
+    form of its sweeps: operator tables as assembled rows or as vertex lists in
+    bricks, or none (the z-march), told by the device bytes that they add to
+    the plan of the mask, beside the iterates that the solve adds."""
+    before = sim.footprint()[0]
+    sim.set_params(case.params)
+    real = 4 if case.precision == 0 else 8
+    fields = 2 * int(case.params.diffusion == 1) + int(case.model == 1 and real == 4 and case.params.solver != 2)
+    per = (sim.footprint()[0] - before - real * fields * case.n) / case.n_tissue * 4 / real
+    return "rows" if per > 100 else "bricks" if per > 20 else "march"
 
 
-def _sweep_kernel(mode, n_tissue, bare):
-    """Name of the FP32 sweep kernel without a torso: over assembled rows, over
-    vertex lists in bricks above the rows' limit (the colour sweeps: rows
-    always), the z-march where no tables are kept: on small handles, on large
-    monodomain ones and on bare ones, whose tables did not fit."""
-    tab_min, rows_only = _table_limits()
-    if bare or n_tissue < tab_min or (mode == "M_IE" and n_tissue > rows_only):
-        return f"k_stencil<float,{mode}>"
-    rows = mode == "M_JAC_GS" or n_tissue <= rows_only
-    return f"k_sweep<float,{mode},{'FORM_ROWS' if rows else 'FORM_BRICKS'}>"
+def _sweep_kernel(mode, form, full):
+    """Name of the FP32 sweep kernel without a torso, by the handle's form; a
+    full mask has nothing but clear items."""
+    if form == "march":
+        return f"k_stencil<float,{mode}{'_CLEAR' if full and mode in ('M_JAC', 'M_JAC_CHEB') else ''}>"
+    return f"k_sweep<float,{mode},FORM_{form.upper()}>"
 
 
 def _traffic_record(stem):
@@ -480,13 +480,13 @@ def solver_legs(ep, case, a, blob0, stream, flush, end_state, peak):
         h = ep.Sim(c.nx, c.ny, c.nz, c.dx, c.model, c.precision, use_torch=True, stream=stream.cuda_stream)
         h.set_mask(c.mask_flat())
         h.set_fibres(c.fib_flat())
-        h.set_params(c.params)
+        form = _set_params(h, c)
         for st in c.stimuli:
             h.add_stimulus(st.lo, st.hi, st.t_start, st.dur, st.amp)
         planned = h.footprint()[0]
         h.write_state(blob0)
         info = h.info()
-        bare = info.device_bytes < planned
+        form = form if info.device_bytes == planned else "march"   # the operator tables did not fit
         h.profile_enable(True)
         ms, iters, statuses = [], [], []
         for _ in range(a.steps):
@@ -507,8 +507,8 @@ def solver_legs(ep, case, a, blob0, stream, flush, end_state, peak):
         total_s = sum(ms) / 1e3
         d = {"value": M * a.steps / total_s, "unit": "tissue voxel-steps/s", "ms_per_step": 1e3 * total_s / a.steps,
              "sweeps_per_step": iters, "step_status": statuses,
-             "kernel": (_sweep_kernel("M_JAC_CHEB", M, bare) + " (correction form)" if solver == 1 else
-                        _sweep_kernel("M_JAC_GS", M, bare) + " (one colour pass; 8 a sweep)"),
+             "kernel": (_sweep_kernel("M_JAC_CHEB", form, M == c.n) + " (correction form)" if solver == 1 else
+                        _sweep_kernel("M_JAC_GS", form, False) + " (one colour pass; 8 a sweep)"),
              "avg_launch_us": launch_s * 1e6, "algorithmic_bytes_per_voxel": per,
              "traffic_bytes_per_voxel": _traffic_record(("chebyshev_sweep_" if solver == 1 else "gauss_seidel_pass_")
                                                         + a.workload),
@@ -623,7 +623,7 @@ def run_ours(a):
                  stream=stream.cuda_stream)
     sim.set_mask(case.mask_flat())
     sim.set_fibres(case.fib_flat())
-    sim.set_params(case.params)
+    form = _set_params(sim, case)
     for s in case.stimuli:
         sim.add_stimulus(s.lo, s.hi, s.t_start, s.dur, s.amp)
     torso = case.torso is not None
@@ -646,7 +646,8 @@ def run_ours(a):
         sim.step(1, allow_noconv=True)
     torch.cuda.synchronize()
     n_dom = sim.info().n_domain   # voxels of the elliptic sweeps (tissue + torso)
-    bare = sim.info().device_bytes < planned   # the operator tables did not fit
+    if sim.info().device_bytes < planned:   # the operator tables did not fit
+        form = "march"
     # snapshot of the state that starts the timed window (the e2e leg replays the same steps)
     nb = sim.state_bytes()
     blobs = [torch.empty(nb, dtype=torch.uint8, pin_memory=True).numpy() for _ in range(2)]
@@ -696,17 +697,15 @@ def run_ours(a):
         # the implicit sweeps dominate the step
         launch_s = prof.ie_sweep_ms / 1e3 / max(prof.ie_sweeps, 1)
         alg_bytes = BYTES_PER_IE_SWEEP_VOXEL * M
-        kname = _sweep_kernel("M_IE", M, bare) + " (implicit-Euler Jacobi sweep)"
+        kname = _sweep_kernel("M_IE", form, False) + " (implicit-Euler Jacobi sweep)"
         share = prof.ie_sweep_ms / 1e3 / total_s
     elif mono:
         # the fused reaction + diffusion launch is the step (plus a one-thread step-counter kernel)
         launch_s = prof.other_ms / 1e3 / max(prof.steps, 1)
         # v, w read and written at the state precision, fibre 6, mask 1
         alg_bytes = (BYTES_PER_MONO_VOXEL if case.precision == 0 else 4 * 8 + 16) * M
-        tab_min, rows_only = _table_limits()
         real = "float" if case.precision == 0 else "double"
-        rows = not bare and M >= tab_min and (case.precision != 0 or M <= rows_only)
-        kname = (f"k_mono_step<{real}>" if rows else f"k_stencil<{real},M_PAR_MONO>") + " (fused reaction + diffusion)"
+        kname = (f"k_mono_step<{real}>" if form == "rows" else f"k_stencil<{real},M_PAR_MONO>") + " (fused reaction + diffusion)"
         share = prof.other_ms / 1e3 / total_s
     else:
         sweep_s = prof.sweep_ms / 1e3
@@ -714,15 +713,15 @@ def run_ours(a):
         per_voxel = (BYTES_PER_CHEB_SWEEP_VOXEL if a.solver == "chebyshev" else
                      BYTES_PER_GS_PASS_VOXEL if a.solver == "gs" else BYTES_PER_SWEEP_VOXEL)
         alg_bytes = per_voxel * n_dom   # over tissue + torso when a torso is set
-        kname = ("k_stencil<float,M_JAC(_CHEB)> over the torso items away from the tissue + "
+        kname = ("k_stencil<float,M_JAC(_CHEB)(_CLEAR)> over the torso items away from the tissue + "
                  "k_stencil<float,M_JAC_BATH(_CHEB)> over the rest (one elliptic sweep over tissue + torso)"
-                 if torso and (bare or M < _table_limits()[0]) else
+                 if torso and form == "march" else
                  "k_sweep<float,M_JAC(_CHEB),FORM_TORSO> (one elliptic sweep over tissue + torso)"
-                 if torso else _sweep_kernel("M_JAC", M, bare) + " (damped Jacobi sweep)")
+                 if torso else _sweep_kernel("M_JAC", form, M == case.n) + " (damped Jacobi sweep)")
         if a.solver == "chebyshev":
             kname += ", Chebyshev-accelerated"
         if a.solver == "gs":
-            kname = _sweep_kernel("M_JAC_GS", M, bare) + " (one colour pass of the eight-colour Gauss-Seidel sweep)"
+            kname = _sweep_kernel("M_JAC_GS", form, False) + " (one colour pass of the eight-colour Gauss-Seidel sweep)"
         share = sweep_s / total_s
     achieved = alg_bytes / launch_s / 1e9 if launch_s > 0 else 0.0
     stem = (f"ie_sweep_slab{a.slab_n}_mono" if mono and implicit else

@@ -313,11 +313,14 @@ typedef struct {
  * the most it holds during set-up (staging of fibres, mask and records).
  * After set-up both equal the bytes held.  From 4096 tissue voxels on they
  * include the operator tables, known once the parameters are set: 112 bytes
- * a tissue voxel in FP32 (224 in FP64), about 90 for FP32 bidomain handles
- * above 720 thousand tissue voxels, none for FP32 monodomain ones of that
- * size; with a torso, for the voxels at the tissue only.  A handle runs
- * without them where they do not fit: if their allocation fails, or a batch
- * or server would else refuse it for its budget.  EP_ESTATE without a mask,
+ * a tissue voxel in FP32 (224 in FP64); 43 to 70 for FP32 bidomain handles
+ * above 720 thousand tissue voxels (about 45 for hearts and shells; not with
+ * the Gauss-Seidel solve) and for smaller dense blocks that sweep faster that
+ * way; none for FP32 monodomain handles above 720 thousand and for dense
+ * blocks that sweep faster without; with a torso (FP32), 112 for the tissue
+ * and the torso voxels next to it or to a hole, and 4 for every grid voxel.
+ * A handle runs without them where they do not fit: if their allocation fails,
+ * or a batch or server would else refuse it for its budget.  EP_ESTATE without a mask,
  * EP_EINVAL if the mask has no tissue.  Host-only; needs no GPU.  No
  * counterpart in the paper: admission control of the served form. */
 ep_status ep_footprint(ep_sim *s, size_t *resident_bytes, size_t *peak_bytes);
@@ -337,7 +340,8 @@ ep_status ep_get_profile(ep_sim *s, ep_profile *prof);
  * convergence loop, is one CUDA graph with device-side loop conditions, so
  * the host is not involved between steps.  Results per instance are the same
  * as ep_step on that instance alone, up to the order of the FP64 reductions
- * (which does not change either). */
+ * (which does not change either); a member whose operator tables a budget
+ * took gives, alone too, what a handle without them gives. */
 typedef struct ep_batch ep_batch;
 
 typedef struct {
@@ -351,7 +355,8 @@ typedef struct {
     int zseg;                    /* z-planes per stencil work item (tuned) */
     size_t group_bytes;          /* members are swept in groups whose working sets total at most
                                     this many bytes, so a group's sweeps stay in L2 (0 = no limit; tuned); members with
-                                    operator tables also share at most 56 MB of them */
+                                    operator tables also share at most 60 MB of them (75 MB two members; the
+                                    tables of large handles, read once a sweep, count half) */
     int groups;                  /* number of such groups */
     int solo_members;            /* members whose Jacobi sweeps run as their own launches, concurrent
                                     with the packed launch of the others: those with at least half a
@@ -367,7 +372,8 @@ ep_status ep_batch_create(int max_instances, size_t hbm_budget_bytes, void *cuda
 /* Admit a handle (FP32, same model as the batch's other members; it is set up
  * here if needed).  The batch does not own it: the caller keeps it alive until
  * ep_batch_remove and reads results with ep_read on it.  EP_EREJECTED if its
- * device memory would exceed the budget, EP_EBUSY if the batch is full.
+ * device memory would exceed the budget (operator tables are given up first,
+ * its own and then the other members'), EP_EBUSY if the batch is full.
  * *slot receives the slot number. */
 ep_status ep_batch_add(ep_batch *b, ep_sim *sim, int *slot);
 ep_status ep_batch_remove(ep_batch *b, int slot);

@@ -601,7 +601,8 @@ __global__ void k_fill(real *p, long long n, real v)
 // solve is unfinished, in row order: act[k] = {items before member k, its
 // row, its control block}; entries n_active .. n hold {total items, -1,
 // null}, so the rest of the list never matches an item; counts = {total
-// items, n_active}.  Sets the condition of the device-side convergence loop:
+// items, n_active}.  (Members with operator tables: `share` of their sweep CTAs
+// make an item.)  Sets the condition of the device-side convergence loop:
 // any member of rows [0, n) still active, packed or not.  One CTA of
 // kActThreads.
 constexpr int kActThreads = 1024;
