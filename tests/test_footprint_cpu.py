@@ -63,8 +63,8 @@ def test_form_of_a_dense_block(lib, n, fill, jacobi, chebyshev):
         assert abs(_tables(c) / c.n_tissue - per) <= (6 if per else 0)
 
 
-@pytest.mark.parametrize("case,per", [(W.config1(), 112), (W.config2(n=144), 112), (W.config2(), 45), (W.sampled_shell(np.random.default_rng(0), 204, 1, "s"), 45)],
-                         ids=["shell128", "heart144", "heart256", "shell204"])
+@pytest.mark.parametrize("case,per", [(W.config1(), 112), (W.config2(n=144), 112), (W.config2(n=176), 45), (W.sampled_shell(np.random.default_rng(0), 204, 1, "s"), 45)],
+                         ids=["shell128", "heart144", "heart176", "shell204"])
 def test_form_of_shells_and_hearts(lib, case, per):
     for solver in (0, 1):
         case.params.solver = solver
