@@ -486,8 +486,8 @@ size_t rows_bytes(size_t rb, long long nrows) { return abytes(rb * kRowLen * (si
 // Rows that no second member like this one would share a batch's group with.
 bool lone_rows(const ep_sim *s) { return rows_bytes(sizeof(float), s->n_tissue) > kGroupTables / 2; }
 
-// Whether the march's items of 32 planes are filled well: 125 voxels a plane and more (210 at most; hearts and shells 80
-// to 120).
+// Whether the march's items of 32 planes are filled well: 125 voxels a plane and more (210 at most; hearts and shells
+// small enough for rows 80 to 120).
 bool dense_items(const ep_sim *s) { return 125 * (s->plan.planes[0] + s->plan.planes[1]) < s->n_tissue; }
 
 // The form of an FP32 Jacobi or Chebyshev sweep without a torso: what should cost least in us of the whole GPU.  Rows 22
@@ -496,7 +496,8 @@ bool dense_items(const ep_sim *s) { return 125 * (s->plan.planes[0] + s->plan.pl
 // march well, and rows that have a batch's group to themselves (kGroupTables) leave the GPU idle at its ends, 30 ps a
 // voxel.  Alone a member is bound by latency as well, and where the forms change places rows would be faster by up to a
 // quarter there; but the choice holds alone and in a batch, which give the same results, and neither is slower than
-// without tables.
+// without tables.  (Rows of hearts that have a group to themselves still are, with Jacobi in a batch of several: six of
+// 130^3 105 us a sweep, 101 in the march; alone 10 against 17, so they stay.)
 // us a sweep before the tables, with tables whatever the mask, and by this rule, Jacobi / Chebyshev: 256^3 block 235 /
 // 266, 239 / 247, 167 / 195; 300^3 347 / 394, 377 / 388, 247 / 289; eight blocks of 80^3 in a batch 66 / 78, 110 / 114,
 // 49 / 61; of 110^3 164 / 193, 212 / 212, 122 / 152; one of 80^3 15.7 / 19.1, 11.0 / 11.5, 12.3 / 12.9.
